@@ -259,9 +259,15 @@ size_t sssp_solve_workspace_size(const sssp_graph* g, uint32_t S, const sssp_opt
  *   pred    : device [S][V] out (may be NULL), canonical predecessor vertex
  *   ws      : device workspace >= sssp_solve_workspace_size(g, S, opt)
  * opt->policy chooses the frontier policy of a round (sssp_policy).
+ * A graph of at least five edges per vertex is swept first, in the default
+ * policy and without held messages, where that is the faster way: all sources
+ * relax it together, in Bellman-Ford order (sweep.cu; tile, split, delta,
+ * threads and hub_count do not apply to it, and its rounds are iterations
+ * without messages between units).  What a sweep leaves (a graph of high
+ * diameter), and every other call, goes to the persistent solve.
  * Launches an init kernel, one persistent cooperative relaxation kernel in
  * which each block owns (source, partition sub-block) units, and an unpack
- * kernel.  Needs every block co-resident; returns SSSP_EUNSUPPORTED if the
+ * kernel.  dist is also scratch until the end.  Needs every block co-resident; returns SSSP_EUNSUPPORTED if the
  * device cannot hold one block per unit... (it then reuses blocks over
  * several units, so it only fails if not even one block fits).
  */

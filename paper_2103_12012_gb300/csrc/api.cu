@@ -25,6 +25,7 @@ constexpr float DEF_DELTA_F32 = 0.0625f;
 
 struct Resolved {
     uint32_t threads, tile, split, bps;
+    bool delta_given;
     uint32_t delta_bits, policy, msg_buffer, hub_count, hub_delta_bits, hub_mid_bits;
     uint64_t timeout_ns;
     uint32_t flags;
@@ -70,6 +71,7 @@ bool resolve(const sssp_options* o, int wtype, Resolved* r) {
     r->tile = o->tile ? o->tile : DEF_TILE;
     r->split = o->split ? o->split : 1u;
     r->bps = o->blocks_per_sm;
+    r->delta_given = o->delta > 0.0;
     r->delta_bits = delta_bits_for(wtype, o->delta);
     r->timeout_ns = o->timeout_ns ? o->timeout_ns : DEF_TIMEOUT_NS;
     r->flags = o->flags;
@@ -89,29 +91,65 @@ bool resolve(const sssp_options* o, int wtype, Resolved* r) {
     return true;
 }
 
-// Workspace of sssp_solve: header | packed[S][V] | bitmap[S][words] | dirty[S*Q] | nfsplit[S*Q]
+// The sweep (sweep.cu) is for graphs with more edges per vertex than a road network or a grid has:
+// those are of high diameter, where its frontiers stay small (a 4-neighbour grid has 4.0 edges per
+// vertex, the random and power-law graphs here 5.6 and more).  The other bounds keep its item,
+// distance and segment numbers in 32 bits.
+bool sweep_graph(const sssp_graph* g, uint32_t S) {
+    const uint64_t groups = (S + 7u) / 8u;
+    return g->E >= 5ull * g->V && g->V >= 64 && g->V < (1u << 31) && g->E < 0xF0000000u && 8ull * groups * g->V < 0xF0000000ull &&
+           groups * g->E < 0xF0000000ull;
+}
+
+// Workspace of sssp_solve: header | counters of the sweep | packed[S][V] | bitmap[S][words] | hub
+// entries[2] of the sweep | dirty[S*Q] | nfsplit[S*Q].  The sweep keeps dist[items][G] at the start
+// of packed.  For S > 1 its marks are in the rest of packed and its lists in the caller's dist array
+// (written only at the end); for S = 1 its marks are the bitmap, one list is the rest of packed and
+// the other the caller's dist.
 struct SolveWs {
-    size_t off_packed, off_bitmap, off_dirty, off_nf, total;
+    size_t off_ctl, off_packed, off_bitmap, off_ex, ex_bytes, off_dirty, off_nf, total;
     uint32_t words, B, Bq, Q;
+    bool sweep;
 };
 
-SolveWs solve_layout(const sssp_graph* g, uint32_t S, uint32_t split) {
+SolveWs solve_layout(const sssp_graph* g, uint32_t S, uint32_t split, bool sweep = true) {
     SolveWs w{};
+    w.sweep = sweep && sweep_graph(g, S);
     w.words = (g->V + 31u) / 32u;
     w.B = (uint32_t)(((uint64_t)g->V + g->partitions - 1) / g->partitions);
     w.Bq = (w.B + split - 1u) / split;
     w.Q = g->partitions * split;
     size_t off = WS_HEADER_BYTES;
+    w.off_ctl = off;
+    if (w.sweep) off += align_up(sizeof(SweepCtl), 256);
     w.off_packed = off;
     off += align_up(8ull * S * g->V, 256);
     w.off_bitmap = off;
     off += align_up(4ull * S * w.words, 256);
+    w.off_ex = off;
+    w.ex_bytes = 8ull * ((uint64_t)S * g->E / SWEEP_HUB + 1);
+    if (w.sweep) off += align_up(2 * w.ex_bytes, 256);
     w.off_dirty = off;
     off += align_up(4ull * S * w.Q, 256);
     w.off_nf = off;
     off += align_up(4ull * S * w.Q, 256);
     w.total = off;
     return w;
+}
+
+// Whether the sweep is the faster one (ms, uint32 weights; V, edges per vertex, P, S, given width):
+//   5 sources or more share rows: R-MAT 4.2 M, 16, 148, 8, tuned: 4.1 against 7.5; 1 M, 16, 148, 16:
+//     2.1 / 6.8; ER 262144, 16, 148, 16, default: 1.7 / 5.4; but ER 256, 16, 32, 16: 0.23 / 0.17
+//   few blocks (units) for the persistent solve: ER 16384, 8, 4, 1, default: 0.24 / 1.6; R-MAT 1 M,
+//     16, 4, 1: 0.6 / 35
+//   small sub-blocks make its rounds cheap: ER 4096, 40, 148, 4 (28 vertices each): 0.29 / 0.24,
+//     R-MAT 1024, 16, 148, 4: 0.21 / 0.14
+//   1 to 4 sources, many units and a given (tuned) width, on graphs without hubs: ER 1 M, 16, 148, 4:
+//     2.3 / 1.8, ER 16384, 16, 148, 1: 0.29 / 0.26; with hubs (those that are worth a layout) R-MAT
+//     1 M, 16, 148, 1: 0.6 / 1.2
+bool sweep_wins(const sssp_graph* g, uint32_t S, const SolveWs& L, bool delta_given) {
+    if (S >= 5) return g->V >= 2048 || L.Bq >= 64;
+    return L.Bq >= 64 && (!delta_given || g->ids || (uint64_t)S * L.Q < 128);
 }
 
 int sm_count() {
@@ -200,12 +238,13 @@ size_t sssp_solve_workspace_size(const sssp_graph* g, uint32_t S, const sssp_opt
 static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint32_t S, void* dist, uint32_t* pred,
                               const sssp_options* opt, void* ws, size_t ws_bytes, sssp_stream_t stream,
                               const uint32_t* tails, uint32_t n_tails, bool warm, int prune_mode = -1,
-                              uint8_t* keep = nullptr, uint32_t* witness = nullptr) {
+                              uint8_t* keep = nullptr, uint32_t* witness = nullptr, bool least = false) {
     Resolved r;
     if (!graph_ok(g) || S == 0 || (!warm && !sources) || !dist || !ws || !resolve(opt, g->wtype, &r))
         return SSSP_EINVAL;
     if (!aligned16(ws) || r.threads > SOLVE_MAX_THREADS) return SSSP_EINVAL;
-    const SolveWs L = solve_layout(g, S, r.split);
+    SolveWs L = solve_layout(g, S, r.split);
+    if (least && ws_bytes < L.total) L = solve_layout(g, S, r.split, false);
     if ((uint64_t)S * L.Q > 0xFFFFFFFFull / 2 || L.Q > MAX_UNITS_PER_SOURCE * 16u) return SSSP_EINVAL;
     if (ws_bytes < L.total) return SSSP_ENOMEM;
     const size_t smem = relax_smem_bytes(r.tile, L.Q, r.msg_buffer != 0);
@@ -260,13 +299,69 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
     l.n_tails = n_tails;
     l.prune_on = prune ? 1u : 0u;
     if (prune) l.prune = trishla_job(g, prune_mode, keep, witness);
-    return launch_solve(l, (cudaStream_t)stream) == cudaSuccess ? SSSP_OK : SSSP_ECUDA;
+    SweepLaunch x{};
+    // Cold solves in the default policy (the others ask for a schedule of the persistent solve).
+    if (L.sweep && !warm && !prune && r.policy == SSSP_POLICY_RELATIVE && r.msg_buffer == 0 && !l.hold_pending &&
+        sweep_wins(g, S, L, r.delta_given)) {
+        x.row_ptr = l.row_ptr;
+        x.col = l.col;
+        x.w = l.w;
+        x.wtype = g->wtype;
+        x.V = g->V;
+        x.E = g->E;
+        x.ids = g->ids;
+        x.slots = g->slots;
+        x.S = S;
+        x.G = S == 1 ? 1u : S == 2 ? 2u : S <= 4 ? 4u : 8u;
+        x.groups = (S + x.G - 1u) / x.G;
+        x.items = x.groups * g->V;
+        x.sources = sources;
+        x.hdr = l.hdr;
+        x.ctl = reinterpret_cast<SweepCtl*>(base + L.off_ctl);
+        // rows of eight are aligned to 32 bytes (the rest of packed has room: V >= 64)
+        x.dist = reinterpret_cast<uint32_t*>(S > 1 ? (reinterpret_cast<uintptr_t>(l.packed) + 31) & ~(uintptr_t)31
+                                                   : reinterpret_cast<uintptr_t>(l.packed));
+        uint32_t* rest = x.dist + (size_t)x.items * x.G;
+        x.mark = S == 1 ? l.bitmap : rest;
+        x.list[0] = l.dist;
+        x.list[1] = S == 1 ? rest : l.dist + x.items;
+        x.ex[0] = reinterpret_cast<unsigned long long*>(base + L.off_ex);
+        x.ex[1] = reinterpret_cast<unsigned long long*>(base + L.off_ex + L.ex_bytes);
+        x.dirty = l.dirty;
+        x.nfsplit = l.nfsplit;
+        x.n_dirty = (size_t)S * L.Q;
+        x.out = l.dist;
+        x.pred = pred;
+        x.inf = g->wtype == SSSP_W_F32 ? F32_INF_BITS : INF32;
+        x.timeout_ns = r.timeout_ns;
+        if (sweep_max_blocks_per_sm(g->wtype, x.G, &per_sm) != cudaSuccess) return SSSP_ECUDA;
+        if (r.bps) per_sm = std::min<int>(per_sm, (int)r.bps);
+        x.grid = (uint32_t)std::min<uint64_t>((uint64_t)std::max(per_sm, 0) * sm_count(),
+                                              std::max<uint64_t>(1, (uint64_t)g->E * x.groups / 1024));
+    }
+    return launch_solve(l, x.grid ? &x : nullptr, (cudaStream_t)stream) == cudaSuccess ? SSSP_OK : SSSP_ECUDA;
 }
 
 sssp_status sssp_solve(const sssp_graph* g, const uint32_t* sources, uint32_t S, void* dist, uint32_t* pred,
                        const sssp_options* opt, void* ws, size_t ws_bytes, sssp_stream_t stream) {
     return solve_impl(g, sources, S, dist, pred, opt, ws, ws_bytes, stream, nullptr, 0, false);
 }
+
+}  // extern "C"
+
+size_t sssp::solve_least_bytes(const sssp_graph* g, uint32_t S, const sssp_options* opt) {
+    Resolved r;
+    if (!graph_ok(g) || S == 0 || !resolve(opt, g->wtype, &r)) return 0;
+    return solve_layout(g, S, r.split, false).total;
+}
+
+sssp_status sssp::solve_in(const sssp_graph* g, const uint32_t* sources, uint32_t S, void* dist, uint32_t* pred,
+                           const sssp_options* opt, void* ws, size_t ws_bytes, sssp_stream_t stream) {
+    return solve_impl(g, sources, S, dist, pred, opt, ws, ws_bytes, stream, nullptr, 0, false, -1, nullptr, nullptr,
+                      true);
+}
+
+extern "C" {
 
 sssp_status sssp_solve_prune(const sssp_graph* g, const uint32_t* sources, uint32_t S, void* dist, uint32_t* pred,
                              int32_t mode, uint8_t* keep, uint32_t* witness, const sssp_options* opt, void* ws,

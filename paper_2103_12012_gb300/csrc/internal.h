@@ -12,6 +12,52 @@ namespace sssp {
 
 struct WsHeader;
 
+// ------------------------------------------------------------------ sweep.cu
+constexpr uint32_t SWEEP_HUB = 512;  // rows of at least this many edges are cut into segments
+
+struct SweepIter {            // counters of one iteration
+    uint32_t nA, nM;          // items in list A (from the front) and list M (from the back)
+    unsigned long long ex;    // hubs << 32 | their segments
+    unsigned long long work;  // relaxations of the iteration before
+    uint32_t pad[26];
+};
+struct SweepCtl {  // zero before the launch
+    uint32_t bar, pad[31];
+    SweepIter it[3];
+};
+
+struct SweepLaunch {
+    const uint32_t* row_ptr;
+    const uint32_t* col;
+    const uint32_t* w;
+    int wtype;
+    uint32_t V, E;
+    const uint32_t* ids;
+    const uint32_t* slots;
+    uint32_t S, G, groups, items;  // items = groups * V; item = group * V + vertex
+    const uint32_t* sources;
+    WsHeader* hdr;
+    SweepCtl* ctl;
+    uint32_t* dist;            // [items][G]
+    uint32_t* mark;            // [items] bits: a distance fell since the item was taken (it is listed)
+    uint32_t* list[2];         // [items] each
+    unsigned long long* ex[2]; // [hubs] each: first segment << 32 | item
+    uint32_t* dirty;           // cleared with the state, for a hand-over
+    uint32_t* nfsplit;
+    size_t n_dirty;
+    uint32_t* out;             // [S][V] results
+    uint32_t* pred;            // [S][V] or NULL
+    uint32_t inf;
+    uint64_t timeout_ns;
+    uint32_t grid;
+};
+
+cudaError_t sweep_max_blocks_per_sm(int wtype, uint32_t G, int* out);
+cudaError_t launch_sweep(const SweepLaunch& L, int sms, cudaStream_t st);
+cudaError_t launch_sweep_out(const SweepLaunch& L, int sms, cudaStream_t st);
+cudaError_t launch_sweep_requeue(const SweepLaunch& L, uint32_t* bitmap, uint32_t words, uint32_t B, uint32_t Bq,
+                                 uint32_t split, uint32_t Q, int sms, cudaStream_t st);
+
 // ------------------------------------------------------------------ relax.cu
 struct SolveLaunch {
     // graph
@@ -65,7 +111,9 @@ constexpr uint32_t BATCH_MAX_THREADS = 1024;  // block size limit of the batched
 size_t relax_smem_bytes(uint32_t tile, uint32_t Q, bool msgs);
 cudaError_t relax_max_blocks_per_sm(int wtype, uint32_t threads, uint32_t tile, uint32_t Q, int* out,
                                     bool prune = false, bool msgs = false, bool hubs = false);
-cudaError_t launch_solve(const SolveLaunch& L, cudaStream_t st);
+// with `sweep`: the sweep first (sweep.cu), then the persistent solve on what it leaves (no vertex is
+// queued when it finished: every block sees a zero count at its first look and ends)
+cudaError_t launch_solve(const SolveLaunch& L, const SweepLaunch* sweep, cudaStream_t st);
 
 // One problem of a batch, in the order blocks take them (largest first).
 struct BatchProblem {
@@ -132,6 +180,12 @@ cudaError_t trishla_launch(const TrishlaJob& J, int wtype, const unsigned long l
 size_t backward_workspace_bytes(uint32_t V, uint32_t E, uint32_t S);
 cudaError_t backward_launch(const sssp_graph* g, uint32_t S, const uint32_t* pred, const float* grad_dist,
                             float* grad_w, void* ws, cudaStream_t st);
+
+// -------------------------------------------------------------------- api.cu
+// sssp_solve in a workspace that may lack the sweep's part (then only the persistent solve runs)
+size_t solve_least_bytes(const sssp_graph* g, uint32_t S, const sssp_options* opt);
+sssp_status solve_in(const sssp_graph* g, const uint32_t* sources, uint32_t S, void* dist, uint32_t* pred,
+                     const sssp_options* opt, void* ws, size_t ws_bytes, sssp_stream_t stream);
 
 // ------------------------------------------------------------------- common
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

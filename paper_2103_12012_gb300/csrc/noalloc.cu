@@ -95,15 +95,16 @@ extern "C" sssp_status sssp_solve_noalloc(const sssp_graph* g, const uint32_t* s
                                           uint32_t* pred, const sssp_options* opt, uint32_t* status_out,
                                           sssp_stream_t stream) {
     if (!g || S == 0 || !sources || !dist) return SSSP_EINVAL;
-    const size_t need = sssp_solve_workspace_size(g, S, opt);
+    const size_t need = sssp::solve_least_bytes(g, S, opt);
     if (need == 0) return SSSP_EINVAL;
     if (need > SSSP_NOALLOC_SCRATCH_BYTES) return SSSP_ENOMEM;
     void* scratch = nullptr;
     const sssp_status st = scratch_for_current_device(&scratch);
     if (st != SSSP_OK) return st;
-    // sssp_solve clears the header and initialises every packed word, inbox word and
+    // the solve clears the header and initialises every packed word, inbox word and
     // doorbell it will read before its relaxation kernel starts.
-    const sssp_status ls = sssp_solve(g, sources, S, dist, pred, opt, scratch, SSSP_NOALLOC_SCRATCH_BYTES, stream);
+    const sssp_status ls =
+        sssp::solve_in(g, sources, S, dist, pred, opt, scratch, SSSP_NOALLOC_SCRATCH_BYTES, stream);
     if (ls != SSSP_OK || !status_out) return ls;
     // the status word is the first field of the scratch header
     if (cudaMemcpyAsync(status_out, scratch, sizeof(uint32_t), cudaMemcpyDeviceToDevice, (cudaStream_t)stream) !=

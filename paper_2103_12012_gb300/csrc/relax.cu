@@ -1053,13 +1053,14 @@ __global__ void k_seed(SolveLaunch L) {
 template <class W>
 __global__ void k_warm_pack(size_t n, uint32_t V, const uint32_t* __restrict__ slots,
                             const uint32_t* __restrict__ dist, const uint32_t* __restrict__ pred,
-                            unsigned long long* __restrict__ packed) {
+                            unsigned long long* __restrict__ packed, const uint32_t* done) {
+    if (done && *done) return;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const size_t s = i / V, j = i - s * V;
         const size_t at = s * V + (slots ? __ldg(&slots[j]) : j);
         const uint32_t d = dist[i];
-        packed[at] = d == W::inf_out() ? INF_KEY : ((unsigned long long)d << 32) | pred[i];
+        packed[at] = d == W::inf_out() ? INF_KEY : ((unsigned long long)d << 32) | (pred ? pred[i] : NONE);
     }
 }
 
@@ -1093,7 +1094,9 @@ __global__ void k_warm_seed(SolveLaunch L) {
 
 template <class W>
 __global__ void k_unpack(const unsigned long long* __restrict__ packed, size_t n, uint32_t V,
-                         const uint32_t* __restrict__ slots, uint32_t* __restrict__ dist, uint32_t* __restrict__ pred) {
+                         const uint32_t* __restrict__ slots, uint32_t* __restrict__ dist, uint32_t* __restrict__ pred,
+                         const uint32_t* done) {
+    if (done && *done) return;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         size_t at = i;
@@ -1391,27 +1394,41 @@ cudaError_t relax_max_blocks_per_sm(int wtype, uint32_t threads, uint32_t tile, 
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k, (int)threads, smem);
 }
 
-cudaError_t launch_solve(const SolveLaunch& L, cudaStream_t st) {
+cudaError_t launch_solve(const SolveLaunch& L, const SweepLaunch* sweep, cudaStream_t st) {
     cudaError_t e;
     const size_t n_packed = (size_t)L.S * L.V;
     const size_t n_words = (size_t)L.S * L.words;
     const size_t n_dirty = (size_t)L.S * L.Q;
-    if ((e = cudaMemsetAsync(L.hdr, 0, WS_HEADER_BYTES, st)) != cudaSuccess) return e;  // (also the prune cursor)
-    if ((e = cudaMemsetAsync(L.nfsplit, 0, 4 * n_dirty, st)) != cudaSuccess) return e;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const uint32_t* const done = sweep ? &L.hdr->swept : nullptr;
+    const size_t hdr_bytes =  // (also the prune cursor; with the sweep its counters, which follow)
+        sweep ? (size_t)(reinterpret_cast<char*>(L.packed) - reinterpret_cast<char*>(L.hdr)) : WS_HEADER_BYTES;
+    if ((e = cudaMemsetAsync(L.hdr, 0, hdr_bytes, st)) != cudaSuccess) return e;
+    if (!sweep && (e = cudaMemsetAsync(L.nfsplit, 0, 4 * n_dirty, st)) != cudaSuccess) return e;
     if (L.prune_on && (e = trishla_init(L.prune, st)) != cudaSuccess) return e;
     {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const size_t want = (n_packed / 2 + 255) / 256;
         const unsigned blocks = (unsigned)std::min<size_t>(std::max<size_t>(want, 1), (size_t)sms * 8);
-        if (L.warm) {
+        if (sweep) {
+            if (L.ev_begin && (e = cudaEventRecord(L.ev_begin, st)) != cudaSuccess) return e;
+            if ((e = launch_sweep(*sweep, sms, st)) != cudaSuccess) return e;
+            if ((e = launch_sweep_out(*sweep, sms, st)) != cudaSuccess) return e;
+            // what a sweep that gave up leaves: its queued vertices, and its results as packed words
+            if ((e = launch_sweep_requeue(*sweep, L.bitmap, L.words, L.B, L.Bq, L.split, L.Q, sms, st)) != cudaSuccess)
+                return e;
+            if (L.wtype == SSSP_W_F32)
+                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, done);
+            else
+                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, done);
+        } else if (L.warm) {
             if ((e = cudaMemsetAsync(L.bitmap, 0, 4 * n_words, st)) != cudaSuccess) return e;
             if ((e = cudaMemsetAsync(L.dirty, 0, 4 * n_dirty, st)) != cudaSuccess) return e;
             if (L.wtype == SSSP_W_F32)
-                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed);
+                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, nullptr);
             else
-                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed);
+                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, nullptr);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             const size_t nt = (size_t)L.S * L.n_tails;
             const unsigned tb = (unsigned)std::min<size_t>(std::max<size_t>((nt + 255) / 256, 1), (size_t)sms * 8);
@@ -1425,7 +1442,7 @@ cudaError_t launch_solve(const SolveLaunch& L, cudaStream_t st) {
     }
     const size_t smem = relax_smem_bytes(L.tile, L.Q, L.msg_buffer != 0u);
     void* args[] = {const_cast<SolveLaunch*>(&L)};
-    if (L.ev_begin && (e = cudaEventRecord(L.ev_begin, st)) != cudaSuccess) return e;
+    if (L.ev_begin && !sweep && (e = cudaEventRecord(L.ev_begin, st)) != cudaSuccess) return e;
     {
         const bool pr = L.prune_on != 0u, held = L.msg_buffer != 0u, hubs = L.hub_count != 0u;
         const void* k = L.wtype == SSSP_W_F32 ? solve_kernel<WF32>(pr, held, hubs) : solve_kernel<WU32>(pr, held, hubs);
@@ -1435,14 +1452,11 @@ cudaError_t launch_solve(const SolveLaunch& L, cudaStream_t st) {
     }
     if (L.ev_end && (e = cudaEventRecord(L.ev_end, st)) != cudaSuccess) return e;
     {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         const unsigned blocks = (unsigned)std::min<size_t>(std::max<size_t>((n_packed + 255) / 256, 1), (size_t)sms * 8);
         if (L.wtype == SSSP_W_F32)
-            k_unpack<WF32><<<blocks, 256, 0, st>>>(L.packed, n_packed, L.V, L.slots, L.dist, L.pred);
+            k_unpack<WF32><<<blocks, 256, 0, st>>>(L.packed, n_packed, L.V, L.slots, L.dist, L.pred, done);
         else
-            k_unpack<WU32><<<blocks, 256, 0, st>>>(L.packed, n_packed, L.V, L.slots, L.dist, L.pred);
+            k_unpack<WU32><<<blocks, 256, 0, st>>>(L.packed, n_packed, L.V, L.slots, L.dist, L.pred, done);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // the Trishla chunks the idle blocks did not reach

@@ -1,0 +1,823 @@
+// K4s sweep: all sources of a solve relax the graph together, Bellman-Ford from a frontier.
+//
+// On graphs of small diameter and several edges per vertex (random and power-law graphs) the
+// persistent solve of relax.cu is bound by its chains of dependent rounds when the graph is small,
+// and by random 32-byte sectors, one per edge and source, when it is large.  Here the distances of
+// up to eight sources of a vertex share one sector (dist[item][G], item = group * V + vertex), so a
+// visit of an edge reads its (col, w) once and one sector for all sources of the group.  The
+// visits can be shared because the sources' wavefronts cross such a graph in the same few hops: a
+// vertex whose distance fell for some sources is relaxed for all of its group at once (the lanes of
+// the others cost nothing more).
+//
+// One cooperative launch, bulk synchronous: an iteration takes every marked item, relaxes its row
+// and marks the items whose distances fall, which are the next iteration's; about 20 iterations in
+// all.  There is no bucket order: thresholds above the least queued distance of each source cut the
+// relaxations of random graphs to a third, but took more iterations and a second look at every item,
+// and on power-law graphs cut nothing (R-MAT scale 22, 8 sources: 4.7 against 4.2 ms; random graph of
+// 16,384 vertices: 0.36 against 0.24 ms).
+//   list A : rows of up to 31 edges; a warp takes 32 of them (fewer when the list is short) and
+//            walks their edges together
+//   list M : rows of 32 to 511 edges, up to 8 a warp in the same way
+//   hubs   : rows of SWEEP_HUB edges or more, cut into segments that all warps share
+//   lowered items go to a buffer of the warp and are marked 128 at a time: the chain of a fence, a
+//            mark and a degree would otherwise be paid by every step
+// Predecessors come from one pass over the edges at the end (k_sweep_out): pred(v) is the least
+// label of a tail u with dist(u) + w = dist(v), to which the packed words of the persistent solve
+// converge too.  The loop then needs 4 bytes per vertex and source instead of 8.
+// Measured against the persistent solve, tuned (whole calls): R-MAT scale 22, edge factor 16, 8
+// sources 4.1 against 7.4 ms, DRAM traffic 7.7 against 13.1 GB; R-MAT scale 18, 32 float32 sources
+// 0.66 against 1.0 ms; random graph, 16,384 vertices, 4 partitions, 1 source 0.24 against 1.6 ms.
+// k_sweep (3.0 ms of the 4.1) is bound by the latency of its L2 accesses and by issue slots (44% busy
+// at the 32 warps per SM that 64 registers allow; with 48 warps at 40 registers it spills and is not
+// faster), k_sweep_out (1.0 ms) by random 32-byte sectors, 61 G a second.
+// A graph that is not of that kind (tiny frontiers, many iterations, or many more relaxations than
+// edges) is handed over: marks become inbox bits, distances packed words, and k_solve goes on.
+// Waits: the grid barrier is bounded by the idle limit, the kernel by LIMIT_FACTOR times it.
+#include <algorithm>
+
+#include "common.cuh"
+#include "internal.h"
+
+namespace sssp {
+namespace {
+
+constexpr uint32_t WT = 512, NW = WT / 32;  // threads and warps per block
+constexpr uint32_t SMALL_ROW = 32;          // rows below it: list A
+constexpr uint32_t SEG = 128;               // edges of a hub segment
+constexpr uint32_t BUF = 64;                // a warp's buffer of newly marked items, per list
+constexpr uint32_t MQ = 4, MARKS = MQ * 32;  // items a lane, a warp marks at a time
+constexpr uint32_t OUT_EDGES = 1024;        // most edges a warp of k_sweep_out takes
+constexpr uint64_t LIMIT_FACTOR = 3;
+// Hand-over, looked at every HAND_EVERY iterations: fewer than HAND_EDGES relaxations an iteration,
+// a pace that predicts more than HAND_ITERS iterations, or more than HAND_INFL relaxations per edge
+// and source (random and power-law graphs: 2 to 10).
+constexpr uint32_t HAND_EVERY = 32, HAND_EDGES = 2048, HAND_ITERS = 1024, HAND_INFL = 24;
+
+template <class W>
+struct Dist;
+template <>
+struct Dist<WU32> {
+    static constexpr uint32_t INF = INF32;
+    __device__ __forceinline__ static uint32_t add(uint32_t d, uint32_t w) { return min(d, ~w) + w; }  // saturates
+};
+template <>
+struct Dist<WF32> {
+    static constexpr uint32_t INF = F32_INF_BITS;
+    __device__ __forceinline__ static uint32_t add(uint32_t d, uint32_t w) {
+        return __float_as_uint(__fadd_rn(__uint_as_float(d), __uint_as_float(w)));  // +inf stays
+    }
+};
+
+struct WarpMem {                              // shared memory of a warp, besides the distances it holds
+    uint4 row[32];                            // rows held: first edge - edges before it, group base, largest distance
+    uint32_t bufA[BUF], bufM[BUF];
+    uint32_t low[MARKS];                      // items whose distances were lowered, to be marked
+    unsigned long long edges;                 // statistics of the launch
+    uint32_t act, vert;
+};
+
+struct BlockMem {
+    uint32_t c[8];
+    uint32_t wA[NW], wM[NW];
+    unsigned long long work, at, imp;
+    uint32_t next;  // the block's next unit of work
+    int ok;
+};
+
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
+// The G distances of an item from L2 (rows are aligned to their size, 32 bytes at most): one
+// 256-bit load for eight (two 128-bit ones made twice the L1 and L2 requests).  Not ordered with
+// other accesses by the compiler: what an older value lets through is settled by the atomic.
+template <int G>
+__device__ __forceinline__ void load_row(const uint32_t* p, uint32_t (&r)[G]) {
+    if constexpr (G == 8) {
+        asm volatile("ld.relaxed.gpu.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                     : "l"(p));
+    } else if constexpr (G == 4) {
+        const uint4 a = __ldcg(reinterpret_cast<const uint4*>(p));
+        r[0] = a.x, r[1] = a.y, r[2] = a.z, r[3] = a.w;
+    } else if constexpr (G == 2) {
+        const uint2 a = __ldcg(reinterpret_cast<const uint2*>(p));
+        r[0] = a.x, r[1] = a.y;
+    } else {
+        r[0] = __ldcg(p);
+    }
+}
+
+// the same from data that no longer changes (through L1: lanes share rows)
+template <int G>
+__device__ __forceinline__ void load_final(const uint32_t* p, uint32_t (&r)[G]) {
+    if constexpr (G == 8) {
+        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+            : "l"(p));
+    } else if constexpr (G == 4) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4*>(p));
+        r[0] = a.x, r[1] = a.y, r[2] = a.z, r[3] = a.w;
+    } else if constexpr (G == 2) {
+        const uint2 a = __ldg(reinterpret_cast<const uint2*>(p));
+        r[0] = a.x, r[1] = a.y;
+    } else {
+        r[0] = __ldg(p);
+    }
+}
+
+template <int G>
+__device__ __forceinline__ void shared_row(const uint32_t* p, uint32_t (&r)[G]) {
+    if constexpr (G >= 4) {
+#pragma unroll
+        for (int i = 0; i < G; i += 4) {
+            const uint4 a = *reinterpret_cast<const uint4*>(p + i);
+            r[i] = a.x, r[i + 1] = a.y, r[i + 2] = a.z, r[i + 3] = a.w;
+        }
+    } else {
+#pragma unroll
+        for (int s = 0; s < G; ++s) r[s] = p[s];
+    }
+}
+
+// All blocks arrive and wait; false once a limit has run out or another block gave up.
+__device__ bool grid_barrier(const SweepLaunch& L, BlockMem& bm, uint32_t& n, uint64_t t_begin) {
+    ++n;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(&L.ctl->bar, 1u);
+        const uint32_t target = n * gridDim.x;
+        const uint64_t t0 = globaltimer_ns();
+        bool late = t0 - t_begin > LIMIT_FACTOR * L.timeout_ns, stop = false;
+        while (!late && !stop && (int32_t)(ld_acquire(&L.ctl->bar) - target) < 0) {
+            stop = ld_relaxed(&L.hdr->abort_flag) != 0u;
+            late = globaltimer_ns() - t0 > L.timeout_ns;
+        }
+        if (late) {
+            set_status(L.hdr, SSSP_ETIMEOUT);
+            atomicExch(&L.hdr->abort_flag, 1u);
+        }
+        __threadfence();
+        bm.ok = !late && !stop;
+    }
+    __syncthreads();
+    return bm.ok != 0;
+}
+
+template <class W, int G>
+struct Worker {
+    const SweepLaunch& L;
+    WarpMem& wm;
+    uint32_t* du;  // [32][G] distances of the rows held
+    BlockMem& bm;
+    uint32_t lane;
+    uint32_t* list;              // list being filled (A from the front, M from the back)
+    SweepIter* it;               // its counters
+    unsigned long long* ex_out;  // hub entries being filled
+    uint32_t nA, nM, nC;         // buffered items: new in the lists, to be marked (warp-uniform)
+    uint32_t bad, s_at, s_imp;
+
+    __device__ __forceinline__ uint32_t vertex(uint32_t item) const { return L.groups == 1u ? item : item % L.V; }
+
+    __device__ __forceinline__ void put(uint32_t at, uint32_t item, bool back) {
+        list[back ? L.items - 1u - at : at] = item;
+    }
+
+    __device__ __forceinline__ void flush_full(uint32_t* buf, uint32_t& n, uint32_t* cnt, bool back) {
+        uint32_t base = 0;
+        if (lane == 0) base = atomicAdd(cnt, 32u);
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        put(base + lane, buf[lane], back);
+        n -= 32u;
+        const uint32_t x = buf[32u + lane];
+        __syncwarp();
+        buf[lane] = x;
+        __syncwarp();
+    }
+
+    // newly marked items of the lanes with `has` (and an edge): hubs get their entry, the others go
+    // to the warp's buffers
+    __device__ __forceinline__ void push(bool has, uint32_t item, uint32_t deg) {
+        has = has && deg != 0u;
+        if (has && deg >= SWEEP_HUB) {
+            const unsigned long long at = atomicAdd(&it->ex, (1ull << 32) | ((deg + SEG - 1u) / SEG));
+            ex_out[at >> 32] = ((unsigned long long)(uint32_t)at << 32) | item;
+            has = false;
+        }
+        const uint32_t ba = __ballot_sync(0xFFFFFFFFu, has && deg < SMALL_ROW);
+        const uint32_t bmm = __ballot_sync(0xFFFFFFFFu, has && deg >= SMALL_ROW);
+        const uint32_t lt = (1u << lane) - 1u;
+        if (has) {
+            if (deg < SMALL_ROW)
+                wm.bufA[nA + __popc(ba & lt)] = item;
+            else
+                wm.bufM[nM + __popc(bmm & lt)] = item;
+        }
+        nA += __popc(ba);
+        nM += __popc(bmm);
+        __syncwarp();
+        if (nA >= 32u) flush_full(wm.bufA, nA, &it->nA, false);
+        if (nM >= 32u) flush_full(wm.bufM, nM, &it->nM, true);
+    }
+
+    // the leftovers of all warps of the block, with one atomic per list (called by every thread)
+    __device__ __forceinline__ void flush_block() {
+        if (!__syncthreads_or((int)(nA | nM))) return;
+        const uint32_t wid = threadIdx.x >> 5;
+        if (lane == 0) bm.wA[wid] = nA, bm.wM[wid] = nM;
+        __syncthreads();
+        if (threadIdx.x < 32u) {
+            // lanes 0..15: list A, lanes 16..31: list M
+            const bool m = lane >= NW;
+            uint32_t* const c = m ? bm.wM : bm.wA;
+            const uint32_t x = c[lane % NW];
+            uint32_t inc = x;
+#pragma unroll
+            for (uint32_t o = 1; o < NW; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o, NW);
+                if (lane % NW >= o) inc += y;
+            }
+            uint32_t base = 0;
+            if (lane % NW == NW - 1u && inc) base = atomicAdd(m ? &it->nM : &it->nA, inc);
+            base = __shfl_sync(0xFFFFFFFFu, base, NW - 1, NW);
+            c[lane % NW] = base + inc - x;
+        }
+        __syncthreads();
+        for (uint32_t i = lane; i < nA; i += 32u) put(bm.wA[wid] + i, wm.bufA[i], false);
+        for (uint32_t i = lane; i < nM; i += 32u) put(bm.wM[wid] + i, wm.bufM[i], true);
+        nA = nM = 0;
+    }
+
+    // Takes the item of each lane with `ok`: its mark is cleared before its distances are read, so a
+    // distance lowered after the read marks it again.
+    __device__ __forceinline__ void take(bool ok, uint32_t item, uint32_t (&r)[G]) {
+#pragma unroll
+        for (int s = 0; s < G; ++s) r[s] = Dist<W>::INF;
+        if (ok) {
+            atomicAnd(&L.mark[item >> 5], ~(1u << (item & 31u)));
+            fence_gpu();
+            load_row<G>(L.dist + (size_t)item * G, r);
+        }
+    }
+
+    // a row into slot `at` (off: its first edge less the edges of the rows before it); returns its
+    // count of finite distances
+    __device__ __forceinline__ uint32_t hold(uint32_t at, const uint32_t (&r)[G], uint32_t item, uint32_t off) {
+        uint32_t fin = 0, mx = 0;
+#pragma unroll
+        for (int s = 0; s < G; ++s)
+            if (r[s] < Dist<W>::INF) ++fin, mx = max(mx, r[s]);
+        if constexpr (G >= 4) {
+#pragma unroll
+            for (int s = 0; s < G; s += 4)
+                *reinterpret_cast<uint4*>(du + at * G + s) = make_uint4(r[s], r[s + 1], r[s + 2], r[s + 3]);
+        } else {
+#pragma unroll
+            for (int s = 0; s < G; ++s) du[at * G + s] = r[s];
+        }
+        wm.row[at] = make_uint4(off, L.groups == 1u ? 0u : item - item % L.V, mx, 0u);
+        return fin;
+    }
+
+    // Marks the nC buffered items, whose distances this warp has lowered, MQ a lane with their
+    // accesses in flight together; newly marked ones go to the list being filled.
+    __device__ __forceinline__ void mark_all() {
+        __syncwarp();
+        fence_gpu();  // the lowered distances before the marks
+        // Most lowered items are marked already: a mark seen here is cleared, if it is, after the fence,
+        // and the distances are read after that.
+        uint32_t fresh = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < MQ; ++i) {
+            const uint32_t x = i * 32u + lane;
+            if (x < nC) {
+                const uint32_t item = wm.low[x];
+                if (!(ld_relaxed(&L.mark[item >> 5]) >> (item & 31u) & 1u)) fresh |= 1u << i;
+            }
+        }
+        uint32_t nact = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < MQ; ++i) {
+            bool f = fresh & (1u << i);
+            if (!__any_sync(0xFFFFFFFFu, f)) continue;
+            uint32_t item = 0, deg = 0;
+            if (f) {
+                item = wm.low[i * 32u + lane];
+                const uint32_t v = vertex(item), bit = 1u << (item & 31u);
+                const uint32_t r0 = __ldg(&L.row_ptr[v]), r1 = __ldg(&L.row_ptr[v + 1]);  // in flight with the atomic
+                f = !(atomicOr(&L.mark[item >> 5], bit) & bit);
+                deg = r1 - r0;
+            }
+            nact += __popc(__ballot_sync(0xFFFFFFFFu, f));
+            push(f, item, deg);
+        }
+        if (lane == 0) wm.act += nact;
+        nC = 0;
+        __syncwarp();
+    }
+
+    // Relaxes edges [0, total) of the rows held.  Row r's edges start at the value p of lane r
+    // (ascending, every row has an edge; lanes without a row: none), so the rows that start within
+    // the 32 edges of a step are a bit mask, and a lane's row is the count of starts up to it.
+    // A pipeline of three: the (col, w) of the steps after next, the distances of the next ones and
+    // the atomics of these are in flight together (EB steps each: eight distances a lane).
+    __device__ __forceinline__ void relax(uint32_t total, uint32_t p) {
+        constexpr int EB = G >= 8 ? 1 : G == 4 ? 2 : 4;
+        uint32_t v[EB], w[EB], a[EB];              // steps after next: head, weight, row
+        uint32_t x[EB], y[EB], b[EB], d[EB][G];    // next steps: item, weight, row, its distances
+        uint32_t seen = 0;                         // rows that start before the step
+        auto fetch = [&](uint32_t k0) {            // k0: first edge of the steps
+#pragma unroll
+            for (int j = 0; j < EB; ++j) {
+                const uint32_t at = k0 + 32u * j;
+                v[j] = NONE;
+                if (at >= total) continue;
+                const uint32_t starts = __reduce_or_sync(0xFFFFFFFFu, p - at < 32u ? 1u << (p - at) : 0u);
+                a[j] = seen + __popc(starts & (0xFFFFFFFFu >> (31u - lane))) - 1u;
+                seen += __popc(starts);
+                if (at + lane < total) {
+                    const uint32_t e = wm.row[a[j]].x + at + lane;
+                    v[j] = __ldg(&L.col[e]);
+                    w[j] = __ldg(&L.w[e]);
+                }
+            }
+        };
+        auto heads = [&]() {
+#pragma unroll
+            for (int j = 0; j < EB; ++j) {
+                x[j] = v[j];
+                y[j] = w[j];
+                b[j] = a[j];
+                if (x[j] == NONE) continue;
+                if (!W::weight_ok(y[j]) || x[j] >= L.V) {
+                    bad |= 1u;
+                    x[j] = NONE;
+                } else {
+                    const uint4 rw = wm.row[b[j]];
+                    uint32_t z;
+                    if (!W::add(rw.z, y[j], z)) bad |= 2u;
+                    x[j] += rw.y;
+                    load_row<G>(L.dist + (size_t)x[j] * G, d[j]);
+                }
+            }
+        };
+        fetch(0);
+        heads();
+        fetch(32u * EB);
+        for (uint32_t k0 = 0; k0 < total; k0 += 32u * EB) {
+            // these steps: candidates c where they beat the distances read, else INF
+            uint32_t c[EB][G], it_[EB], imp[EB], any = 0;
+#pragma unroll
+            for (int j = 0; j < EB; ++j) {
+                it_[j] = x[j];
+                imp[j] = 0;
+                if (x[j] != NONE) {
+                    uint32_t dj[G];
+                    shared_row<G>(du + b[j] * G, dj);
+#pragma unroll
+                    for (int s = 0; s < G; ++s) {
+                        c[j][s] = Dist<W>::add(dj[s], y[j]);
+                        if (c[j][s] < d[j][s]) imp[j] |= 1u << s;
+                    }
+                }
+                any |= imp[j];
+            }
+            heads();
+            fetch(k0 + 64u * EB);
+            if (!__any_sync(0xFFFFFFFFu, any != 0u)) continue;
+            uint32_t low[EB];
+#pragma unroll
+            for (int j = 0; j < EB; ++j) {
+                low[j] = 0;
+                uint32_t* const row = L.dist + (size_t)it_[j] * G;
+                uint32_t old[G];
+#pragma unroll
+                for (int s = 0; s < G; ++s) {
+                    old[s] = 0;
+                    if (imp[j] & (1u << s)) old[s] = atomicMin(row + s, c[j][s]);
+                }
+#pragma unroll
+                for (int s = 0; s < G; ++s)
+                    if (old[s] > c[j][s]) low[j] |= imp[j] & (1u << s);
+            }
+            uint32_t na = 0, nl = 0;
+#pragma unroll
+            for (int j = 0; j < EB; ++j) {
+                na += __popc(imp[j]);
+                nl += __popc(low[j]);
+                const uint32_t bl = __ballot_sync(0xFFFFFFFFu, low[j] != 0u);
+                if (!bl) continue;
+                if (low[j]) wm.low[nC + __popc(bl & ((1u << lane) - 1u))] = it_[j];
+                nC += __popc(bl);
+                if (nC > MARKS - 32u) mark_all();
+            }
+            s_at += na;
+            s_imp += nl;
+        }
+    }
+
+    // An iteration's work: hub segments, then the rows of M, then those of A, in units that the
+    // block's warps take in turn (unit i of block b is unit b + i * blocks of the iteration).
+    __device__ __forceinline__ void work(const uint32_t* in, const unsigned long long* ex, uint32_t cA, uint32_t cM,
+                                         uint32_t cX, uint32_t segs) {
+        const uint32_t TW = gridDim.x * NW;
+        // segments and rows of a unit: fewer when there are few, so that all warps get some
+        const uint32_t rX = min(max(segs / (2u * TW), 1u), 8u), rM = min(max(cM / TW, 1u), 8u);
+        const uint32_t rA = cA >= TW * 32u ? 32u : cA >= TW * 16u ? 16u : 8u;
+        const uint32_t uX = (segs + rX - 1u) / rX, uM = (cM + rM - 1u) / rM, uA = (cA + rA - 1u) / rA;
+        uint32_t t = 0, t1 = 0, k = 0;  // hub segments of the unit, entry of the first
+        for (;;) {
+            uint32_t total = 0, p = 0xFFFFFFFFu;
+            if (t >= t1) {
+                uint32_t u = 0;
+                if (lane == 0) u = atomicAdd(&bm.next, 1u);
+                u = blockIdx.x + __shfl_sync(0xFFFFFFFFu, u, 0) * gridDim.x;
+                if (u < uX) {
+                    t = u * rX;
+                    t1 = min(t + rX, segs);
+                    k = 0;  // last entry whose start is <= t: 32-way search of start << 32 | item
+                    uint32_t len = cX;
+                    while (len > 1u) {
+                        const uint32_t step = (len + 31u) / 32u, i = lane * step;
+                        const bool le = i < len && (uint32_t)(__ldcg(&ex[k + i]) >> 32) <= t;
+                        const uint32_t f = 31u - (uint32_t)__clz(__ballot_sync(0xFFFFFFFFu, le));
+                        k += f * step;
+                        len = min(step, len - f * step);
+                    }
+                } else if (u < uX + uM + uA) {
+                    const bool m = u < uX + uM;
+                    const uint32_t c = m ? (u - uX) * rM : (u - uX - uM) * rA;
+                    const bool ok = lane < (m ? rM : rA) && c + lane < (m ? cM : cA);
+                    uint32_t item = 0, beg = 0, deg = 0, r[G];
+                    if (ok) {
+                        item = __ldcg(&in[m ? L.items - 1u - (c + lane) : c + lane]);
+                        const uint32_t x = vertex(item);
+                        beg = __ldg(&L.row_ptr[x]);
+                        deg = __ldg(&L.row_ptr[x + 1]) - beg;
+                    }
+                    take(ok, item, r);
+                    uint32_t inc = deg;
+#pragma unroll
+                    for (uint32_t o = 1; o < 32u; o <<= 1) {
+                        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+                        if (lane >= o) inc += y;
+                    }
+                    const uint32_t fin = hold(lane, r, item, beg - (inc - deg));
+                    if (ok) p = inc - deg;
+                    total = __shfl_sync(0xFFFFFFFFu, inc, 31);
+                    const uint32_t se = __reduce_add_sync(0xFFFFFFFFu, fin * deg), sv = __reduce_add_sync(0xFFFFFFFFu, fin);
+                    if (lane == 0) wm.edges += se, wm.vert += sv;
+                } else {
+                    break;
+                }
+            }
+            if (t < t1) {  // the unit's segments of one hub (its mark was cleared before the iteration)
+                const unsigned long long x = __ldcg(&ex[k]);
+                const uint32_t item = (uint32_t)x, u = vertex(item), s0 = t - (uint32_t)(x >> 32);
+                const uint32_t beg = __ldg(&L.row_ptr[u]) + s0 * SEG, left = __ldg(&L.row_ptr[u + 1]) - beg;
+                const uint32_t n = min((left + SEG - 1u) / SEG, t1 - t);
+                total = min(left, n * SEG);
+                if (lane == 0) {
+                    uint32_t r[G];
+                    load_row<G>(L.dist + (size_t)item * G, r);
+                    const uint32_t fin = hold(0, r, item, beg);
+                    wm.edges += (unsigned long long)fin * total;
+                    if (s0 == 0) wm.vert += fin;
+                    p = 0;
+                }
+                t += n;
+                ++k;
+            }
+            __syncwarp();
+            relax(total, p);
+            __syncwarp();
+        }
+        if (nC) mark_all();
+    }
+};
+
+// Every distance to INF, marks to zero, predecessors to NONE.
+__global__ void k_sweep_init(SweepLaunch L, uint32_t inf) {
+    const size_t stride = (size_t)gridDim.x * blockDim.x, i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const size_t nd = (size_t)L.items * L.G;
+    uint4* d4 = reinterpret_cast<uint4*>(L.dist);
+    for (size_t i = i0; i < nd / 4; i += stride) d4[i] = make_uint4(inf, inf, inf, inf);
+    if (i0 < (nd & 3u)) L.dist[(nd & ~(size_t)3) + i0] = inf;
+    for (size_t i = i0; i < ((size_t)L.items + 31) / 32; i += stride) L.mark[i] = 0u;
+    for (size_t i = i0; i < L.n_dirty; i += stride) L.dirty[i] = 0u, L.nfsplit[i] = 0u;
+    if (L.pred)
+        for (size_t i = i0; i < (size_t)L.S * L.V; i += stride) L.pred[i] = NONE;
+}
+
+template <class W, int G>
+__global__ void __launch_bounds__(WT, 2) k_sweep(SweepLaunch L) {
+    extern __shared__ __align__(16) uint32_t dsm[];  // [NW][32][G] rows
+    __shared__ BlockMem bm;
+    __shared__ WarpMem wmem[NW];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, wid = tid >> 5;
+    WarpMem& wm = wmem[wid];
+    const uint64_t t_begin = globaltimer_ns();
+    uint32_t nbar = 0;
+    if (tid == 0) bm.work = bm.at = bm.imp = 0ull;
+    if (lane == 0) {
+        wm.edges = 0ull;
+        wm.act = wm.vert = 0u;
+    }
+    if (blockIdx.x == 0) {  // seeds
+        for (uint32_t s = tid; s < L.S; s += WT) {
+            uint32_t src = L.sources[s];
+            if (src >= L.V) {
+                set_status(L.hdr, SSSP_EINVAL);
+                continue;
+            }
+            if (L.slots) src = L.slots[src];
+            const uint32_t item = s / G * L.V + src, bit = 1u << (item & 31u);
+            L.dist[(size_t)item * G + s % G] = 0u;
+            if (atomicOr(&L.mark[item >> 5], bit) & bit) continue;
+            const uint32_t deg = __ldg(&L.row_ptr[src + 1]) - __ldg(&L.row_ptr[src]);
+            if (deg >= SWEEP_HUB) {
+                const unsigned long long at = atomicAdd(&L.ctl->it[0].ex, (1ull << 32) | ((deg + SEG - 1u) / SEG));
+                L.ex[0][at >> 32] = ((unsigned long long)(uint32_t)at << 32) | item;
+            } else if (deg >= SMALL_ROW) {
+                L.list[0][L.items - 1u - atomicAdd(&L.ctl->it[0].nM, 1u)] = item;
+            } else if (deg) {
+                L.list[0][atomicAdd(&L.ctl->it[0].nA, 1u)] = item;
+            }
+        }
+    }
+    uint32_t slot = 0, par = 0, iters = 0;
+    unsigned long long work = 0;
+    const unsigned long long all = (unsigned long long)L.E * L.S;
+    bool done = false;
+    while (grid_barrier(L, bm, nbar, t_begin)) {
+        if (tid < 2u) {  // the counters of this iteration (nobody adds to them any more)
+            const uint4 x = __ldcg(reinterpret_cast<const uint4*>(&L.ctl->it[slot]) + tid);
+            bm.next = 0u;
+            bm.c[tid * 4] = x.x, bm.c[tid * 4 + 1] = x.y, bm.c[tid * 4 + 2] = x.z, bm.c[tid * 4 + 3] = x.w;
+        }
+        __syncthreads();
+        const uint32_t cA = bm.c[0], cM = bm.c[1], segs = bm.c[2], cX = bm.c[3];
+        work += ((unsigned long long)bm.c[5] << 32) | bm.c[4];
+        if (!(cA | cM | cX)) {
+            done = true;
+            break;
+        }
+        const uint32_t next = slot == 2u ? 0u : slot + 1u, after = next == 2u ? 0u : next + 1u;
+        if (blockIdx.x == 0 && tid == 0) {  // its counters were last read before this barrier
+            SweepIter& z = L.ctl->it[after];
+            z.nA = z.nM = 0u;
+            z.ex = z.work = 0ull;
+        }
+        ++iters;
+        if (iters % HAND_EVERY == 0u &&
+            (work < (unsigned long long)iters * HAND_EDGES || all / (work + 1ull) * iters > HAND_ITERS ||
+             work / HAND_INFL > all))
+            break;  // the listed items keep their marks
+        if (cX) {
+            // hubs are taken before the iteration, since several warps relax one: a distance that
+            // falls from here on marks it again
+            for (uint32_t i = blockIdx.x * WT + tid; i < cX; i += gridDim.x * WT) {
+                const uint32_t item = (uint32_t)__ldcg(&L.ex[par][i]);
+                atomicAnd(&L.mark[item >> 5], ~(1u << (item & 31u)));
+            }
+            if (!grid_barrier(L, bm, nbar, t_begin)) break;
+        }
+        Worker<W, G> wk{L, wm, dsm + wid * 32u * G, bm, lane, L.list[par ^ 1u], &L.ctl->it[next], L.ex[par ^ 1u], 0, 0, 0, 0, 0, 0};
+        const unsigned long long before = wm.edges;
+        wk.work(L.list[par], L.ex[par], cA, cM, cX, segs);
+        wk.bad = __reduce_or_sync(0xFFFFFFFFu, wk.bad);
+        wk.s_at = __reduce_add_sync(0xFFFFFFFFu, wk.s_at);
+        wk.s_imp = __reduce_add_sync(0xFFFFFFFFu, wk.s_imp);
+        if (lane == 0) {
+            if (wk.s_at) atomicAdd(&bm.at, (unsigned long long)wk.s_at);
+            if (wk.s_imp) atomicAdd(&bm.imp, (unsigned long long)wk.s_imp);
+            if (wm.edges != before) atomicAdd(&bm.work, wm.edges - before);
+            if (wk.bad & 1u) set_status(L.hdr, SSSP_EINVAL);
+            if (wk.bad & 2u) set_status(L.hdr, SSSP_EOVERFLOW);
+        }
+        wk.flush_block();
+        if (tid == 0 && bm.work) {
+            atomicAdd(&L.ctl->it[next].work, bm.work);
+            bm.work = 0ull;
+        }
+        slot = next;
+        par ^= 1u;
+    }
+    __syncthreads();
+    if (lane == 0) {  // edges_scanned, atomics, improved, activations, vertices
+        if (wm.edges) atomicAdd(&L.hdr->stats[0], wm.edges);
+        if (wm.act) atomicAdd(&L.hdr->stats[3], (unsigned long long)wm.act);
+        if (wm.vert) atomicAdd(&L.hdr->stats[5], (unsigned long long)wm.vert);
+    }
+    if (tid == 0) {
+        if (bm.at) atomicAdd(&L.hdr->stats[1], bm.at);
+        if (bm.imp) atomicAdd(&L.hdr->stats[2], bm.imp);
+    }
+    if (blockIdx.x == 0 && tid == 0) {
+        atomicAdd(&L.hdr->stats[4], (unsigned long long)iters);
+        L.hdr->swept = done ? 1u : 0u;
+    }
+}
+
+// The results: distances in the caller's order, and predecessors by one pass over the edges.  A
+// warp takes a range of edges (its first row by a 32-way search of row_ptr) and holds the starts of
+// the rows with an edge among 32 rows at a time, one a lane, so that a lane finds its row as in
+// relax().  The (col, w) of the step after next and the heads' distances of the next one are in
+// flight while a step is compared; the tails' distances come through L1.
+template <class W, int G>
+__global__ void __launch_bounds__(256) k_sweep_out(SweepLaunch L, uint32_t per) {
+    __shared__ uint32_t rows[8][32], starts[8][32];
+    using D = Dist<W>;
+    const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+    for (uint32_t g = 0; g < L.groups; ++g) {
+        for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < L.V; c += gridDim.x * blockDim.x) {
+            const uint32_t at = L.slots ? __ldg(&L.slots[c]) : c;
+            uint32_t r[G];
+            load_final<G>(L.dist + ((size_t)g * L.V + at) * G, r);
+#pragma unroll
+            for (int s = 0; s < G; ++s)
+                if (g * G + s < L.S) L.out[(size_t)(g * G + s) * L.V + c] = r[s];
+        }
+    }
+    if (!L.pred) return;
+    const unsigned long long first = (unsigned long long)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;
+    if (first >= L.E) return;
+    const uint32_t e0 = (uint32_t)first, e1 = (uint32_t)min(first + per, (unsigned long long)L.E);
+    uint32_t lo = 0, len = L.V;  // last row r with row_ptr[r] <= e0
+    while (len > 1u) {
+        const uint32_t step = (len + 31u) / 32u, i = lane * step;
+        const bool le = i < len && __ldg(&L.row_ptr[lo + i]) <= e0;
+        const uint32_t k = 31u - (uint32_t)__clz(__ballot_sync(0xFFFFFFFFu, le) | 1u);
+        lo += k * step;
+        len = min(step, len - k * step);
+    }
+    uint32_t* const row = rows[wid];
+    uint32_t r0 = lo, p, end, seen;  // the window: its first row, the start of the lane's row, its last edge, rows passed
+    auto window = [&]() {
+        const uint32_t r = r0 + lane;
+        const uint32_t a = __ldg(&L.row_ptr[min(r, L.V)]), b = __ldg(&L.row_ptr[min(r + 1u, L.V)]);
+        const bool has = b > a;
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, has), k = __popc(m & ((1u << lane) - 1u));
+        __syncwarp();
+        if (has) row[k] = r, starts[wid][k] = a;
+        __syncwarp();
+        p = lane < (uint32_t)__popc(m) ? starts[wid][lane] : 0xFFFFFFFFu;
+        end = __shfl_sync(0xFFFFFFFFu, b, 31);
+        seen = 0;
+    };
+    window();
+    seen = __popc(__ballot_sync(0xFFFFFFFFu, p < e0));
+    uint32_t v = 0, w = 0;  // the step after next
+    auto fetch = [&](uint32_t e) {
+        v = NONE;
+        if (e < e1) v = __ldg(&L.col[e]), w = __ldg(&L.w[e]);
+        if (v != NONE && (v >= L.V || !W::weight_ok(w))) v = NONE;  // (reported by the sweep)
+    };
+    uint32_t x, y, h[G];  // the next step: head, weight, and (one group) the head's distances
+    auto heads = [&]() {
+        x = v;
+        y = w;
+        if (L.groups == 1u && x != NONE) load_final<G>(L.dist + (size_t)x * G, h);
+    };
+    fetch(e0 + lane);
+    heads();
+    fetch(e0 + 32u + lane);
+    for (uint32_t eb = e0; eb < e1; eb += 32u) {
+        // rows of the step's edges
+        uint32_t u = 0;
+        for (;;) {
+            const uint32_t at = __reduce_or_sync(0xFFFFFFFFu, p - eb < 32u ? 1u << (p - eb) : 0u);
+            // (a lane at or past the window's end finds its row in a later window, and overwrites this)
+            const uint32_t k = seen + __popc(at & (0xFFFFFFFFu >> (31u - lane)));
+            if (k) u = row[k - 1u];
+            seen += __popc(at);
+            if (end >= min(eb + 32u, e1)) break;
+            r0 += 32u;
+            window();
+        }
+        uint32_t hv[G];
+        const uint32_t head = x, wt = y;
+#pragma unroll
+        for (int s = 0; s < G; ++s) hv[s] = h[s];
+        heads();
+        fetch(eb + 64u + lane);
+        if (head == NONE) continue;
+        for (uint32_t g = 0; g < L.groups; ++g) {
+            uint32_t a[G];
+            load_final<G>(L.dist + ((size_t)g * L.V + u) * G, a);
+            if (L.groups != 1u) load_final<G>(L.dist + ((size_t)g * L.V + head) * G, hv);
+            uint32_t tight = 0;
+#pragma unroll
+            for (int s = 0; s < G; ++s)
+                if (D::add(a[s], wt) == hv[s]) tight |= 1u << s;
+            if (tight) {
+                const uint32_t lab = L.ids ? __ldg(&L.ids[u]) : u, to = L.ids ? __ldg(&L.ids[head]) : head;
+#pragma unroll
+                for (int s = 0; s < G; ++s)
+                    if ((tight & (1u << s)) && hv[s] < D::INF) atomicMin(&L.pred[(size_t)(g * G + s) * L.V + to], lab);
+            }
+        }
+    }
+}
+
+// Handed over: the marked vertices become inbox bits of the sources that have reached them, their
+// units' doorbells are rung and they are counted.  One thread per inbox word (G = 1: the marks are
+// the inbox words already).
+template <int G>
+__global__ void k_sweep_requeue(SweepLaunch L, uint32_t* bitmap, uint32_t words, uint32_t B, uint32_t Bq, uint32_t split,
+                                uint32_t Q) {
+    if (L.hdr->swept) return;
+    const size_t n = (size_t)L.S * words, stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        const uint32_t s = (uint32_t)(i / words), wd = (uint32_t)(i - (size_t)s * words);
+        uint32_t bits = 0;
+        for (uint32_t j = 0; j < 32u && wd * 32u + j < L.V; ++j) {
+            const uint32_t item = s / G * L.V + wd * 32u + j;
+            if ((L.mark[item >> 5] >> (item & 31u) & 1u) && L.dist[(size_t)item * G + s % G] < L.inf) bits |= 1u << j;
+        }
+        bitmap[i] = bits;
+        if (!bits) continue;
+        atomicAdd(&L.hdr->pending, (unsigned long long)__popc(bits));
+        while (bits) {
+            const uint32_t v = wd * 32u + (uint32_t)__ffs(bits) - 1u;
+            bits &= bits - 1u;
+            const uint32_t p = v / B;
+            L.dirty[(size_t)s * Q + p * split + (v - p * B) / Bq] = 1u;
+        }
+    }
+}
+
+template <class W>
+const void* sweep_kernel(uint32_t G) {
+    switch (G) {
+        case 1: return (const void*)k_sweep<W, 1>;
+        case 2: return (const void*)k_sweep<W, 2>;
+        case 4: return (const void*)k_sweep<W, 4>;
+        default: return (const void*)k_sweep<W, 8>;
+    }
+}
+
+template <class W>
+void out_kernel(const SweepLaunch& L, uint32_t per, unsigned grid, cudaStream_t st) {
+    switch (L.G) {
+        case 1: k_sweep_out<W, 1><<<grid, 256, 0, st>>>(L, per); break;
+        case 2: k_sweep_out<W, 2><<<grid, 256, 0, st>>>(L, per); break;
+        case 4: k_sweep_out<W, 4><<<grid, 256, 0, st>>>(L, per); break;
+        default: k_sweep_out<W, 8><<<grid, 256, 0, st>>>(L, per); break;
+    }
+}
+
+size_t sweep_smem(uint32_t G) { return 4 * (size_t)NW * 32 * G; }
+
+}  // namespace
+
+cudaError_t sweep_max_blocks_per_sm(int wtype, uint32_t G, int* out) {
+    const void* k = wtype == SSSP_W_F32 ? sweep_kernel<WF32>(G) : sweep_kernel<WU32>(G);
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem(G))) != cudaSuccess)
+        return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k, (int)WT, sweep_smem(G));
+}
+
+cudaError_t launch_sweep(const SweepLaunch& L, int sms, cudaStream_t st) {
+    cudaError_t e;
+    const size_t n = std::max((size_t)L.items * L.G / 4, L.pred ? (size_t)L.S * L.V : (size_t)1);
+    const unsigned blocks = (unsigned)std::min<size_t>(std::max<size_t>((n + 255) / 256, 1), (size_t)sms * 8);
+    k_sweep_init<<<blocks, 256, 0, st>>>(L, L.inf);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    const void* k = L.wtype == SSSP_W_F32 ? sweep_kernel<WF32>(L.G) : sweep_kernel<WU32>(L.G);
+    void* args[] = {const_cast<SweepLaunch*>(&L)};
+    return cudaLaunchCooperativeKernel(k, dim3(L.grid), dim3(WT), args, sweep_smem(L.G), st);
+}
+
+cudaError_t launch_sweep_out(const SweepLaunch& L, int sms, cudaStream_t st) {
+    // a range per warp: long enough to pay for its search, short enough to give every warp one
+    const uint32_t per = (uint32_t)std::min<uint64_t>(std::max<uint64_t>((L.E / ((uint64_t)sms * 64) + 31) & ~31ull, 64),
+                                                      OUT_EDGES);
+    const uint64_t edges = ((uint64_t)L.E + 8 * per - 1) / (8 * per);
+    const unsigned grid = (unsigned)std::max<uint64_t>(edges, std::min<uint64_t>((L.V + 255) / 256, (uint64_t)sms * 8));
+    if (L.wtype == SSSP_W_F32)
+        out_kernel<WF32>(L, per, grid, st);
+    else
+        out_kernel<WU32>(L, per, grid, st);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sweep_requeue(const SweepLaunch& L, uint32_t* bitmap, uint32_t words, uint32_t B, uint32_t Bq,
+                                 uint32_t split, uint32_t Q, int sms, cudaStream_t st) {
+    const unsigned grid = (unsigned)std::min<uint64_t>(((uint64_t)L.S * words + 255) / 256, (uint64_t)sms * 8);
+    switch (L.G) {
+        case 1: k_sweep_requeue<1><<<grid, 256, 0, st>>>(L, bitmap, words, B, Bq, split, Q); break;
+        case 2: k_sweep_requeue<2><<<grid, 256, 0, st>>>(L, bitmap, words, B, Bq, split, Q); break;
+        case 4: k_sweep_requeue<4><<<grid, 256, 0, st>>>(L, bitmap, words, B, Bq, split, Q); break;
+        default: k_sweep_requeue<8><<<grid, 256, 0, st>>>(L, bitmap, words, B, Bq, split, Q); break;
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace sssp
