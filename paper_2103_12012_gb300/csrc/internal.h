@@ -167,6 +167,7 @@ cudaError_t sort_pairs_u64(void* tmp, unsigned long long* k0, unsigned long long
                            uint64_t n, int end_bit, cudaStream_t st, bool* in_second);
 size_t scan_temp_bytes(uint64_t n);
 cudaError_t inclusive_scan_u32(void* tmp, const uint32_t* in, uint32_t* out, uint64_t n, cudaStream_t st);
+cudaError_t exclusive_scan_u32(void* tmp, const uint32_t* in, uint32_t* out, uint64_t n, cudaStream_t st);  // out may be in
 
 // ------------------------------------------------------------------ prune.cu
 cudaError_t prune_launch(const sssp_graph* g, int mode, uint8_t* keep, uint32_t* witness, cudaStream_t st);

@@ -249,6 +249,10 @@ cudaError_t inclusive_scan_u32(void* tmp, const uint32_t* in, uint32_t* out, uin
     return scan_u32(static_cast<uint32_t*>(tmp), in, out, n, true, st);
 }
 
+cudaError_t exclusive_scan_u32(void* tmp, const uint32_t* in, uint32_t* out, uint64_t n, cudaStream_t st) {
+    return scan_u32(static_cast<uint32_t*>(tmp), in, out, n, false, st);
+}
+
 cudaError_t sort_pairs_u64(void* tmp, unsigned long long* k0, unsigned long long* k1, uint32_t* v0, uint32_t* v1,
                            uint64_t n, int end_bit, cudaStream_t st, bool* in_second) {
     *in_second = false;
