@@ -1,17 +1,20 @@
 // K1 CSR builder, K2 block partitioner, edge compaction.
 //
-// K1 turns a raw edge list into the canonical adjacency (Sec. III.A's Padj
-// for all partitions at once): keys (tail, head) are radix-sorted with their
-// input index (a stable sort, so equal keys keep input order), runs of equal
-// keys become one edge whose weight is the run's minimum (lowest input index
-// on ties, via a 64-bit atomicMin on (weight bits << 32 | index)), and
-// row_ptr is filled from the run boundaries.  Self-loops and bad ids sort to
-// the end behind a sentinel key and are dropped.  The radix sort and the
-// prefix sums are this library's own (sort.cu).
+// K1 turns a raw edge list into the canonical adjacency (Sec. III.A's Padj for all partitions at
+// once): keys (tail, head) are radix-sorted with their input index (a stable sort, so equal keys
+// keep input order; self-loops and bad ids make no pair), runs of equal keys become one edge whose
+// weight is the run's minimum (lowest input index on ties: the minimum of weight bits << 32 | index),
+// and row_ptr is filled from the run boundaries.  After the sort (sort.cu) the runs are counted per
+// tile, the counts scanned, and one kernel gathers the weights, reduces the runs in shared memory and
+// writes the edges; the runs that cross tiles (at most one a tile) are finished by a last small one.
+// R-MAT scale 22 (67 M edges): 2.6 -> 1.3 ms after the sort, where run minima were 64-bit atomics on
+// an array of their own and row numbers came from 64-bit divisions.  k_csr_emit (1.2 ms) is bound by
+// the random gather of the weights (8 a thread in flight; 4: the same, 16: 1.5 ms, fewer warps).
 #include <algorithm>
 
 #include "common.cuh"
 #include "internal.h"
+#include "rowwalk.cuh"
 
 namespace sssp {
 namespace {
@@ -22,13 +25,19 @@ __host__ __device__ inline uint32_t bits_for(unsigned long long x) {
     return b;
 }
 
+constexpr uint32_t EMIT_THREADS = 256, EMIT_WARPS = EMIT_THREADS / 32, EMIT_STEPS = 8;
+constexpr uint32_t EMIT_RUN = 32 * EMIT_STEPS, EMIT_TILE = EMIT_WARPS * EMIT_RUN;  // sorted pairs of a warp, a block
+constexpr unsigned long long NO_EDGE = ~0ull;
+
 struct CsrWs {
     WsHeader* hdr;
-    unsigned long long *keys_in, *keys_out;
-    uint32_t *vals_in, *vals_out;
-    uint32_t* runinc;             // [E_raw] inclusive run index
-    unsigned long long* runbest;  // [E_raw] (weight bits << 32 | input index)
-    void* tmp;                    // sort and scan temporaries
+    unsigned long long* keys[2];
+    uint32_t* vals[2];
+    uint32_t* totals;          // [tiles] runs that start in a tile, then before it
+    unsigned long long* lead;  // [tiles] minimum of a tile's pairs before its first run
+    void* sort;                // sort temporaries
+    void* scan;
+    uint64_t tiles;
     size_t total;
 };
 
@@ -42,79 +51,135 @@ CsrWs carve_csr(void* ws, uint32_t V, uint64_t n) {
         off += align_up(bytes, 256);
         return r;
     };
+    c.tiles = (n + EMIT_TILE - 1) / EMIT_TILE;
     c.hdr = reinterpret_cast<WsHeader*>(take(WS_HEADER_BYTES));
-    c.keys_in = reinterpret_cast<unsigned long long*>(take(8 * n));
-    c.keys_out = reinterpret_cast<unsigned long long*>(take(8 * n));
-    c.vals_in = reinterpret_cast<uint32_t*>(take(4 * n));
-    c.vals_out = reinterpret_cast<uint32_t*>(take(4 * n));
-    c.runinc = reinterpret_cast<uint32_t*>(take(4 * n));
-    c.runbest = reinterpret_cast<unsigned long long*>(take(8 * n));
-    c.tmp = take(std::max(sort_temp_bytes(n), scan_temp_bytes(n)));
+    for (int i = 0; i < 2; ++i) c.keys[i] = reinterpret_cast<unsigned long long*>(take(8 * n));
+    for (int i = 0; i < 2; ++i) c.vals[i] = reinterpret_cast<uint32_t*>(take(4 * n));
+    c.totals = reinterpret_cast<uint32_t*>(take(4 * (c.tiles + 1)));
+    c.lead = reinterpret_cast<unsigned long long*>(take(8 * (c.tiles + 1)));
+    c.sort = take(sort_temp_bytes(n));
+    c.scan = take(scan_temp_bytes(c.tiles + 1));
     c.total = off;
     return c;
 }
 
-template <class W>
-__global__ void k_make_keys(uint32_t V, uint64_t n, const uint32_t* __restrict__ src, const uint32_t* __restrict__ dst,
-                            const uint32_t* __restrict__ w, unsigned long long* keys, uint32_t* vals, WsHeader* hdr) {
-    const unsigned long long sentinel = (unsigned long long)V * V;
-    bool bad = false;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t s = src[i], d = dst[i];
-        unsigned long long k = sentinel;
-        if (s >= V || d >= V || !W::weight_ok(w[i]))
-            bad = true;
-        else if (s != d)
-            k = (unsigned long long)s * V + d;
-        keys[i] = k;
-        vals[i] = (uint32_t)i;
+// runs that start in each tile (totals[tiles] = 0 for the scan's last word)
+__global__ void __launch_bounds__(EMIT_THREADS) k_csr_runs(const unsigned long long* __restrict__ count,
+                                                           const unsigned long long* __restrict__ keys, uint32_t* totals) {
+    __shared__ uint32_t sum;
+    const unsigned long long n = *count, base = (unsigned long long)blockIdx.x * EMIT_TILE;
+    if (threadIdx.x == 0) sum = 0;
+    __syncthreads();
+    uint32_t mine = 0;
+    for (uint32_t i = threadIdx.x; i < EMIT_TILE; i += EMIT_THREADS) {
+        const unsigned long long at = base + i;
+        if (at < n && (at == 0 || keys[at - 1] != keys[at])) ++mine;
     }
-    if (bad) set_status(hdr, SSSP_EINVAL);
+    mine = __reduce_add_sync(0xFFFFFFFFu, mine);
+    if ((threadIdx.x & 31u) == 0 && mine) atomicAdd(&sum, mine);
+    __syncthreads();
+    if (threadIdx.x == 0) totals[blockIdx.x] = sum;
 }
 
-// run head flag: first element of a run of equal valid keys
-__global__ void k_heads(uint64_t n, unsigned long long sentinel, const unsigned long long* __restrict__ keys,
-                        uint32_t* heads) {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        const unsigned long long k = keys[i];
-        heads[i] = (k != sentinel && (i == 0 || keys[i - 1] != k)) ? 1u : 0u;
+// The edges of a tile's runs.  Each warp marks the run starts of its 256 pairs with ballots; a start
+// writes its head and the row_ptr entries up to its tail, and every pair lowers its run's (weight
+// bits << 32 | index) in shared memory, from which weights and indices go out in run order.
+// (before: runs before each tile, one word past the last tile the number of edges)
+__global__ void __launch_bounds__(EMIT_THREADS) k_csr_emit(uint32_t V, uint32_t bits,
+                                                           const unsigned long long* __restrict__ count,
+                                                           const unsigned long long* __restrict__ keys,
+                                                           const uint32_t* __restrict__ vals, const uint32_t* __restrict__ w,
+                                                           const uint32_t* __restrict__ before, unsigned long long* lead,
+                                                           uint32_t tiles, uint32_t* row_ptr, uint32_t* col,
+                                                           uint32_t* w_out, uint32_t* eid, uint32_t* E_out,
+                                                           const WsHeader* hdr) {
+    __shared__ unsigned long long best[EMIT_TILE + 1];  // [0]: pairs of a run that starts in an earlier tile
+    __shared__ uint32_t wsum[EMIT_WARPS];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, wid = tid >> 5;
+    const unsigned long long n = *count, tile0 = (unsigned long long)blockIdx.x * EMIT_TILE;
+    const bool failed = hdr->status == SSSP_EINTERNAL;  // the sort gave up: its pairs mean nothing
+    if (blockIdx.x == 0 && tid == 0) *E_out = failed ? 0u : before[tiles];
+    if (tile0 >= n || failed) {
+        if (tid == 0) lead[blockIdx.x] = NO_EDGE;
+        return;
+    }
+    const unsigned long long first = tile0 + wid * EMIT_RUN + lane;
+    unsigned long long k[EMIT_STEPS];
+    uint32_t v[EMIT_STEPS], starts[EMIT_STEPS];  // starts: ballots (uniform)
+    unsigned long long last = first - lane < n && first - lane ? keys[first - lane - 1] : NO_EDGE;  // key before the step
+    const unsigned long long last0 = last;
+    uint32_t mine = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < EMIT_STEPS; ++j) {
+        const unsigned long long at = first + 32u * j;
+        k[j] = at < n ? keys[at] : NO_EDGE;
+        v[j] = at < n ? vals[at] : 0u;
+    }
+    uint32_t x32[EMIT_STEPS];  // the weights, gathered together
+#pragma unroll
+    for (uint32_t j = 0; j < EMIT_STEPS; ++j) x32[j] = __ldg(&w[v[j]]);
+#pragma unroll
+    for (uint32_t j = 0; j < EMIT_STEPS; ++j) {
+        unsigned long long prev = __shfl_up_sync(0xFFFFFFFFu, k[j], 1);
+        if (lane == 0) prev = last;
+        last = __shfl_sync(0xFFFFFFFFu, k[j], 31);
+        starts[j] = __ballot_sync(0xFFFFFFFFu, k[j] != NO_EDGE && k[j] != prev);
+        mine += __popc(starts[j]);
+    }
+    if (lane == 0) wsum[wid] = mine;
+    for (uint32_t i = tid; i <= EMIT_TILE; i += EMIT_THREADS) best[i] = NO_EDGE;
+    __syncthreads();
+    uint32_t run = 0, all = 0;  // runs of the tile before this warp's
+    for (uint32_t i = 0; i < EMIT_WARPS; ++i) {
+        if (i < wid) run += wsum[i];
+        all += wsum[i];
+    }
+    const uint32_t base = before[blockIdx.x], R = before[tiles];
+    const unsigned long long hmask = (1ull << bits) - 1ull;
+    last = last0;
+#pragma unroll
+    for (uint32_t j = 0; j < EMIT_STEPS; ++j) {
+        unsigned long long prev = __shfl_up_sync(0xFFFFFFFFu, k[j], 1);
+        if (lane == 0) prev = last;
+        last = __shfl_sync(0xFFFFFFFFu, k[j], 31);
+        const uint32_t at = run + __popc(starts[j] & (0xFFFFFFFFu >> (31u - lane)));  // runs up to this pair
+        run += __popc(starts[j]);
+        if (k[j] != NO_EDGE) {
+            const unsigned long long x = (unsigned long long)x32[j] << 32 | v[j];
+            const bool alone = (starts[j] >> lane & 1u) && lane < 31u && (starts[j] >> (lane + 1u) & 1u);
+            if (alone)
+                best[at] = x;
+            else
+                atomicMin(&best[at], x);
+            if (starts[j] >> lane & 1u) {
+                const uint32_t r = base + at - 1u, s = (uint32_t)(k[j] >> bits);
+                col[r] = (uint32_t)(k[j] & hmask);
+                for (uint32_t u = prev == NO_EDGE ? 0u : (uint32_t)(prev >> bits) + 1u; u <= s; ++u) row_ptr[u] = r;
+            }
+            if (first + 32u * j + 1u == n)
+                for (uint32_t u = (uint32_t)(k[j] >> bits) + 1u; u <= V; ++u) row_ptr[u] = R;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) lead[blockIdx.x] = best[0];
+    for (uint32_t i = tid; i < all; i += EMIT_THREADS) {
+        const unsigned long long x = best[i + 1u];
+        w_out[base + i] = (uint32_t)(x >> 32);
+        if (eid) eid[base + i] = (uint32_t)x;
     }
 }
 
-__global__ void k_run_min(uint64_t n, unsigned long long sentinel, const unsigned long long* __restrict__ keys,
-                          const uint32_t* __restrict__ vals, const uint32_t* __restrict__ w,
-                          const uint32_t* __restrict__ runinc, unsigned long long* runbest) {
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        if (keys[i] == sentinel) continue;
-        const uint32_t id = vals[i];
-        atomicMin(&runbest[runinc[i] - 1u], ((unsigned long long)w[id] << 32) | id);
-    }
-}
-
-// one thread per run head: emit the edge and the row_ptr entries up to its tail
-__global__ void k_emit(uint32_t V, uint64_t n, unsigned long long sentinel, const unsigned long long* __restrict__ keys,
-                       const uint32_t* __restrict__ runinc, const unsigned long long* __restrict__ runbest,
-                       uint32_t* row_ptr, uint32_t* col, uint32_t* w_out, uint32_t* eid, uint32_t* E_out) {
-    const uint32_t R = n ? runinc[n - 1] : 0u;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-        const unsigned long long k = keys[i];
-        if (k == sentinel || (i > 0 && keys[i - 1] == k)) continue;
-        const uint32_t r = runinc[i] - 1u;
-        const uint32_t s = (uint32_t)(k / V), d = (uint32_t)(k % V);
-        const unsigned long long best = runbest[r];
-        col[r] = d;
-        w_out[r] = (uint32_t)(best >> 32);
-        if (eid) eid[r] = (uint32_t)best;
-        // rows (s_prev, s] start at r
-        const uint32_t s_prev = (r == 0) ? 0u : (uint32_t)(keys[i - 1] / V) + 1u;
-        for (uint32_t u = (r == 0 ? 0u : s_prev); u <= s; ++u) row_ptr[u] = r;
-        if (r + 1u == R)
-            for (uint32_t u = s + 1u; u <= V; ++u) row_ptr[u] = R;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *E_out = R;
-        if (R == 0)
-            for (uint32_t u = 0; u <= V; ++u) row_ptr[u] = 0;
+// a run that crosses into tile t and starts before it: the minimum of what the tiles from t on hold of it
+__global__ void k_csr_cross(uint32_t tiles, const uint32_t* __restrict__ before,
+                            const unsigned long long* __restrict__ lead, uint32_t* w_out, uint32_t* eid) {
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0 || t >= tiles || lead[t] == NO_EDGE || before[t] == before[t - 1]) return;
+    unsigned long long m = lead[t];
+    for (uint32_t x = t; before[x + 1] == before[x] && x + 1 < tiles && lead[x + 1] != NO_EDGE; ++x) m = min(m, lead[x + 1]);
+    const uint32_t r = before[t] - 1u;
+    if (m < ((unsigned long long)w_out[r] << 32 | (eid ? eid[r] : 0xFFFFFFFFu))) {
+        w_out[r] = (uint32_t)(m >> 32);
+        if (eid) eid[r] = (uint32_t)m;
     }
 }
 
@@ -294,21 +359,32 @@ __global__ void k_lay_slots(uint32_t V, const uint32_t* __restrict__ order, uint
     for (uint32_t n = blockIdx.x * blockDim.x + threadIdx.x; n < V; n += gridDim.x * blockDim.x) {
         const uint32_t v = order[n];
         ids[n] = v;
-        slots[v] = n;
+        if (v < V) slots[v] = n;  // (always, unless the sort gave up)
     }
 }
 
-// one warp per stored row: the edge list in the new numbering, in the old edge order
-__global__ void k_lay_coo(uint32_t V, const uint32_t* __restrict__ row_ptr, const uint32_t* __restrict__ col,
-                          const uint32_t* __restrict__ slots, uint32_t* src, uint32_t* dst) {
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-    for (uint64_t u = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < V; u += warps) {
-        const uint32_t beg = row_ptr[u], end = row_ptr[u + 1], su = slots[u];
-        for (uint32_t e = beg + lane; e < end; e += 32u) {
-            src[e] = su;
-            const uint32_t v = col[e];
-            dst[e] = v < V ? slots[v] : 0xFFFFFFFFu;  // a bad head stays bad: the CSR builder reports it
+// The edge list in the new numbering, in the old edge order: a warp walks a range of edges.  (R-MAT
+// scale 22: 2.4 ms with a warp per row, half of whose lanes had no edge, -> 0.31 ms, bound by the random
+// reads of slots.)
+constexpr uint32_t COO_RANGE = 1024;
+
+__global__ void __launch_bounds__(256) k_lay_coo(uint32_t V, uint32_t E, const uint32_t* __restrict__ row_ptr,
+                                                 const uint32_t* __restrict__ col, const uint32_t* __restrict__ slots,
+                                                 uint32_t* src, uint32_t* dst) {
+    __shared__ uint32_t rows[8][32], starts[8][32];
+    const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+    const unsigned long long first = ((unsigned long long)blockIdx.x * 8u + wid) * COO_RANGE;
+    if (first >= E) return;
+    const uint32_t e0 = (uint32_t)first, e1 = (uint32_t)min(first + COO_RANGE, (unsigned long long)E);
+    RowWalk walk{row_ptr, V, rows[wid], starts[wid]};
+    walk.seek(e0);
+    uint32_t v = e0 + lane < e1 ? __ldg(&col[e0 + lane]) : 0u;
+    for (uint32_t eb = e0; eb < e1 && eb >= e0; eb += 32u) {
+        const uint32_t e = eb + lane, u = walk.step(eb, e1), x = v;
+        if (e1 - eb > 32u + lane) v = __ldg(&col[e + 32u]);  // the next step's
+        if (e < e1) {
+            src[e] = __ldg(&slots[u]);
+            dst[e] = x < V ? __ldg(&slots[x]) : 0xFFFFFFFFu;  // a bad head stays bad: the CSR builder reports it
         }
     }
 }
@@ -332,33 +408,29 @@ size_t csr_workspace_bytes(uint32_t V, uint64_t E_raw) { return carve_csr(nullpt
 
 sssp_status csr_build(uint32_t V, uint64_t n, const uint32_t* src, const uint32_t* dst, const uint32_t* w, int wtype,
                       uint32_t* row_ptr, uint32_t* col, uint32_t* w_out, uint32_t* eid, uint32_t* E_out, void* ws,
-                      size_t ws_bytes, cudaStream_t st) {
+                      size_t ws_bytes, cudaStream_t st, bool clear) {
     CsrWs c = carve_csr(ws, V, n);
     if (ws_bytes < c.total) return SSSP_ENOMEM;
-    const unsigned long long sentinel = (unsigned long long)V * V;
-    const int end_bit = (int)bits_for(sentinel);
-    CK(cudaMemsetAsync(c.hdr, 0, WS_HEADER_BYTES, st));
+    const uint32_t bits = bits_for(V - 1u);
+    if (clear) CK(cudaMemsetAsync(c.hdr, 0, WS_HEADER_BYTES, st));
     CK(cudaMemsetAsync(row_ptr, 0, sizeof(uint32_t) * ((size_t)V + 1), st));
-    CK(cudaMemsetAsync(E_out, 0, sizeof(uint32_t), st));
-    if (n == 0) return SSSP_OK;
-    const unsigned g = grid_for(n);
-    if (wtype == SSSP_W_F32)
-        k_make_keys<WF32><<<g, 256, 0, st>>>(V, n, src, dst, w, c.keys_in, c.vals_in, c.hdr);
-    else
-        k_make_keys<WU32><<<g, 256, 0, st>>>(V, n, src, dst, w, c.keys_in, c.vals_in, c.hdr);
-    CK(cudaGetLastError());
+    if (n == 0) {
+        CK(cudaMemsetAsync(E_out, 0, sizeof(uint32_t), st));
+        return SSSP_OK;
+    }
     bool second = false;
-    CK(sort_pairs_u64(c.tmp, c.keys_in, c.keys_out, c.vals_in, c.vals_out, n, end_bit, st, &second));
-    const unsigned long long* sk = second ? c.keys_out : c.keys_in;  // sorted pairs
-    const uint32_t* sv = second ? c.vals_out : c.vals_in;
-    uint32_t* heads = second ? c.vals_in : c.vals_out;  // the other value buffer: head flags
-    k_heads<<<g, 256, 0, st>>>(n, sentinel, sk, heads);
+    CK(sort_edges(c.sort, V, bits, src, dst, w, wtype, n, c.keys[0], c.keys[1], c.vals[0], c.vals[1], c.hdr, st, &second));
+    const unsigned long long* keys = c.keys[second];
+    const uint32_t* vals = c.vals[second];
+    const unsigned long long* count = sort_count(c.sort);
+    const unsigned tiles = (unsigned)c.tiles;
+    k_csr_runs<<<tiles + 1, EMIT_THREADS, 0, st>>>(count, keys, c.totals);  // (the last block counts nothing)
     CK(cudaGetLastError());
-    CK(inclusive_scan_u32(c.tmp, heads, c.runinc, n, st));
-    CK(cudaMemsetAsync(c.runbest, 0xFF, 8 * n, st));
-    k_run_min<<<g, 256, 0, st>>>(n, sentinel, sk, sv, w, c.runinc, c.runbest);
+    CK(exclusive_scan_u32(c.scan, c.totals, c.totals, c.tiles + 1, st));
+    k_csr_emit<<<tiles, EMIT_THREADS, 0, st>>>(V, bits, count, keys, vals, w, c.totals, c.lead, tiles, row_ptr, col, w_out,
+                                               eid, E_out, c.hdr);
     CK(cudaGetLastError());
-    k_emit<<<g, 256, 0, st>>>(V, n, sentinel, sk, c.runinc, c.runbest, row_ptr, col, w_out, eid, E_out);
+    k_csr_cross<<<(tiles + 255) / 256, 256, 0, st>>>(tiles, c.totals, c.lead, w_out, eid);
     CK(cudaGetLastError());
     return SSSP_OK;
 }
@@ -437,17 +509,20 @@ sssp_status layout_build(const sssp_graph* g, uint32_t* row_ptr_out, uint32_t* c
     k_lay_keys<<<gv, 256, 0, st>>>(g->V, B, deg, kin, vin);
     CK(cudaGetLastError());
     bool second = false;
-    CK(sort_pairs_u64(p + L.off_tmp, kin, kout, vin, vout, g->V, 32 + (int)bits_for(g->partitions - 1u), st, &second));
+    CK(cudaMemsetAsync(p, 0, WS_HEADER_BYTES, st));
+    CK(sort_pairs_u64(p + L.off_tmp, kin, kout, vin, vout, g->V, 32 + (int)bits_for(g->partitions - 1u),
+                      reinterpret_cast<WsHeader*>(p), st, &second));
     k_lay_slots<<<gv, 256, 0, st>>>(g->V, second ? vout : vin, ids_out, slots_out);
     CK(cudaGetLastError());
     if (g->E) {
-        k_lay_coo<<<grid_for((uint64_t)g->V * 32), 256, 0, st>>>(g->V, g->row_ptr, g->col, slots_out, src, dst);
+        k_lay_coo<<<(unsigned)((g->E + 8ull * COO_RANGE - 1) / (8ull * COO_RANGE)), 256, 0, st>>>(
+            g->V, g->E, g->row_ptr, g->col, slots_out, src, dst);
         CK(cudaGetLastError());
     }
     // the renumbered edge list through the CSR builder: rows sorted by new head id, and
     // its input-index output maps each stored edge back to its index in g
     return csr_build(g->V, g->E, src, dst, static_cast<const uint32_t*>(g->w), g->wtype, row_ptr_out, col_out, w_out,
-                     emap_out, eout, ws, L.csr_bytes, st);
+                     emap_out, eout, ws, L.csr_bytes, st, false);  // (the status of the vertex sort stays)
 }
 
 namespace {

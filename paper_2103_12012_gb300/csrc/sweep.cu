@@ -37,6 +37,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "rowwalk.cuh"
 
 namespace sssp {
 namespace {
@@ -625,9 +626,7 @@ __global__ void __launch_bounds__(WT, 2) k_sweep(SweepLaunch L) {
 }
 
 // The results: distances in the caller's order, and predecessors by one pass over the edges.  A
-// warp takes a range of edges (its first row by a 32-way search of row_ptr) and holds the starts of
-// the rows with an edge among 32 rows at a time, one a lane, so that a lane finds its row as in
-// relax().  The (col, w) of the step after next and the heads' distances of the next one are in
+// warp walks a range of edges (rowwalk.cuh).  The (col, w) of the step after next and the heads' distances of the next one are in
 // flight while a step is compared; the tails' distances come through L1.
 template <class W, int G>
 __global__ void __launch_bounds__(256) k_sweep_out(SweepLaunch L, uint32_t per) {
@@ -648,30 +647,8 @@ __global__ void __launch_bounds__(256) k_sweep_out(SweepLaunch L, uint32_t per) 
     const unsigned long long first = (unsigned long long)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;
     if (first >= L.E) return;
     const uint32_t e0 = (uint32_t)first, e1 = (uint32_t)min(first + per, (unsigned long long)L.E);
-    uint32_t lo = 0, len = L.V;  // last row r with row_ptr[r] <= e0
-    while (len > 1u) {
-        const uint32_t step = (len + 31u) / 32u, i = lane * step;
-        const bool le = i < len && __ldg(&L.row_ptr[lo + i]) <= e0;
-        const uint32_t k = 31u - (uint32_t)__clz(__ballot_sync(0xFFFFFFFFu, le) | 1u);
-        lo += k * step;
-        len = min(step, len - k * step);
-    }
-    uint32_t* const row = rows[wid];
-    uint32_t r0 = lo, p, end, seen;  // the window: its first row, the start of the lane's row, its last edge, rows passed
-    auto window = [&]() {
-        const uint32_t r = r0 + lane;
-        const uint32_t a = __ldg(&L.row_ptr[min(r, L.V)]), b = __ldg(&L.row_ptr[min(r + 1u, L.V)]);
-        const bool has = b > a;
-        const uint32_t m = __ballot_sync(0xFFFFFFFFu, has), k = __popc(m & ((1u << lane) - 1u));
-        __syncwarp();
-        if (has) row[k] = r, starts[wid][k] = a;
-        __syncwarp();
-        p = lane < (uint32_t)__popc(m) ? starts[wid][lane] : 0xFFFFFFFFu;
-        end = __shfl_sync(0xFFFFFFFFu, b, 31);
-        seen = 0;
-    };
-    window();
-    seen = __popc(__ballot_sync(0xFFFFFFFFu, p < e0));
+    RowWalk walk{L.row_ptr, L.V, rows[wid], starts[wid]};
+    walk.seek(e0);
     uint32_t v = 0, w = 0;  // the step after next
     auto fetch = [&](uint32_t e) {
         v = NONE;
@@ -688,18 +665,7 @@ __global__ void __launch_bounds__(256) k_sweep_out(SweepLaunch L, uint32_t per) 
     heads();
     fetch(e0 + 32u + lane);
     for (uint32_t eb = e0; eb < e1; eb += 32u) {
-        // rows of the step's edges
-        uint32_t u = 0;
-        for (;;) {
-            const uint32_t at = __reduce_or_sync(0xFFFFFFFFu, p - eb < 32u ? 1u << (p - eb) : 0u);
-            // (a lane at or past the window's end finds its row in a later window, and overwrites this)
-            const uint32_t k = seen + __popc(at & (0xFFFFFFFFu >> (31u - lane)));
-            if (k) u = row[k - 1u];
-            seen += __popc(at);
-            if (end >= min(eb + 32u, e1)) break;
-            r0 += 32u;
-            window();
-        }
+        const uint32_t u = walk.step(eb, e1);
         uint32_t hv[G];
         const uint32_t head = x, wt = y;
 #pragma unroll

@@ -66,3 +66,76 @@ def test_compact_words_and_tiles(sssp, E, share, off):
     assert np.array_equal(u32(gp.row_ptr), rp.row_ptr)
     assert np.array_equal(u32(gp.col)[:gp.E], rp.col[:gp.E]) and np.array_equal(u32(gp.w)[:gp.E], rp.w[:gp.E])
     assert np.array_equal(u32(gp.eid)[:gp.E], np.flatnonzero(keep).astype(np.uint32))
+
+
+def check_build(sssp, V, src, dst, w, **kw):
+    ref = oracle.csr(V, src, dst, w)
+    g = sssp.build_csr(V, src, dst, w, **kw)
+    assert g.E == ref.E
+    assert np.array_equal(u32(g.row_ptr), ref.row_ptr)
+    E = g.E
+    assert np.array_equal(u32(g.col)[:E], ref.col[:E])
+    assert np.array_equal(u32(g.w)[:E], ref.w[:E].view(np.uint32))
+    assert np.array_equal(u32(g.eid)[:E], first_of_least(src, dst, w, V))
+    return g, ref
+
+
+def first_of_least(src, dst, w, V):
+    """Input index of every canonical edge: the lowest index among the least weights of its pair."""
+    idx = np.flatnonzero(src != dst)
+    order = idx[np.lexsort((idx, w[idx], dst[idx], src[idx]))]
+    key = src[order].astype(np.uint64) * V + dst[order]
+    return order[np.concatenate([[True], key[1:] != key[:-1]])].astype(np.uint32) if order.size else order.astype(np.uint32)
+
+
+@pytest.mark.parametrize("V,E", [(V, E) for V in (2, 3, 17, 512, 513, 70000) for E in (1, 2, 4095, 4096, 4097, 12289, 150001)]
+                         + [((1 << 26) + 5, 12289)])
+def test_build_tiles_and_key_widths(sssp, V, E):
+    """One to six digits, tiles of 4,096 pairs and their remainders, many repeated pairs (small V)."""
+    src, dst, w = edges(V % 1000 + E, V, E, hi=7)
+    src[-1:], dst[-1:] = V - 1, 0
+    check_build(sssp, V, src, dst, w)
+
+
+@pytest.mark.parametrize("f32", [False, True])
+def test_build_runs_across_tiles(sssp, f32):
+    """A run of equal pairs inside a warp, across warps, across one and several tiles, with its least
+    weight first, last and in the middle, and ties."""
+    rng = np.random.default_rng(3)
+    V = 40
+    for reps in (31, 700, 5000, 30000):
+        src = np.concatenate([np.full(reps, 3), rng.integers(0, V, 9000), np.full(reps, 20), [39, 39]]).astype(np.uint32)
+        dst = np.concatenate([np.full(reps, 5), rng.integers(0, V, 9000), np.full(reps, 7), [0, 0]]).astype(np.uint32)
+        for least in (0, reps // 2, reps - 1):
+            w = rng.integers(2, 6, src.size).astype(np.float32 if f32 else np.uint32)
+            w[least] = 1
+            w[reps + 9000 + least] = 1
+            perm = rng.permutation(src.size)
+            check_build(sssp, V, src[perm], dst[perm], w[perm])
+            check_build(sssp, V, src, dst, w)
+
+
+def test_build_without_an_edge_left_and_bad_edges_reported(sssp):
+    v = np.arange(9000, dtype=np.uint32)
+    g = sssp.build_csr(9000, v, v, np.ones(9000, np.uint32))  # loops only
+    assert g.E == 0 and not u32(g.row_ptr).any()
+    src, dst, w = edges(1, 100, 9000)
+    for a, k, x in ((src, 5000, 100), (dst, 8999, 0xFFFFFFFF), (w, 4096, 0)):
+        b = a.copy()
+        b[k] = x
+        with pytest.raises(sssp.SsspError):
+            sssp.build_csr(100, *(b if y is a else y for y in (src, dst, w)))
+
+
+@pytest.mark.parametrize("V,E,P", [(33, 4000, 2), (5000, 1023, 7), (5000, 1024, 7), (60001, 1025, 148), (60001, 900000, 1)])
+def test_layout_ranges(sssp, V, E, P):
+    """Ranges of 1,024 edges over empty rows, long rows and the last rows."""
+    rng = np.random.default_rng(V + E)
+    src, dst, w = edges(V + E, V, E)
+    src[: E // 3] = rng.integers(0, 3, E // 3)
+    ref = oracle.csr(V, src, dst, w)
+    h = sssp.layout(sssp.build_csr(V, src, dst, w, partitions=P))
+    ids, slots, lay = oracle.layout(ref, P)
+    assert np.array_equal(u32(h.ids), ids) and np.array_equal(u32(h.slots), slots)
+    assert np.array_equal(u32(h.row_ptr), lay.row_ptr)
+    assert np.array_equal(u32(h.col)[:h.E], lay.col[:h.E]) and np.array_equal(u32(h.w)[:h.E], lay.w[:h.E])
