@@ -1239,7 +1239,7 @@ __global__ void __launch_bounds__(SOLVE_MAX_THREADS, 4) k_solve(SolveLaunch L) {
                     if (lane == 0) ch = atomicAdd(&L.hdr->work_next, 1ull);
                     ch = __shfl_sync(0xFFFFFFFFu, ch, 0);
                     if (ch < L.prune.nchunks) {
-                        trishla_chunk<W>(L.prune, (uint32_t)ch, TRI_LIGHT);
+                        trishla_chunk<W>(L.prune, (uint32_t)ch);
                         if (lane == 0) atomicAdd(&sm.st[ST_PRUNE], 1ull);
                     } else if (lane == 0) {
                         sc.prune_done = 1u;

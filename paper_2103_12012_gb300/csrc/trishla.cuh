@@ -1,15 +1,15 @@
-// The Trishla test of Sec. III.B (Algorithm 1) on one chunk of consecutive edges, by one warp.
-// Shared by the stand-alone prune kernel (prune.cu) and by idle blocks of the persistent
-// solve (relax.cu), which prune while they wait for messages (the paper's use of idle time).
+// The Trishla test of Sec. III.B (Algorithm 1) as the idle blocks of the persistent solve run it
+// (relax.cu), which prune while they wait for messages (the paper's use of idle time), and what they
+// share with the prune kernel (prune.cu).
 //
-// The lanes read 32 edges (u, v_i) of the chunk at a time (their tails found inside the
-// chunk's row range) and a ballot picks the ones whose v_i may serve as a witness (local mode:
-// v_i in u's partition); for each of those the whole warp intersects the sorted adjacency
-// lists N(u) and N(v_i) -- walking the shorter and binary-searching the longer -- and for
-// every common head v_j tests  w(u, v_j) > w(u, v_i) + w(v_i, v_j).  A hit clears
-// keep[(u, v_j)] and lowers witness[(u, v_j)] to v_i with atomicMin, so the recorded witness
-// is the smallest one whatever the schedule.  All reads are of the unpruned graph (a
-// snapshot), so the result does not depend on the order in which chunks run.
+// A warp takes a chunk of consecutive edges: the lanes read 32 edges (u, v_i) at a time (their tails
+// found inside the chunk's row range) and a ballot picks the ones whose v_i may serve as a witness
+// (local mode: v_i in u's partition); for each of those the whole warp intersects the sorted adjacency
+// lists N(u) and N(v_i) -- walking the shorter and binary-searching the longer -- and for every common
+// head v_j tests  w(u, v_j) > w(u, v_i) + w(v_i, v_j).  A hit clears keep[(u, v_j)] and lowers
+// witness[(u, v_j)] to v_i with atomicMin, so the recorded witness is the smallest one whatever the
+// schedule.  All reads are of the unpruned graph (a snapshot), so the result does not depend on the
+// order in which chunks run.
 #pragma once
 
 #include "common.cuh"
@@ -64,16 +64,13 @@ struct TrishlaJob {
     uint32_t* witness;  // may be NULL
 };
 
-// Which candidate pairs (u, v_i) a call tests: all, only the light ones (both adjacency lists
-// at most TRISHLA_LIGHT long: a few dependent loads, so a solve block that runs them between
-// its rounds stays responsive), or only the heavy ones (the rest).  Tests are idempotent, so a
-// pair may be tested once or twice; splitting a chunk's pairs into light and heavy covers each.
-enum : int { TRI_ALL = 0, TRI_LIGHT = 1, TRI_HEAVY = 2 };
+// Light pairs have adjacency lists of at most this length: a few dependent loads, so a solve block
+// that runs them between its rounds stays responsive.  The prune kernel tests the others afterwards.
 constexpr uint32_t TRISHLA_LIGHT = 64;
 
-// Chunk `ch` (< J.nchunks) of the job, by the calling warp (all 32 lanes).
+// The light pairs of chunk `ch` (< J.nchunks) of the job, by the calling warp (all 32 lanes).
 template <class W>
-__device__ __noinline__ void trishla_chunk(const TrishlaJob& J, uint32_t ch, int which = TRI_ALL) {
+__device__ __noinline__ void trishla_chunk(const TrishlaJob& J, uint32_t ch) {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t e0 = ch * J.chunk, e1 = min(e0 + J.chunk, J.E);
     const uint32_t r0 = tri_row_of(J.row_ptr, 0u, J.V, e0);
@@ -93,7 +90,7 @@ __device__ __noinline__ void trishla_chunk(const TrishlaJob& J, uint32_t ch, int
             const uint32_t w_uvi = __ldg(&J.w[base + f]);
             const uint32_t a0 = __ldg(&J.row_ptr[uu]), a1 = __ldg(&J.row_ptr[uu + 1]);
             const uint32_t b0 = __ldg(&J.row_ptr[v]), b1 = __ldg(&J.row_ptr[v + 1]);
-            if (which != TRI_ALL && ((max(a1 - a0, b1 - b0) <= TRISHLA_LIGHT) != (which == TRI_LIGHT))) continue;
+            if (max(a1 - a0, b1 - b0) > TRISHLA_LIGHT) continue;
             if (a1 - a0 <= b1 - b0) {
                 // walk N(u), search N(v_i)
                 for (uint32_t j = a0 + lane; j < a1; j += 32u) {

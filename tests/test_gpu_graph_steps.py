@@ -1,6 +1,6 @@
 """The one-time graph steps at the sizes where their kernels change path: partition counts up to a
 vertex each (ranges that cross many partitions, empty ones among them), compaction around its mask
-words and tiles and with an unaligned keep mask, all against the CPU oracle (integers: equal)."""
+words and tiles and with an unaligned keep mask, the prune around its blocks and shares, all against the CPU oracle (integers: equal)."""
 import numpy as np
 import pytest
 
@@ -139,3 +139,33 @@ def test_layout_ranges(sssp, V, E, P):
     assert np.array_equal(u32(h.ids), ids) and np.array_equal(u32(h.slots), slots)
     assert np.array_equal(u32(h.row_ptr), lay.row_ptr)
     assert np.array_equal(u32(h.col)[:h.E], lay.col[:h.E]) and np.array_equal(u32(h.w)[:h.E], lay.w[:h.E])
+
+
+def distinct_edges(rng, V, E, hubs=0):
+    """Exactly E distinct edges without loops, the first `hubs` rows full."""
+    key = np.concatenate([np.arange(hubs * V), rng.permutation(V * V) if V * V < 10 * E else rng.integers(0, V * V, 2 * E + 100)])
+    key = key[key // V != key % V]
+    _, at = np.unique(key, return_index=True)
+    key = key[np.sort(at)][:E]
+    assert key.size == E
+    return (key // V).astype(np.uint32), (key % V).astype(np.uint32)
+
+
+@pytest.mark.parametrize("V,E,hubs,P", [(40, 1, 0, 1), (40, 31, 0, 8), (40, 33, 0, 1), (300, 255, 0, 1), (300, 257, 0, 8),
+                                        (300, 1025, 3, 1), (600, 8191, 9, 8), (600, 8193, 9, 9), (600, 8193, 9, 1),
+                                        (1500, 60000, 35, 8), (1500, 60000, 35, 1), (20000, 2553599, 3, 64)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_prune_blocks_and_shares(sssp, V, E, hubs, P, mode):
+    """Edge counts around a block's rounds (one round of 256 edges, of 1,024 edges and, from 2.5 M edges on,
+    several), with rows of every length up to V - 1: pairs of many shares, and many pairs in a share."""
+    if mode == 1 and E > 100000:
+        V, E, hubs = 5000, 120000, 5
+    rng = np.random.default_rng(E + P)
+    src, dst = distinct_edges(rng, V, E, hubs)
+    w = rng.integers(1, 60, E).astype(np.uint32)
+    ref = oracle.csr(V, src, dst, w)
+    g = sssp.build_csr(V, src, dst, w, partitions=P)
+    keep, wit = sssp.prune(g, mode)
+    rk, rw = oracle.trishla(ref, P, mode)
+    assert np.array_equal(keep.cpu().numpy(), rk)
+    assert np.array_equal(u32(wit), rw)
