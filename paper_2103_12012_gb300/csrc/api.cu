@@ -105,7 +105,8 @@ bool sweep_graph(const sssp_graph* g, uint32_t S) {
 // entries[2] of the sweep | dirty[S*Q] | nfsplit[S*Q].  The sweep keeps dist[items][G] at the start
 // of packed.  For S > 1 its marks are in the rest of packed and its lists in the caller's dist array
 // (written only at the end); for S = 1 its marks are the bitmap, one list is the rest of packed and
-// the other the caller's dist.
+// the other the caller's dist.  A warm start keeps rows of packed words in packed, and marks and lists
+// in the caller's dist (read at the start, written at the end).
 struct SolveWs {
     size_t off_ctl, off_packed, off_bitmap, off_ex, ex_bytes, off_dirty, off_nf, total;
     uint32_t words, B, Bq, Q;
@@ -150,6 +151,16 @@ SolveWs solve_layout(const sssp_graph* g, uint32_t S, uint32_t split, bool sweep
 bool sweep_wins(const sssp_graph* g, uint32_t S, const SolveWs& L, bool delta_given) {
     if (S >= 5) return g->V >= 2048 || L.Bq >= 64;
     return L.Bq >= 64 && (!delta_given || g->ids || (uint64_t)S * L.Q < 128);
+}
+
+// A warm start by the sweep: from about ten thousand tails on its passes over the vertices and its grid
+// barriers cost less than the persistent solve's chains of rounds (R-MAT, 16 edges a vertex; vertices,
+// sources, tails: persistent / sweep us): 131,072, 1, 20,971: 267 / 203; 524,288, 4, 8,388: 288 / 278;
+// 1 M, 4, 16,777: 345 / 263; 2 M, 8, 335,544: 2,320 / 795; but 32,768, 4, 524: 151 / 180; 262,144, 4,
+// 4,194: 211 / 225.  An odd number of sources has rows of one and wants more: 3 sources, 524,288, 8,388:
+// 251 / 274; 1 M, 16,777: 328 / 311.  Rows of four are loaded with 32-byte accesses.
+bool warm_sweep_wins(uint32_t S, uint32_t n_tails, const void* packed) {
+    return n_tails >= (S % 2u && S > 1u ? 16384u : 8192u) && (S % 4u || (reinterpret_cast<uintptr_t>(packed) & 31u) == 0);
 }
 
 int sm_count() {
@@ -250,11 +261,12 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
     const size_t smem = relax_smem_bytes(r.tile, L.Q, r.msg_buffer != 0);
     if (smem > 200 * 1024) return SSSP_EINVAL;
     const bool prune = prune_mode >= 0;
-    // The sweep takes cold solves in the default policy (the others ask for a schedule of the persistent
-    // solve).  The persistent solve alone keeps its own, tighter layout: behind a gap, 276 doorbells made a
-    // solve of 0.71 ms (random graph, 89,656 vertices, 4 sources, 69 partitions) one of 0.84.
-    const bool sweep = L.sweep && !warm && !prune && r.policy == SSSP_POLICY_RELATIVE && r.msg_buffer == 0 &&
-                       !(r.flags & SSSP_FLAG_TEST_HOLD_PENDING) && sweep_wins(g, S, L, r.delta_given);
+    // The sweep takes solves in the default policy (the others ask for a schedule of the persistent solve).
+    // The persistent solve alone keeps its own, tighter layout: behind a gap, 276 doorbells made a solve of
+    // 0.71 ms (random graph, 89,656 vertices, 4 sources, 69 partitions) one of 0.84.
+    const bool sweep =
+        L.sweep && !prune && r.policy == SSSP_POLICY_RELATIVE && r.msg_buffer == 0 && !(r.flags & SSSP_FLAG_TEST_HOLD_PENDING) &&
+        (warm ? warm_sweep_wins(S, n_tails, static_cast<char*>(ws) + L.off_packed) : sweep_wins(g, S, L, r.delta_given));
     if (!sweep) L = solve_layout(g, S, r.split, false);
     int per_sm = 0;
     const uint32_t hubs = g->ids ? std::min(r.hub_count, L.B) : 0u;  // layout graphs only
@@ -305,7 +317,7 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
     l.n_tails = n_tails;
     l.prune_on = prune ? 1u : 0u;
     if (prune) l.prune = trishla_job(g, prune_mode, keep, witness);
-    SweepLaunch x{};
+    WarmLaunch x{};
     if (sweep) {
         x.row_ptr = l.row_ptr;
         x.col = l.col;
@@ -317,6 +329,7 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
         x.slots = g->slots;
         x.S = S;
         x.G = S == 1 ? 1u : S == 2 ? 2u : S <= 4 ? 4u : 8u;
+        if (warm) x.G = S % 4u == 0 ? 4u : S % 2u == 0 ? 2u : 1u;  // (no padding: the rows take packed's place)
         x.groups = (S + x.G - 1u) / x.G;
         x.items = x.groups * g->V;
         x.sources = sources;
@@ -329,6 +342,17 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
         x.mark = S == 1 ? l.bitmap : rest;
         x.list[0] = l.dist;
         x.list[1] = S == 1 ? rest : l.dist + x.items;
+        if (warm) {
+            x.tails = tails;
+            x.n_tails = n_tails;
+            x.dist = reinterpret_cast<uint32_t*>(l.packed);
+            x.mark = l.dist;
+            x.list[0] = l.dist + (x.items + 31u) / 32u;
+            const uint32_t cap = (uint32_t)std::min<size_t>((l.dist + (size_t)S * g->V - x.list[0]) / 2, x.items);
+            x.list[1] = x.list[0] + cap;
+            x.capM = cap / 4u;
+            x.capA = cap - x.capM;
+        }
         x.ex[0] = reinterpret_cast<unsigned long long*>(base + L.off_ex);
         x.ex[1] = reinterpret_cast<unsigned long long*>(base + L.off_ex + L.ex_bytes);
         x.dirty = l.dirty;
@@ -338,7 +362,7 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
         x.pred = pred;
         x.inf = g->wtype == SSSP_W_F32 ? F32_INF_BITS : INF32;
         x.timeout_ns = r.timeout_ns;
-        if (sweep_max_blocks_per_sm(g->wtype, x.G, &per_sm) != cudaSuccess) return SSSP_ECUDA;
+        if (sweep_max_blocks_per_sm(g->wtype, x.G, warm, &per_sm) != cudaSuccess) return SSSP_ECUDA;
         if (r.bps) per_sm = std::min<int>(per_sm, (int)r.bps);
         x.grid = (uint32_t)std::min<uint64_t>((uint64_t)std::max(per_sm, 0) * sm_count(),
                                               std::max<uint64_t>(1, (uint64_t)g->E * x.groups / 1024));

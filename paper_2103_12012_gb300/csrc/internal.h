@@ -19,7 +19,7 @@ struct SweepIter {            // counters of one iteration
     uint32_t nA, nM;          // items in list A (from the front) and list M (from the back)
     unsigned long long ex;    // hubs << 32 | their segments
     unsigned long long work;  // relaxations of the iteration before
-    uint32_t pad[26];
+    uint32_t stop, pad[25];   // (warm) a list was full
 };
 struct SweepCtl {  // zero before the launch
     uint32_t bar, pad[31];
@@ -52,9 +52,21 @@ struct SweepLaunch {
     uint32_t grid;
 };
 
-cudaError_t sweep_max_blocks_per_sm(int wtype, uint32_t G, int* out);
+// A warm start: out and pred hold a previous result, which is brought up to date.  The rows are of packed
+// words (distance << 32 | predecessor), four at most; the lists and marks are in out meanwhile.
+struct WarmLaunch : SweepLaunch {
+    const uint32_t* tails;  // [n_tails] caller's ids
+    uint32_t n_tails;
+    uint32_t capA, capM;    // items that a list holds of either kind
+};
+
+cudaError_t sweep_max_blocks_per_sm(int wtype, uint32_t G, bool warm, int* out);
 cudaError_t launch_sweep(const SweepLaunch& L, int sms, cudaStream_t st);
 cudaError_t launch_sweep_out(const SweepLaunch& L, int sms, cudaStream_t st);
+cudaError_t launch_warm_sweep(const WarmLaunch& L, int sms, cudaStream_t st);
+cudaError_t launch_warm_out(const WarmLaunch& L, int sms, cudaStream_t st);
+cudaError_t launch_warm_requeue(const WarmLaunch& L, uint32_t* bitmap, uint32_t words, uint32_t B, uint32_t Bq,
+                                uint32_t split, uint32_t Q, int sms, cudaStream_t st);
 cudaError_t launch_sweep_requeue(const SweepLaunch& L, uint32_t* bitmap, uint32_t words, uint32_t B, uint32_t Bq,
                                  uint32_t split, uint32_t Q, int sms, cudaStream_t st);
 
@@ -113,7 +125,7 @@ cudaError_t relax_max_blocks_per_sm(int wtype, uint32_t threads, uint32_t tile, 
                                     bool prune = false, bool msgs = false, bool hubs = false);
 // with `sweep`: the sweep first (sweep.cu), then the persistent solve on what it leaves (no vertex is
 // queued when it finished: every block sees a zero count at its first look and ends)
-cudaError_t launch_solve(const SolveLaunch& L, const SweepLaunch* sweep, cudaStream_t st);
+cudaError_t launch_solve(const SolveLaunch& L, const SweepLaunch* sweep, cudaStream_t st);  // (L.warm: a WarmLaunch)
 
 // One problem of a batch, in the order blocks take them (largest first).
 struct BatchProblem {

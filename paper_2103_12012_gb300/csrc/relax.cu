@@ -1413,11 +1413,18 @@ cudaError_t launch_solve(const SolveLaunch& L, const SweepLaunch* sweep, cudaStr
         const unsigned blocks = (unsigned)std::min<size_t>(std::max<size_t>(want, 1), (size_t)sms * 8);
         if (sweep) {
             if (L.ev_begin && (e = cudaEventRecord(L.ev_begin, st)) != cudaSuccess) return e;
-            if ((e = launch_sweep(*sweep, sms, st)) != cudaSuccess) return e;
-            if ((e = launch_sweep_out(*sweep, sms, st)) != cudaSuccess) return e;
-            // what a sweep that gave up leaves: its queued vertices, and its results as packed words
-            if ((e = launch_sweep_requeue(*sweep, L.bitmap, L.words, L.B, L.Bq, L.split, L.Q, sms, st)) != cudaSuccess)
-                return e;
+            // (then, what a sweep that gave up leaves: its queued vertices, and its results as packed words)
+            if (L.warm) {
+                const WarmLaunch& w = static_cast<const WarmLaunch&>(*sweep);
+                if ((e = launch_warm_sweep(w, sms, st)) != cudaSuccess) return e;
+                if ((e = launch_warm_requeue(w, L.bitmap, L.words, L.B, L.Bq, L.split, L.Q, sms, st)) != cudaSuccess) return e;
+                if ((e = launch_warm_out(w, sms, st)) != cudaSuccess) return e;
+            } else {
+                if ((e = launch_sweep(*sweep, sms, st)) != cudaSuccess) return e;
+                if ((e = launch_sweep_out(*sweep, sms, st)) != cudaSuccess) return e;
+                if ((e = launch_sweep_requeue(*sweep, L.bitmap, L.words, L.B, L.Bq, L.split, L.Q, sms, st)) != cudaSuccess)
+                    return e;
+            }
             if (L.wtype == SSSP_W_F32)
                 k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, done);
             else

@@ -30,10 +30,15 @@
 // k_sweep (3.0 ms of the 4.1) is bound by the latency of its L2 accesses and by issue slots (44% busy
 // at the 32 warps per SM that 64 registers allow; with 48 warps at 40 registers it spills and is not
 // faster), k_sweep_out (1.0 ms) by random 32-byte sectors, 61 G a second.
+// A warm start (sssp_update) with many tails goes the same way, from the tails' rows: there the rows are of
+// packed words (up to four), so that predecessors come along and no pass over all edges is needed, and
+// the lists and marks take the caller's dist.  R-MAT, 1 M vertices, 15 M edges, 4 sources, 15,000 tails: 0.39 ->
+// 0.27 ms; k_sweep has 0.19 of it, most in the first iteration (the tails' rows are a third of the edges).
 // A graph that is not of that kind (tiny frontiers, many iterations, or many more relaxations than
 // edges) is handed over: marks become inbox bits, distances packed words, and k_solve goes on.
 // Waits: the grid barrier is bounded by the idle limit, the kernel by LIMIT_FACTOR times it.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -52,6 +57,7 @@ constexpr uint64_t LIMIT_FACTOR = 3;
 // Hand-over, looked at every HAND_EVERY iterations: fewer than HAND_EDGES relaxations an iteration,
 // a pace that predicts more than HAND_ITERS iterations, or more than HAND_INFL relaxations per edge
 // and source (random and power-law graphs: 2 to 10).
+constexpr uint32_t WARM_ITERS = 32;  // a warm start is handed over
 constexpr uint32_t HAND_EVERY = 32, HAND_EDGES = 2048, HAND_ITERS = 1024, HAND_INFL = 24;
 
 template <class W>
@@ -131,6 +137,15 @@ __device__ __forceinline__ void load_final(const uint32_t* p, uint32_t (&r)[G]) 
     }
 }
 
+// G packed words of an item: predecessors, distances
+template <int G>
+__device__ __forceinline__ void load_keys(const uint32_t* dist, uint32_t item, uint32_t (&lo)[G], uint32_t (&hi)[G]) {
+    uint32_t x[2 * G];
+    load_row<2 * G>(dist + (size_t)item * (2 * G), x);
+#pragma unroll
+    for (int s = 0; s < G; ++s) lo[s] = x[2 * s], hi[s] = x[2 * s + 1];
+}
+
 template <int G>
 __device__ __forceinline__ void shared_row(const uint32_t* p, uint32_t (&r)[G]) {
     if constexpr (G >= 4) {
@@ -170,9 +185,10 @@ __device__ bool grid_barrier(const SweepLaunch& L, BlockMem& bm, uint32_t& n, ui
     return bm.ok != 0;
 }
 
-template <class W, int G>
+template <class W, int G, class Launch>
 struct Worker {
-    const SweepLaunch& L;
+    static constexpr bool WARM = std::is_same<Launch, WarmLaunch>::value;
+    const Launch& L;
     WarpMem& wm;
     uint32_t* du;  // [32][G] distances of the rows held
     BlockMem& bm;
@@ -186,7 +202,14 @@ struct Worker {
     __device__ __forceinline__ uint32_t vertex(uint32_t item) const { return L.groups == 1u ? item : item % L.V; }
 
     __device__ __forceinline__ void put(uint32_t at, uint32_t item, bool back) {
-        list[back ? L.items - 1u - at : at] = item;
+        if constexpr (WARM) {
+            if (at < (back ? L.capM : L.capA))
+                list[back ? L.capA + L.capM - 1u - at : at] = item;
+            else
+                it->stop = 1u;  // (its mark stays)
+        } else {
+            list[back ? L.items - 1u - at : at] = item;
+        }
     }
 
     __device__ __forceinline__ void flush_full(uint32_t* buf, uint32_t& n, uint32_t* cnt, bool back) {
@@ -254,6 +277,17 @@ struct Worker {
         nA = nM = 0;
     }
 
+    __device__ __forceinline__ void load_dist(uint32_t item, uint32_t (&r)[G]) const {
+        if constexpr (WARM) {
+            uint32_t lo[G];
+            load_keys<G>(L.dist, item, lo, r);
+#pragma unroll
+            for (int s = 0; s < G; ++s) r[s] = min(r[s], Dist<W>::INF);
+        } else {
+            load_row<G>(L.dist + (size_t)item * G, r);
+        }
+    }
+
     // Takes the item of each lane with `ok`: its mark is cleared before its distances are read, so a
     // distance lowered after the read marks it again.
     __device__ __forceinline__ void take(bool ok, uint32_t item, uint32_t (&r)[G]) {
@@ -262,7 +296,7 @@ struct Worker {
         if (ok) {
             atomicAnd(&L.mark[item >> 5], ~(1u << (item & 31u)));
             fence_gpu();
-            load_row<G>(L.dist + (size_t)item * G, r);
+            load_dist(item, r);
         }
     }
 
@@ -281,7 +315,9 @@ struct Worker {
 #pragma unroll
             for (int s = 0; s < G; ++s) du[at * G + s] = r[s];
         }
-        wm.row[at] = make_uint4(off, L.groups == 1u ? 0u : item - item % L.V, mx, 0u);
+        uint32_t lab = 0;
+        if constexpr (WARM) lab = L.ids ? __ldg(&L.ids[vertex(item)]) : vertex(item);
+        wm.row[at] = make_uint4(off, L.groups == 1u ? 0u : item - item % L.V, mx, lab);
         return fin;
     }
 
@@ -328,9 +364,10 @@ struct Worker {
     // A pipeline of three: the (col, w) of the steps after next, the distances of the next ones and
     // the atomics of these are in flight together (EB steps each: eight distances a lane).
     __device__ __forceinline__ void relax(uint32_t total, uint32_t p) {
-        constexpr int EB = G >= 8 ? 1 : G == 4 ? 2 : 4;
+        constexpr int EB = G >= 8 || (WARM && G >= 4) ? 1 : G == 4 || (WARM && G == 2) ? 2 : 4;
         uint32_t v[EB], w[EB], a[EB];              // steps after next: head, weight, row
         uint32_t x[EB], y[EB], b[EB], d[EB][G];    // next steps: item, weight, row, its distances
+        uint32_t pr[EB][WARM ? G : 1];             // (warm) and predecessors
         uint32_t seen = 0;                         // rows that start before the step
         auto fetch = [&](uint32_t k0) {            // k0: first edge of the steps
 #pragma unroll
@@ -363,7 +400,10 @@ struct Worker {
                     uint32_t z;
                     if (!W::add(rw.z, y[j], z)) bad |= 2u;
                     x[j] += rw.y;
-                    load_row<G>(L.dist + (size_t)x[j] * G, d[j]);
+                    if constexpr (WARM)
+                        load_keys<G>(L.dist, x[j], pr[j], d[j]);
+                    else
+                        load_row<G>(L.dist + (size_t)x[j] * G, d[j]);
                 }
             }
         };
@@ -372,7 +412,7 @@ struct Worker {
         fetch(32u * EB);
         for (uint32_t k0 = 0; k0 < total; k0 += 32u * EB) {
             // these steps: candidates c where they beat the distances read, else INF
-            uint32_t c[EB][G], it_[EB], imp[EB], any = 0;
+            uint32_t c[EB][G], it_[EB], imp[EB], lab[EB], any = 0;
 #pragma unroll
             for (int j = 0; j < EB; ++j) {
                 it_[j] = x[j];
@@ -380,10 +420,17 @@ struct Worker {
                 if (x[j] != NONE) {
                     uint32_t dj[G];
                     shared_row<G>(du + b[j] * G, dj);
+                    if constexpr (WARM) lab[j] = wm.row[b[j]].w;
 #pragma unroll
                     for (int s = 0; s < G; ++s) {
                         c[j][s] = Dist<W>::add(dj[s], y[j]);
-                        if (c[j][s] < d[j][s]) imp[j] |= 1u << s;
+                        if constexpr (WARM) {
+                            if (c[j][s] < Dist<W>::INF &&
+                                (c[j][s] < d[j][s] || (c[j][s] == d[j][s] && lab[j] < pr[j][s])))
+                                imp[j] |= 1u << s;
+                        } else if (c[j][s] < d[j][s]) {
+                            imp[j] |= 1u << s;
+                        }
                     }
                 }
                 any |= imp[j];
@@ -395,12 +442,18 @@ struct Worker {
 #pragma unroll
             for (int j = 0; j < EB; ++j) {
                 low[j] = 0;
-                uint32_t* const row = L.dist + (size_t)it_[j] * G;
+                uint32_t* const row = L.dist + (size_t)it_[j] * (WARM ? 2 * G : G);
                 uint32_t old[G];
 #pragma unroll
                 for (int s = 0; s < G; ++s) {
                     old[s] = 0;
-                    if (imp[j] & (1u << s)) old[s] = atomicMin(row + s, c[j][s]);
+                    if constexpr (WARM) {
+                        if (imp[j] & (1u << s))
+                            old[s] = (uint32_t)(atomicMin(reinterpret_cast<unsigned long long*>(row) + s,
+                                                          (unsigned long long)c[j][s] << 32 | lab[j]) >> 32);
+                    } else {
+                        if (imp[j] & (1u << s)) old[s] = atomicMin(row + s, c[j][s]);
+                    }
                 }
 #pragma unroll
                 for (int s = 0; s < G; ++s)
@@ -427,6 +480,8 @@ struct Worker {
     __device__ __forceinline__ void work(const uint32_t* in, const unsigned long long* ex, uint32_t cA, uint32_t cM,
                                          uint32_t cX, uint32_t segs) {
         const uint32_t TW = gridDim.x * NW;
+        uint32_t last = L.items - 1u;  // of a list
+        if constexpr (WARM) last = L.capA + L.capM - 1u;
         // segments and rows of a unit: fewer when there are few, so that all warps get some
         const uint32_t rX = min(max(segs / (2u * TW), 1u), 8u), rM = min(max(cM / TW, 1u), 8u);
         const uint32_t rA = cA >= TW * 32u ? 32u : cA >= TW * 16u ? 16u : 8u;
@@ -456,7 +511,7 @@ struct Worker {
                     const bool ok = lane < (m ? rM : rA) && c + lane < (m ? cM : cA);
                     uint32_t item = 0, beg = 0, deg = 0, r[G];
                     if (ok) {
-                        item = __ldcg(&in[m ? L.items - 1u - (c + lane) : c + lane]);
+                        item = __ldcg(&in[m ? last - (c + lane) : c + lane]);
                         const uint32_t x = vertex(item);
                         beg = __ldg(&L.row_ptr[x]);
                         deg = __ldg(&L.row_ptr[x + 1]) - beg;
@@ -485,7 +540,7 @@ struct Worker {
                 total = min(left, n * SEG);
                 if (lane == 0) {
                     uint32_t r[G];
-                    load_row<G>(L.dist + (size_t)item * G, r);
+                    load_dist(item, r);
                     const uint32_t fin = hold(0, r, item, beg);
                     wm.edges += (unsigned long long)fin * total;
                     if (s0 == 0) wm.vert += fin;
@@ -515,8 +570,9 @@ __global__ void k_sweep_init(SweepLaunch L, uint32_t inf) {
         for (size_t i = i0; i < (size_t)L.S * L.V; i += stride) L.pred[i] = NONE;
 }
 
-template <class W, int G>
-__global__ void __launch_bounds__(WT, 2) k_sweep(SweepLaunch L) {
+template <class W, int G, class Launch>
+__global__ void __launch_bounds__(WT, 2) k_sweep(Launch L) {
+    constexpr bool WARM = std::is_same<Launch, WarmLaunch>::value;
     extern __shared__ __align__(16) uint32_t dsm[];  // [NW][32][G] rows
     __shared__ BlockMem bm;
     __shared__ WarpMem wmem[NW];
@@ -529,7 +585,31 @@ __global__ void __launch_bounds__(WT, 2) k_sweep(SweepLaunch L) {
         wm.edges = 0ull;
         wm.act = wm.vert = 0u;
     }
-    if (blockIdx.x == 0) {  // seeds
+    if constexpr (WARM) {  // the tails that a source has reached
+        __syncthreads();
+        Worker<W, G, Launch> wk{L, wm, dsm + wid * 32u * G, bm, lane, L.list[0], &L.ctl->it[0], L.ex[0], 0, 0, 0, 0, 0, 0};
+        for (unsigned long long i0 = (unsigned long long)blockIdx.x * WT + wid * 32u; i0 < L.n_tails;
+             i0 += (unsigned long long)gridDim.x * WT) {
+            uint32_t t = i0 + lane < L.n_tails ? __ldg(&L.tails[i0 + lane]) : NONE;
+            if (i0 + lane < L.n_tails && t >= L.V) set_status(L.hdr, SSSP_EINVAL);
+            const bool ok = i0 + lane < L.n_tails && t < L.V;
+            if (ok && L.slots) t = __ldg(&L.slots[t]);
+            const uint32_t deg = ok ? __ldg(&L.row_ptr[t + 1]) - __ldg(&L.row_ptr[t]) : 0u;
+            for (uint32_t g = 0; g < L.groups; ++g) {
+                const uint32_t item = g * L.V + t, bit = 1u << (item & 31u);
+                bool has = false;
+                if (ok) {
+                    uint32_t r[G];
+                    wk.load_dist(item, r);
+#pragma unroll
+                    for (int s = 0; s < G; ++s) has = has || r[s] < Dist<W>::INF;
+                }
+                if (has) has = !(atomicOr(&L.mark[item >> 5], bit) & bit);  // (a tail may be listed twice)
+                wk.push(has, item, deg);
+            }
+        }
+        wk.flush_block();
+    } else if (blockIdx.x == 0) {  // seeds
         for (uint32_t s = tid; s < L.S; s += WT) {
             uint32_t src = L.sources[s];
             if (src >= L.V) {
@@ -568,14 +648,17 @@ __global__ void __launch_bounds__(WT, 2) k_sweep(SweepLaunch L) {
             done = true;
             break;
         }
+        if (WARM && bm.c[6]) break;
         const uint32_t next = slot == 2u ? 0u : slot + 1u, after = next == 2u ? 0u : next + 1u;
         if (blockIdx.x == 0 && tid == 0) {  // its counters were last read before this barrier
             SweepIter& z = L.ctl->it[after];
             z.nA = z.nM = 0u;
+            if (WARM) z.stop = 0u;
             z.ex = z.work = 0ull;
         }
         ++iters;
-        if (iters % HAND_EVERY == 0u &&
+        if (WARM && iters == WARM_ITERS) break;
+        if (!WARM && iters % HAND_EVERY == 0u &&
             (work < (unsigned long long)iters * HAND_EDGES || all / (work + 1ull) * iters > HAND_ITERS ||
              work / HAND_INFL > all))
             break;  // the listed items keep their marks
@@ -588,7 +671,7 @@ __global__ void __launch_bounds__(WT, 2) k_sweep(SweepLaunch L) {
             }
             if (!grid_barrier(L, bm, nbar, t_begin)) break;
         }
-        Worker<W, G> wk{L, wm, dsm + wid * 32u * G, bm, lane, L.list[par ^ 1u], &L.ctl->it[next], L.ex[par ^ 1u], 0, 0, 0, 0, 0, 0};
+        Worker<W, G, Launch> wk{L, wm, dsm + wid * 32u * G, bm, lane, L.list[par ^ 1u], &L.ctl->it[next], L.ex[par ^ 1u], 0, 0, 0, 0, 0, 0};
         const unsigned long long before = wm.edges;
         wk.work(L.list[par], L.ex[par], cA, cM, cX, segs);
         wk.bad = __reduce_or_sync(0xFFFFFFFFu, wk.bad);
@@ -691,11 +774,59 @@ __global__ void __launch_bounds__(256) k_sweep_out(SweepLaunch L, uint32_t per) 
     }
 }
 
+// Warm start: the rows from the previous result.
+template <int G>
+__global__ void k_warm_rows(WarmLaunch L) {
+    const size_t stride = (size_t)gridDim.x * blockDim.x, i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    for (size_t i = i0; i < L.n_dirty; i += stride) L.dirty[i] = 0u, L.nfsplit[i] = 0u;
+    for (size_t c = i0; c < L.V; c += stride) {
+        const uint32_t at = L.slots ? __ldg(&L.slots[c]) : (uint32_t)c;
+        for (uint32_t g = 0; g < L.groups; ++g) {
+            uint32_t* const row = L.dist + ((size_t)g * L.V + at) * (2 * G);
+            uint32_t x[2 * G];
+#pragma unroll
+            for (int s = 0; s < G; ++s) {
+                const size_t i = (size_t)(g * G + s) * L.V + c;
+                const uint32_t d = g * G + s < L.S ? __ldg(&L.out[i]) : L.inf;
+                x[2 * s] = d != L.inf ? __ldg(&L.pred[i]) : NONE;
+                x[2 * s + 1] = d != L.inf ? d : 0xFFFFFFFFu;
+            }
+            if constexpr (G >= 2) {
+#pragma unroll
+                for (int s = 0; s < 2 * G; s += 4)
+                    *reinterpret_cast<uint4*>(row + s) = make_uint4(x[s], x[s + 1], x[s + 2], x[s + 3]);
+            } else {
+                *reinterpret_cast<uint2*>(row) = make_uint2(x[0], x[1]);
+            }
+        }
+    }
+}
+
+// Warm start: the result from the rows (also that of a sweep that gave up, to be packed again).
+template <int G>
+__global__ void k_warm_out(WarmLaunch L) {
+    const size_t stride = (size_t)gridDim.x * blockDim.x;
+    for (size_t c = (size_t)blockIdx.x * blockDim.x + threadIdx.x; c < L.V; c += stride) {
+        const uint32_t at = L.slots ? __ldg(&L.slots[c]) : (uint32_t)c;
+        for (uint32_t g = 0; g < L.groups; ++g) {
+            uint32_t x[2 * G];
+            load_final<2 * G>(L.dist + ((size_t)g * L.V + at) * (2 * G), x);
+#pragma unroll
+            for (int s = 0; s < G; ++s) {
+                if (g * G + s >= L.S) continue;
+                const size_t i = (size_t)(g * G + s) * L.V + c;
+                L.out[i] = min(x[2 * s + 1], L.inf);
+                L.pred[i] = x[2 * s];
+            }
+        }
+    }
+}
+
 // Handed over: the marked vertices become inbox bits of the sources that have reached them, their
 // units' doorbells are rung and they are counted.  One thread per inbox word (G = 1: the marks are
 // the inbox words already).
-template <int G>
-__global__ void k_sweep_requeue(SweepLaunch L, uint32_t* bitmap, uint32_t words, uint32_t B, uint32_t Bq, uint32_t split,
+template <int G, class Launch>
+__global__ void k_sweep_requeue(Launch L, uint32_t* bitmap, uint32_t words, uint32_t B, uint32_t Bq, uint32_t split,
                                 uint32_t Q) {
     if (L.hdr->swept) return;
     const size_t n = (size_t)L.S * words, stride = (size_t)gridDim.x * blockDim.x;
@@ -704,7 +835,9 @@ __global__ void k_sweep_requeue(SweepLaunch L, uint32_t* bitmap, uint32_t words,
         uint32_t bits = 0;
         for (uint32_t j = 0; j < 32u && wd * 32u + j < L.V; ++j) {
             const uint32_t item = s / G * L.V + wd * 32u + j;
-            if ((L.mark[item >> 5] >> (item & 31u) & 1u) && L.dist[(size_t)item * G + s % G] < L.inf) bits |= 1u << j;
+            size_t d = (size_t)item * G + s % G;
+            if (std::is_same<Launch, WarmLaunch>::value) d = 2 * d + 1;
+            if ((L.mark[item >> 5] >> (item & 31u) & 1u) && L.dist[d] < L.inf) bits |= 1u << j;
         }
         bitmap[i] = bits;
         if (!bits) continue;
@@ -718,13 +851,13 @@ __global__ void k_sweep_requeue(SweepLaunch L, uint32_t* bitmap, uint32_t words,
     }
 }
 
-template <class W>
+template <class W, class Launch>
 const void* sweep_kernel(uint32_t G) {
     switch (G) {
-        case 1: return (const void*)k_sweep<W, 1>;
-        case 2: return (const void*)k_sweep<W, 2>;
-        case 4: return (const void*)k_sweep<W, 4>;
-        default: return (const void*)k_sweep<W, 8>;
+        case 1: return (const void*)k_sweep<W, 1, Launch>;
+        case 2: return (const void*)k_sweep<W, 2, Launch>;
+        case 4: return (const void*)k_sweep<W, 4, Launch>;
+        default: return std::is_same<Launch, WarmLaunch>::value ? nullptr : (const void*)k_sweep<W, 8, SweepLaunch>;
     }
 }
 
@@ -742,8 +875,10 @@ size_t sweep_smem(uint32_t G) { return 4 * (size_t)NW * 32 * G; }
 
 }  // namespace
 
-cudaError_t sweep_max_blocks_per_sm(int wtype, uint32_t G, int* out) {
-    const void* k = wtype == SSSP_W_F32 ? sweep_kernel<WF32>(G) : sweep_kernel<WU32>(G);
+cudaError_t sweep_max_blocks_per_sm(int wtype, uint32_t G, bool warm, int* out) {
+    const bool f32 = wtype == SSSP_W_F32;
+    const void* k = warm ? (f32 ? sweep_kernel<WF32, WarmLaunch>(G) : sweep_kernel<WU32, WarmLaunch>(G))
+                         : (f32 ? sweep_kernel<WF32, SweepLaunch>(G) : sweep_kernel<WU32, SweepLaunch>(G));
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sweep_smem(G))) != cudaSuccess)
         return e;
@@ -756,9 +891,35 @@ cudaError_t launch_sweep(const SweepLaunch& L, int sms, cudaStream_t st) {
     const unsigned blocks = (unsigned)std::min<size_t>(std::max<size_t>((n + 255) / 256, 1), (size_t)sms * 8);
     k_sweep_init<<<blocks, 256, 0, st>>>(L, L.inf);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const void* k = L.wtype == SSSP_W_F32 ? sweep_kernel<WF32>(L.G) : sweep_kernel<WU32>(L.G);
+    const void* k = L.wtype == SSSP_W_F32 ? sweep_kernel<WF32, SweepLaunch>(L.G) : sweep_kernel<WU32, SweepLaunch>(L.G);
     void* args[] = {const_cast<SweepLaunch*>(&L)};
     return cudaLaunchCooperativeKernel(k, dim3(L.grid), dim3(WT), args, sweep_smem(L.G), st);
+}
+
+cudaError_t launch_warm_sweep(const WarmLaunch& L, int sms, cudaStream_t st) {
+    cudaError_t e;
+    const unsigned blocks = (unsigned)std::min<size_t>(((size_t)L.V + 255) / 256, (size_t)sms * 8);
+    switch (L.G) {
+        case 1: k_warm_rows<1><<<blocks, 256, 0, st>>>(L); break;
+        case 2: k_warm_rows<2><<<blocks, 256, 0, st>>>(L); break;
+        default: k_warm_rows<4><<<blocks, 256, 0, st>>>(L); break;
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // (the previous result has been read: its place holds the marks and the lists)
+    if ((e = cudaMemsetAsync(L.mark, 0, 4 * (((size_t)L.items + 31) / 32), st)) != cudaSuccess) return e;
+    const void* k = L.wtype == SSSP_W_F32 ? sweep_kernel<WF32, WarmLaunch>(L.G) : sweep_kernel<WU32, WarmLaunch>(L.G);
+    void* args[] = {const_cast<WarmLaunch*>(&L)};
+    return cudaLaunchCooperativeKernel(k, dim3(L.grid), dim3(WT), args, sweep_smem(L.G), st);
+}
+
+cudaError_t launch_warm_out(const WarmLaunch& L, int sms, cudaStream_t st) {
+    const unsigned blocks = (unsigned)std::min<size_t>(((size_t)L.V + 255) / 256, (size_t)sms * 8);
+    switch (L.G) {
+        case 1: k_warm_out<1><<<blocks, 256, 0, st>>>(L); break;
+        case 2: k_warm_out<2><<<blocks, 256, 0, st>>>(L); break;
+        default: k_warm_out<4><<<blocks, 256, 0, st>>>(L); break;
+    }
+    return cudaGetLastError();
 }
 
 cudaError_t launch_sweep_out(const SweepLaunch& L, int sms, cudaStream_t st) {
@@ -782,6 +943,17 @@ cudaError_t launch_sweep_requeue(const SweepLaunch& L, uint32_t* bitmap, uint32_
         case 2: k_sweep_requeue<2><<<grid, 256, 0, st>>>(L, bitmap, words, B, Bq, split, Q); break;
         case 4: k_sweep_requeue<4><<<grid, 256, 0, st>>>(L, bitmap, words, B, Bq, split, Q); break;
         default: k_sweep_requeue<8><<<grid, 256, 0, st>>>(L, bitmap, words, B, Bq, split, Q); break;
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_warm_requeue(const WarmLaunch& L, uint32_t* bitmap, uint32_t words, uint32_t B, uint32_t Bq,
+                                uint32_t split, uint32_t Q, int sms, cudaStream_t st) {
+    const unsigned grid = (unsigned)std::min<uint64_t>(((uint64_t)L.S * words + 255) / 256, (uint64_t)sms * 8);
+    switch (L.G) {
+        case 1: k_sweep_requeue<1><<<grid, 256, 0, st>>>(L, bitmap, words, B, Bq, split, Q); break;
+        case 2: k_sweep_requeue<2><<<grid, 256, 0, st>>>(L, bitmap, words, B, Bq, split, Q); break;
+        default: k_sweep_requeue<4><<<grid, 256, 0, st>>>(L, bitmap, words, B, Bq, split, Q); break;
     }
     return cudaGetLastError();
 }

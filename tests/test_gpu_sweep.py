@@ -150,3 +150,75 @@ def test_without_predecessors_and_in_an_unaligned_workspace(sssp):
                 d, pr, _ = oracle.dijkstra(ref, 600 * i)
                 assert np.array_equal(u32(dist[i]), d)
                 assert q is None or np.array_equal(u32(pred[i]), pr)
+
+
+@pytest.mark.parametrize("S", [1, 2, 3, 4, 6, 8, 12])
+@pytest.mark.parametrize("layout", [False, True])
+@pytest.mark.parametrize("f32", [False, True])
+def test_warm_start(sssp, S, layout, f32):
+    """Many tails (some listed twice): rows of 1, 2 and 4 packed words, several groups, hubs among the
+    tails, ties that a lower label wins."""
+    rng = np.random.default_rng(10 * S + layout)
+    V, E = 30011, 260000
+    src, dst, w = graph(rng, V, E, f32, hi=9)
+    src[:3000], dst[:3000] = 7, np.arange(3000)
+    src[3000:9000], dst[3000:9000] = 11, np.arange(6000)
+    sources = rng.integers(0, V, S).astype(np.uint32)
+    sources[0] = 7
+    g = sssp.build_csr(V, src, dst, w, partitions=13)
+    dist, pred = sssp.solve(sssp.layout(g) if layout else g, sources)[:2]
+    at = rng.permutation(E)[:17000]
+    w2 = w.copy()
+    w2[at] = w[at] * np.float32(0.6) if f32 else np.maximum(1, w[at] // 2)
+    g2 = sssp.build_csr(V, src, dst, w2, partitions=13)
+    dist, pred, st, stats = sssp.update(sssp.layout(g2) if layout else g2, dist, pred,
+                                        np.concatenate([src[at], src[at[:100]]]))
+    assert st == 0
+    ref = oracle.csr(V, src, dst, w2)
+    for i, s in enumerate(sources):
+        d, p, _ = oracle.dijkstra(ref, int(s))
+        assert np.array_equal(u32(dist[i]), d.view(np.uint32)), f"dist, source {s}"
+        assert np.array_equal(u32(pred[i]), p), f"pred, source {s}"
+
+
+@pytest.mark.parametrize("S", [1, 4])
+@pytest.mark.parametrize("kind", ["full lists", "chain"])
+def test_warm_start_handed_over(sssp, S, kind):
+    """More items than a list holds, and a chain of more iterations than a warm sweep takes."""
+    rng = np.random.default_rng(S)
+    if kind == "full lists":
+        V = 40000
+        src, dst, w = graph(rng, V, 6 * V)
+        w2 = np.maximum(1, w // 3).astype(np.uint32)
+        tails = src
+    else:  # each vertex to the next six
+        V = 20000
+        src = np.repeat(np.arange(V - 6), 6).astype(np.uint32)
+        dst = src + np.tile(np.arange(1, 7), V - 6).astype(np.uint32)
+        w = rng.integers(50, 60, src.size).astype(np.uint32)
+        w2 = w.copy()
+        w2[:12] = 1
+        tails = np.concatenate([src[:12], np.full(20000, V - 1, np.uint32)])
+    sources = np.arange(S).astype(np.uint32)
+    dist, pred = sssp.solve(sssp.build_csr(V, src, dst, w), sources)[:2]
+    dist, pred, st, _ = sssp.update(sssp.build_csr(V, src, dst, w2), dist, pred, tails)
+    assert st == 0
+    ref = oracle.csr(V, src, dst, w2)
+    for i, s in enumerate(sources):
+        d, p, _ = oracle.dijkstra(ref, int(s))
+        assert np.array_equal(u32(dist[i]), d), f"dist, source {s}"
+        assert np.array_equal(u32(pred[i]), p), f"pred, source {s}"
+
+
+def test_warm_start_with_a_bad_tail(sssp):
+    rng = np.random.default_rng(4)
+    V = 20000
+    src, dst, w = graph(rng, V, 8 * V)
+    g = sssp.build_csr(V, src, dst, w)
+    dist, pred = sssp.solve(g, np.array([3, 4], np.uint32))[:2]
+    d0, p0 = dist.clone(), pred.clone()
+    tails = src.copy()
+    tails[5] = V
+    dist, pred, st, _ = sssp.update(g, dist, pred, tails, check=False)
+    assert st == sssp.SSSP_EINVAL
+    assert torch.equal(dist, d0) and torch.equal(pred, p0)
