@@ -21,7 +21,8 @@ struct WsHeader {
     unsigned long long work_next;  // batched work-queue cursor
     unsigned long long stats[9];   // sssp_stats
     uint32_t swept;         // the sweep finished: nothing is left for the persistent solve
-    uint32_t pad[(256 - 4 - 4 - 8 - 8 - 72 - 4) / 4];
+    uint32_t lay_general;   // layout: the rows cannot be sorted segment by segment
+    uint32_t pad[(256 - 4 - 4 - 8 - 8 - 72 - 8) / 4];
 };
 static_assert(sizeof(WsHeader) == 256, "header size");
 

@@ -65,8 +65,10 @@ CsrWs carve_csr(void* ws, uint32_t V, uint64_t n) {
 
 // runs that start in each tile (totals[tiles] = 0 for the scan's last word)
 __global__ void __launch_bounds__(EMIT_THREADS) k_csr_runs(const unsigned long long* __restrict__ count,
-                                                           const unsigned long long* __restrict__ keys, uint32_t* totals) {
+                                                           const unsigned long long* __restrict__ keys, uint32_t* totals,
+                                                           const uint32_t* run) {
     __shared__ uint32_t sum;
+    if (run && !*run) return;
     const unsigned long long n = *count, base = (unsigned long long)blockIdx.x * EMIT_TILE;
     if (threadIdx.x == 0) sum = 0;
     __syncthreads();
@@ -92,7 +94,8 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_csr_emit(uint32_t V, uint32_t 
                                                            const uint32_t* __restrict__ before, unsigned long long* lead,
                                                            uint32_t tiles, uint32_t* row_ptr, uint32_t* col,
                                                            uint32_t* w_out, uint32_t* eid, uint32_t* E_out,
-                                                           const WsHeader* hdr) {
+                                                           const WsHeader* hdr, const uint32_t* sorted) {
+    if (sorted && !*sorted) return;
     __shared__ unsigned long long best[EMIT_TILE + 1];  // [0]: pairs of a run that starts in an earlier tile
     __shared__ uint32_t wsum[EMIT_WARPS];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, wid = tid >> 5;
@@ -171,8 +174,9 @@ __global__ void __launch_bounds__(EMIT_THREADS) k_csr_emit(uint32_t V, uint32_t 
 
 // a run that crosses into tile t and starts before it: the minimum of what the tiles from t on hold of it
 __global__ void k_csr_cross(uint32_t tiles, const uint32_t* __restrict__ before,
-                            const unsigned long long* __restrict__ lead, uint32_t* w_out, uint32_t* eid) {
+                            const unsigned long long* __restrict__ lead, uint32_t* w_out, uint32_t* eid, const uint32_t* run) {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (run && !*run) return;
     if (t == 0 || t >= tiles || lead[t] == NO_EDGE || before[t] == before[t - 1]) return;
     unsigned long long m = lead[t];
     for (uint32_t x = t; before[x + 1] == before[x] && x + 1 < tiles && lead[x + 1] != NO_EDGE; ++x) m = min(m, lead[x + 1]);
@@ -333,24 +337,141 @@ __global__ void __launch_bounds__(256) k_compact(uint32_t V, uint32_t E, const u
 
 // ---- locality layout: renumber vertices inside each block partition by degree
 
+constexpr uint32_t COO_RANGE = 1024;
+constexpr uint32_t LAY_TILE = 1024, LAY_SEG = 2048;     // stored edges of a block; longest segment
+constexpr uint32_t LAY_CAP = LAY_TILE + LAY_SEG + 32u;  // stored edges that a block holds
+
 __global__ void k_lay_deg(uint32_t V, const uint32_t* __restrict__ row_ptr, uint32_t* deg) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x)
         deg[v] = row_ptr[v + 1] - row_ptr[v];
 }
 
-__global__ void k_lay_indeg(uint32_t V, uint32_t E, const uint32_t* __restrict__ col, uint32_t* deg) {
-    for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < E; e += gridDim.x * blockDim.x) {
-        const uint32_t v = col[e];
-        if (v < V) atomicAdd(&deg[v], 1u);
+// In-degrees; and whether the rows can be sorted segment by segment (k_lay_rows): they are as sssp_build_csr
+// makes them, and no segment is longer than LAY_SEG.
+__global__ void __launch_bounds__(256) k_lay_check(uint32_t V, uint32_t E, uint32_t B, const uint32_t* __restrict__ row_ptr,
+                                                   const uint32_t* __restrict__ col, const uint32_t* __restrict__ w, int wtype,
+                                                   uint32_t* deg, WsHeader* hdr) {
+    __shared__ uint32_t rows[8][32], starts[8][32];
+    const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+    const unsigned long long first = ((unsigned long long)blockIdx.x * 8u + wid) * COO_RANGE;
+    if (first >= E) return;
+    const uint32_t e0 = (uint32_t)first, e1 = (uint32_t)min(first + COO_RANGE, (unsigned long long)E);
+    RowWalk walk{row_ptr, V, rows[wid], starts[wid]};
+    walk.seek(e0);
+    uint32_t before = e0 ? __ldg(&col[e0 - 1u]) : 0u;  // head of the edge before the step
+    bool odd = false;
+    uint32_t v = e0 + lane < e1 ? __ldg(&col[e0 + lane]) : 0u;
+    for (uint32_t eb = e0; eb < e1 && eb >= e0; eb += 32u) {
+        const uint32_t e = eb + lane, u = walk.step(eb, e1), x = v;
+        if (e1 - eb > 32u + lane) v = __ldg(&col[e + 32u]);  // the next step's
+        uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, 1);
+        if (lane == 0) y = before;
+        before = __shfl_sync(0xFFFFFFFFu, x, 31);
+        if (e < e1) {
+            const uint32_t at = e - __ldg(&row_ptr[u]), wt = __ldg(&w[e]);
+            odd = odd || x >= V || x == u || (at && y >= x) || !(wtype == SSSP_W_F32 ? WF32::weight_ok(wt) : WU32::weight_ok(wt));
+            if (at >= LAY_SEG && __ldg(&col[e - LAY_SEG]) / B == x / B) odd = true;
+            if (x < V) atomicAdd(&deg[x], 1u);
+        }
+    }
+    if (first == 0 && (row_ptr[0] != 0u || row_ptr[V] != E)) odd = true;
+    if (__any_sync(0xFFFFFFFFu, odd) && lane == 0) hdr->lay_general = 1u;
+}
+
+// Degrees of the stored vertices (and a last word for the scan).
+__global__ void k_lay_degrees(uint32_t V, const uint32_t* __restrict__ row_ptr, const uint32_t* __restrict__ ids, uint32_t* deg) {
+    for (uint32_t n = blockIdx.x * blockDim.x + threadIdx.x; n <= V; n += gridDim.x * blockDim.x) {
+        const uint32_t v = n < V ? ids[n] : 0u;
+        deg[n] = n < V && v < V ? row_ptr[v + 1] - row_ptr[v] : 0u;
     }
 }
 
-// key = (partition << 32) | ~degree: an ascending stable sort gives partitions in
-// order, each by degree descending, ties by id ascending (the values start in id order)
+// The stored rows' starts, and how far each row's edges have come from.
+__global__ void k_lay_starts(uint32_t V, const uint32_t* __restrict__ row_ptr, const uint32_t* __restrict__ ids,
+                             const uint32_t* __restrict__ start, uint32_t* from, uint32_t* row_ptr_out, const WsHeader* hdr) {
+    if (hdr->lay_general || hdr->status == SSSP_EINTERNAL) return;  // (EINTERNAL: the vertex sort gave up)
+    for (uint32_t n = blockIdx.x * blockDim.x + threadIdx.x; n <= V; n += gridDim.x * blockDim.x) {
+        row_ptr_out[n] = start[n];
+        if (n < V && ids[n] < V) from[n] = row_ptr[ids[n]] - start[n];
+    }
+}
+
+// The renumbered rows.  Renumbering keeps every head in its partition, and rows are sorted, so a row's edges
+// to one partition (a segment) stay where they are in the row and only change places among themselves.  A
+// block takes the segments that start in a tile of LAY_TILE stored edges, holds their new heads in shared
+// memory, and every edge counts the smaller heads of its segment: most segments are of a few edges (148
+// partitions), so this costs less than two passes of a sort.  Bound by instructions (350 a step of 32 edges,
+// 55% of the issue slots).  R-MAT, 4.2 M vertices, 63 M edges, 148 partitions: 1.0 ms where the renumbered
+// edge list and its sort took 4.1; the whole layout 10.7 -> 4.87 -> 2.06 ms.  Tiles of 512, 1,024, 2,048 and 4,096
+// edges: 2.11, 2.08, 2.12, 2.19; two, four and eight steps of a warp in flight: 2.12, 2.19, 2.37.
+// A row with a longer segment (hubs, few partitions) sends the whole graph to the builder, whose launches
+// otherwise find an empty list (0.11 ms): 1 M vertices, one partition 3.68 -> 3.74 ms.
+__global__ void __launch_bounds__(256) k_lay_rows(uint32_t V, uint32_t E, uint32_t B, const uint32_t* __restrict__ start,
+                                                  const uint32_t* __restrict__ from, const uint32_t* __restrict__ col,
+                                                  const uint32_t* __restrict__ w, const uint32_t* __restrict__ slots,
+                                                  const WsHeader* hdr, uint32_t* col_out, uint32_t* w_out, uint32_t* emap) {
+    __shared__ uint32_t head[LAY_CAP], old[LAY_CAP], flags[LAY_CAP / 32], rows[8][32], starts[8][32], total;
+    if (hdr->lay_general || hdr->status == SSSP_EINTERNAL) return;  // (EINTERNAL: the vertex sort gave up)
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, wid = tid >> 5;
+    const uint32_t k0 = blockIdx.x * LAY_TILE, most = min(LAY_CAP, E - k0);
+    const uint32_t a = wid * (LAY_TILE / 8u), z = wid == 7u ? most : min(a + LAY_TILE / 8u, most);
+    if (tid == 0) total = min(LAY_TILE, most);
+    __syncthreads();
+    if (a < most) {
+        RowWalk walk{start, V, rows[wid], starts[wid]};
+        walk.seek(k0 + a);
+        uint32_t row = 0, part = 0;  // of the edge before the step
+        for (uint32_t at = a; at < z; at += 32u) {
+            const uint32_t k = k0 + at + lane, u = walk.step(k0 + at, E);
+            const bool on = k < E;
+            const uint32_t e = on ? k + __ldg(&from[u]) : 0u, v = on ? __ldg(&col[e]) : 0u, p = v / B;
+            uint32_t r = __shfl_up_sync(0xFFFFFFFFu, u, 1), q = __shfl_up_sync(0xFFFFFFFFu, p, 1);
+            if (lane == 0) {
+                if (at == a) {
+                    const bool opens = __ldg(&start[u]) == k;
+                    row = opens ? NONE : u;
+                    part = opens ? 0u : __ldg(&col[e - 1u]) / B;
+                }
+                r = row;
+                q = part;
+            }
+            row = __shfl_sync(0xFFFFFFFFu, u, 31);
+            part = __shfl_sync(0xFFFFFFFFu, p, 31);
+            const uint32_t f = __ballot_sync(0xFFFFFFFFu, on && (r != u || q != p));
+            head[at + lane] = on ? __ldg(&slots[v]) : 0u;
+            old[at + lane] = e;
+            if (lane == 0) flags[at >> 5] = f;
+            if (at >= LAY_TILE) {  // the last warp, to the end of the tile's last segment
+                if (lane == 0) total = min(at + 32u, most);
+                if (f) break;
+            }
+        }
+    }
+    __syncthreads();
+    const uint32_t n = total;
+    for (uint32_t i = tid; i < n; i += 256u) {
+        uint32_t wd = i >> 5, m = flags[wd] & (0xFFFFFFFFu >> (31u - (i & 31u)));
+        while (!m && wd) m = flags[--wd];
+        const uint32_t s = wd * 32u + 31u - (uint32_t)__clz(m);
+        if (!m || s >= LAY_TILE) continue;  // another tile's
+        wd = i >> 5;
+        m = (i & 31u) == 31u ? 0u : flags[wd] & (0xFFFFFFFEu << (i & 31u));
+        while (!m && (wd + 1u) * 32u < n) m = flags[++wd];
+        const uint32_t end = m ? wd * 32u + (uint32_t)__ffs(m) - 1u : n;
+        const uint32_t h = head[i], e = old[i];
+        uint32_t c = 0;
+        for (uint32_t j = s; j < end; ++j) c += head[j] < h;
+        const uint32_t o = k0 + s + c;
+        col_out[o] = h;
+        w_out[o] = __ldg(&w[e]);
+        if (emap) emap[o] = e;
+    }
+}
+
 __global__ void k_lay_keys(uint32_t V, unsigned long long B, const uint32_t* __restrict__ deg,
-                           unsigned long long* keys, uint32_t* vals) {
+                           uint32_t bits, unsigned long long* keys, uint32_t* vals) {
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
-        keys[v] = ((unsigned long long)(v / B) << 32) | (0xFFFFFFFFu - deg[v]);
+        keys[v] = ((unsigned long long)(v / B) << bits) | ((0xFFFFFFFFu >> (32u - bits)) - deg[v]);
         vals[v] = v;
     }
 }
@@ -366,15 +487,14 @@ __global__ void k_lay_slots(uint32_t V, const uint32_t* __restrict__ order, uint
 // The edge list in the new numbering, in the old edge order: a warp walks a range of edges.  (R-MAT
 // scale 22: 2.4 ms with a warp per row, half of whose lanes had no edge, -> 0.31 ms, bound by the random
 // reads of slots.)
-constexpr uint32_t COO_RANGE = 1024;
 
 __global__ void __launch_bounds__(256) k_lay_coo(uint32_t V, uint32_t E, const uint32_t* __restrict__ row_ptr,
                                                  const uint32_t* __restrict__ col, const uint32_t* __restrict__ slots,
-                                                 uint32_t* src, uint32_t* dst) {
+                                                 const uint32_t* run, uint32_t* src, uint32_t* dst) {
     __shared__ uint32_t rows[8][32], starts[8][32];
     const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
     const unsigned long long first = ((unsigned long long)blockIdx.x * 8u + wid) * COO_RANGE;
-    if (first >= E) return;
+    if (first >= E || (run && !*run)) return;
     const uint32_t e0 = (uint32_t)first, e1 = (uint32_t)min(first + COO_RANGE, (unsigned long long)E);
     RowWalk walk{row_ptr, V, rows[wid], starts[wid]};
     walk.seek(e0);
@@ -408,7 +528,7 @@ size_t csr_workspace_bytes(uint32_t V, uint64_t E_raw) { return carve_csr(nullpt
 
 sssp_status csr_build(uint32_t V, uint64_t n, const uint32_t* src, const uint32_t* dst, const uint32_t* w, int wtype,
                       uint32_t* row_ptr, uint32_t* col, uint32_t* w_out, uint32_t* eid, uint32_t* E_out, void* ws,
-                      size_t ws_bytes, cudaStream_t st, bool clear) {
+                      size_t ws_bytes, cudaStream_t st, bool clear, const uint32_t* run) {
     CsrWs c = carve_csr(ws, V, n);
     if (ws_bytes < c.total) return SSSP_ENOMEM;
     const uint32_t bits = bits_for(V - 1u);
@@ -419,18 +539,18 @@ sssp_status csr_build(uint32_t V, uint64_t n, const uint32_t* src, const uint32_
         return SSSP_OK;
     }
     bool second = false;
-    CK(sort_edges(c.sort, V, bits, src, dst, w, wtype, n, c.keys[0], c.keys[1], c.vals[0], c.vals[1], c.hdr, st, &second));
+    CK(sort_edges(c.sort, V, bits, src, dst, w, wtype, n, c.keys[0], c.keys[1], c.vals[0], c.vals[1], run, c.hdr, st, &second));
     const unsigned long long* keys = c.keys[second];
     const uint32_t* vals = c.vals[second];
     const unsigned long long* count = sort_count(c.sort);
     const unsigned tiles = (unsigned)c.tiles;
-    k_csr_runs<<<tiles + 1, EMIT_THREADS, 0, st>>>(count, keys, c.totals);  // (the last block counts nothing)
+    k_csr_runs<<<tiles + 1, EMIT_THREADS, 0, st>>>(count, keys, c.totals, run);  // (the last block counts nothing)
     CK(cudaGetLastError());
     CK(exclusive_scan_u32(c.scan, c.totals, c.totals, c.tiles + 1, st));
     k_csr_emit<<<tiles, EMIT_THREADS, 0, st>>>(V, bits, count, keys, vals, w, c.totals, c.lead, tiles, row_ptr, col, w_out,
-                                               eid, E_out, c.hdr);
+                                               eid, E_out, c.hdr, run);
     CK(cudaGetLastError());
-    k_csr_cross<<<(tiles + 255) / 256, 256, 0, st>>>(tiles, c.totals, c.lead, w_out, eid);
+    k_csr_cross<<<(tiles + 255) / 256, 256, 0, st>>>(tiles, c.totals, c.lead, w_out, eid, run);
     CK(cudaGetLastError());
     return SSSP_OK;
 }
@@ -499,30 +619,45 @@ sssp_status layout_build(const sssp_graph* g, uint32_t* row_ptr_out, uint32_t* c
     uint32_t* dst = reinterpret_cast<uint32_t*>(p + L.off_dst);
     uint32_t* eout = reinterpret_cast<uint32_t*>(p + L.off_eout);
     const unsigned long long B = ((unsigned long long)g->V + g->partitions - 1) / g->partitions;
-    const unsigned gv = grid_for(g->V), ge = grid_for(std::max<uint32_t>(g->E, 1));
+    const unsigned gv = grid_for(g->V), gr = (unsigned)((g->E + 8ull * COO_RANGE - 1) / (8ull * COO_RANGE));
+    const uint32_t* const w = static_cast<const uint32_t*>(g->w);
+    WsHeader* const hdr = reinterpret_cast<WsHeader*>(p);
+    const bool segments = g->E != 0u && g->E < 0xF0000000u;
+    CK(cudaMemsetAsync(p, 0, WS_HEADER_BYTES, st));
     k_lay_deg<<<gv, 256, 0, st>>>(g->V, g->row_ptr, deg);
     CK(cudaGetLastError());
     if (g->E) {
-        k_lay_indeg<<<ge, 256, 0, st>>>(g->V, g->E, g->col, deg);
+        k_lay_check<<<gr, 256, 0, st>>>(g->V, g->E, (uint32_t)B, g->row_ptr, g->col, w, g->wtype, deg, hdr);
         CK(cudaGetLastError());
     }
-    k_lay_keys<<<gv, 256, 0, st>>>(g->V, B, deg, kin, vin);
+    const uint32_t bits = std::min(std::max(bits_for(g->E) + 1u, 1u), 32u);  // of a degree (in + out: at most 2 E)
+    k_lay_keys<<<gv, 256, 0, st>>>(g->V, B, deg, bits, kin, vin);
     CK(cudaGetLastError());
     bool second = false;
-    CK(cudaMemsetAsync(p, 0, WS_HEADER_BYTES, st));
-    CK(sort_pairs_u64(p + L.off_tmp, kin, kout, vin, vout, g->V, 32 + (int)bits_for(g->partitions - 1u),
-                      reinterpret_cast<WsHeader*>(p), st, &second));
+    CK(sort_pairs_u64(p + L.off_tmp, kin, kout, vin, vout, g->V, (int)(bits + bits_for(g->partitions - 1u)), hdr, st, &second));
     k_lay_slots<<<gv, 256, 0, st>>>(g->V, second ? vout : vin, ids_out, slots_out);
     CK(cudaGetLastError());
+    const uint32_t* const run = segments ? &hdr->lay_general : nullptr;
     if (g->E) {
-        k_lay_coo<<<(unsigned)((g->E + 8ull * COO_RANGE - 1) / (8ull * COO_RANGE)), 256, 0, st>>>(
-            g->V, g->E, g->row_ptr, g->col, slots_out, src, dst);
+        k_lay_coo<<<gr, 256, 0, st>>>(g->V, g->E, g->row_ptr, g->col, slots_out, run, src, dst);
         CK(cudaGetLastError());
     }
     // the renumbered edge list through the CSR builder: rows sorted by new head id, and
     // its input-index output maps each stored edge back to its index in g
-    return csr_build(g->V, g->E, src, dst, static_cast<const uint32_t*>(g->w), g->wtype, row_ptr_out, col_out, w_out,
-                     emap_out, eout, ws, L.csr_bytes, st, false);  // (the status of the vertex sort stays)
+    const sssp_status built = csr_build(g->V, g->E, src, dst, w, g->wtype, row_ptr_out, col_out, w_out, emap_out, eout, ws,
+                                        L.csr_bytes, st, false, run);  // (the status of the vertex sort stays)
+    if (built != SSSP_OK || !segments) return built;
+    uint32_t* const start = reinterpret_cast<uint32_t*>(kin);
+    uint32_t* const from = reinterpret_cast<uint32_t*>(kout);
+    k_lay_degrees<<<gv, 256, 0, st>>>(g->V, g->row_ptr, ids_out, start);
+    CK(cudaGetLastError());
+    CK(exclusive_scan_u32(deg, start, start, (uint64_t)g->V + 1, st));
+    k_lay_starts<<<gv, 256, 0, st>>>(g->V, g->row_ptr, ids_out, start, from, row_ptr_out, hdr);
+    CK(cudaGetLastError());
+    k_lay_rows<<<(g->E + LAY_TILE - 1u) / LAY_TILE, 256, 0, st>>>(g->V, g->E, (uint32_t)B, start, from, g->col, w, slots_out, hdr,
+                                                                  col_out, w_out, emap_out);
+    CK(cudaGetLastError());
+    return SSSP_OK;
 }
 
 namespace {

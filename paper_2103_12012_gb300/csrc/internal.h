@@ -161,7 +161,7 @@ size_t csr_workspace_bytes(uint32_t V, uint64_t E_raw);
 // clear: the workspace header first (else the caller has)
 sssp_status csr_build(uint32_t V, uint64_t E_raw, const uint32_t* src, const uint32_t* dst, const uint32_t* w,
                       int wtype, uint32_t* row_ptr, uint32_t* col, uint32_t* w_out, uint32_t* eid, uint32_t* E_out,
-                      void* ws, size_t ws_bytes, cudaStream_t st, bool clear = true);
+                      void* ws, size_t ws_bytes, cudaStream_t st, bool clear = true, const uint32_t* run = nullptr);
 cudaError_t partition_launch(const sssp_graph* g, uint32_t* bounds, uint64_t* inter, cudaStream_t st);
 size_t layout_workspace_bytes(uint32_t V, uint32_t E);
 sssp_status layout_build(const sssp_graph* g, uint32_t* row_ptr_out, uint32_t* col_out, uint32_t* w_out,
@@ -179,10 +179,11 @@ size_t sort_temp_bytes(uint64_t n);
 cudaError_t sort_pairs_u64(void* tmp, unsigned long long* k0, unsigned long long* k1, uint32_t* v0, uint32_t* v1,
                            uint64_t n, int end_bit, WsHeader* hdr, cudaStream_t st, bool* in_second);
 // The same for an edge list: keys (tail << bits) | head and values the edges' indices, loops and bad
-// edges (which set SSSP_EINVAL) left out; *sort_count(tmp) is the number of pairs, on the device.
+// edges (which set SSSP_EINVAL) left out; *sort_count(tmp) is the number of pairs, on the device.  With `run`
+// (device) and *run zero, the edge list is taken to be empty.
 cudaError_t sort_edges(void* tmp, uint32_t V, uint32_t bits, const uint32_t* src, const uint32_t* dst, const uint32_t* w,
                        int wtype, uint64_t n, unsigned long long* k0, unsigned long long* k1, uint32_t* v0, uint32_t* v1,
-                       WsHeader* hdr, cudaStream_t st, bool* in_second);
+                       const uint32_t* run, WsHeader* hdr, cudaStream_t st, bool* in_second);
 const unsigned long long* sort_count(const void* tmp);
 size_t scan_temp_bytes(uint64_t n);
 cudaError_t exclusive_scan_u32(void* tmp, const uint32_t* in, uint32_t* out, uint64_t n, cudaStream_t st);  // out may be in

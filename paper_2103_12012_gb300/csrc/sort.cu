@@ -91,6 +91,7 @@ struct Source {
     const uint32_t* src;
     const uint32_t* dst;
     uint32_t V, bits;
+    const uint32_t* run;  // edges: not NULL and zero: there are none
 };
 
 __device__ __forceinline__ bool edge_key(const Source& s, uint32_t a, uint32_t b, unsigned long long& k) {
@@ -133,6 +134,7 @@ __global__ void __launch_bounds__(512) k_sort_hist(Source s, unsigned long long 
     constexpr bool EDGES = !std::is_void<W>::value;
     __shared__ uint32_t h[PASSES][RADIX];
     __shared__ uint32_t cnt;
+    if (EDGES && s.run && !*s.run) return;
     for (uint32_t i = threadIdx.x; i < dg.passes * RADIX; i += blockDim.x) (&h[0][0])[i] = 0u;
     if (threadIdx.x == 0) cnt = 0u;
     __syncthreads();
@@ -202,7 +204,8 @@ __global__ void __launch_bounds__(THREADS, 3) k_sort_pass(Source s, unsigned lon
     extern __shared__ __align__(16) unsigned char raw[];
     PassMem& m = *reinterpret_cast<PassMem*>(raw);
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nd = 1u << bits;
-    const unsigned long long count = tmp->count, n = EDGES ? n_in : count;
+    const unsigned long long count = tmp->count, n = EDGES ? (s.run && !*s.run ? 0ull : n_in) : count;
+    if (n == 0) return;
     if (tid == 0) {
         m.tile = atomicAdd(&tmp->ticket[pass], 1u);
         m.fail = 0;
@@ -420,7 +423,7 @@ cudaError_t run_passes(const Source& first, uint64_t n, const Digits& dg, SortTm
         (p ? k_sort_pass<false, D> : k_sort_pass<EDGES, D>)<<<(unsigned)tiles, THREADS, sizeof(PassMem), st>>>(
             s, n, dg.shift[p], dg.bits[p], p, tmp, desc + (size_t)p * tiles * RADIX, k0, v0, hdr);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        s = Source{k0, v0, nullptr, nullptr, 0u, 0u};
+        s = Source{k0, v0, nullptr, nullptr, 0u, 0u, nullptr};
         std::swap(k0, k1);
         std::swap(v0, v1);
     }
@@ -461,7 +464,7 @@ cudaError_t sort_pairs_u64(void* tmp, unsigned long long* k0, unsigned long long
     cudaError_t e;
     if ((e = clear_sort(tmp, dg, n, st)) != cudaSuccess) return e;
     SortTmp* t = static_cast<SortTmp*>(tmp);
-    const Source s{k0, v0, nullptr, nullptr, 0u, 0u};
+    const Source s{k0, v0, nullptr, nullptr, 0u, 0u, nullptr};
     k_sort_hist<void><<<hist_grid(n), 512, 0, st>>>(s, n, nullptr, dg, t, hdr);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     *in_second = dg.passes & 1u;
@@ -471,12 +474,12 @@ cudaError_t sort_pairs_u64(void* tmp, unsigned long long* k0, unsigned long long
 
 cudaError_t sort_edges(void* tmp, uint32_t V, uint32_t bits, const uint32_t* src, const uint32_t* dst, const uint32_t* w,
                        int wtype, uint64_t n, unsigned long long* k0, unsigned long long* k1, uint32_t* v0, uint32_t* v1,
-                       WsHeader* hdr, cudaStream_t st, bool* in_second) {
+                       const uint32_t* run, WsHeader* hdr, cudaStream_t st, bool* in_second) {
     const Digits dg = digits_for(std::max<uint32_t>(2u * bits, 1u));
     cudaError_t e;
     if ((e = clear_sort(tmp, dg, n, st)) != cudaSuccess) return e;
     SortTmp* t = static_cast<SortTmp*>(tmp);
-    const Source s{nullptr, nullptr, src, dst, V, bits};
+    const Source s{nullptr, nullptr, src, dst, V, bits, run};
     if (wtype == SSSP_W_F32)
         k_sort_hist<WF32><<<hist_grid(n), 512, 0, st>>>(s, n, w, dg, t, hdr);
     else

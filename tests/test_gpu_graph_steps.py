@@ -169,3 +169,62 @@ def test_prune_blocks_and_shares(sssp, V, E, hubs, P, mode):
     rk, rw = oracle.trishla(ref, P, mode)
     assert np.array_equal(keep.cpu().numpy(), rk)
     assert np.array_equal(u32(wit), rw)
+
+
+@pytest.mark.parametrize("V,P,deg", [(2100, 1, 2048), (2100, 1, 2049), (70000, 12, 3000), (70000, 148, 60000), (70000, 1, 30000),
+                                     (5000, 2, 2047), (1025, 1025, 900)])
+@pytest.mark.parametrize("f32", [False, True])
+def test_layout_segments(sssp, V, P, deg, f32):
+    """Rows whose edges to one partition are as long as a block holds (2,048), longer (sorted by the
+    builder), and in several tiles; with rows of one edge between them."""
+    rng = np.random.default_rng(V + deg)
+    src, dst, w = edges(V, V, 5 * V)
+    hub = np.concatenate([np.stack([np.full(deg, h), rng.choice(V - 1, deg, replace=False)]) for h in (V - 1, V // 2, 3)], axis=1)
+    src, dst = np.concatenate([src, hub[0]]).astype(np.uint32), np.concatenate([dst, hub[1]]).astype(np.uint32)
+    w = rng.uniform(0.5, 2.0, src.size).astype(np.float32) if f32 else rng.integers(1, 99, src.size).astype(np.uint32)
+    ref = oracle.csr(V, src, dst, w)
+    h = sssp.layout(sssp.build_csr(V, src, dst, w, partitions=P))
+    ids, slots, lay = oracle.layout(ref, P)
+    assert np.array_equal(u32(h.ids), ids) and np.array_equal(u32(h.slots), slots)
+    assert np.array_equal(u32(h.row_ptr), lay.row_ptr)
+    assert np.array_equal(u32(h.col)[:h.E], lay.col[:h.E])
+    assert np.array_equal(u32(h.w)[:h.E], lay.w[:h.E].view(np.uint32))
+    e = u32(h.eid)[:h.E]  # the edges of the graph that they were
+    assert np.array_equal(np.sort(e), np.arange(h.E))
+    assert np.array_equal(slots[ref.col[:h.E]][e], lay.col[:h.E]) and np.array_equal(ref.w[:h.E].view(np.uint32)[e], u32(h.w)[:h.E])
+
+
+@pytest.mark.parametrize("what", ["order", "twice", "loop", "head", "weight"])
+def test_layout_of_rows_that_are_not_canonical(sssp, what):
+    """Rows out of order, repeated heads and loops go through the builder, as an edge list would; bad heads
+    and weights are reported."""
+    V, P = 3000, 7
+    src, dst, w = edges(5, V, 8 * V)
+    g = sssp.build_csr(V, src, dst, w, partitions=P)
+    rp, col, wt = u32(g.row_ptr), u32(g.col)[:g.E].copy(), u32(g.w)[:g.E].copy()
+    r = int(np.argmax(np.diff(rp.astype(np.int64))))
+    a = int(rp[r])
+    if what == "order":
+        col[a], col[a + 1] = col[a + 1], col[a]
+    elif what == "twice":
+        col[a + 1] = col[a]
+    elif what == "loop":
+        col[a] = r
+    elif what == "head":
+        col[a] = V
+    else:
+        wt[a] = 0
+    dev = lambda x: torch.from_numpy(x.view(np.int32)).cuda()
+    h = sssp.DeviceGraph(V, g.E, dev(rp.copy()), dev(col), dev(wt), g.wtype, P)
+    if what in ("head", "weight"):
+        with pytest.raises(sssp.SsspError):
+            sssp.layout(h)
+        return
+    out = sssp.layout(h)
+    tails = np.repeat(np.arange(V), np.diff(rp.astype(np.int64))).astype(np.uint32)
+    # the edge list renumbered by the ids that the layout found, through the oracle
+    slots = u32(out.slots)
+    want = oracle.csr(V, slots[tails], slots[col], wt)
+    E = int(want.row_ptr[-1])
+    assert np.array_equal(u32(out.row_ptr), want.row_ptr)
+    assert np.array_equal(u32(out.col)[:E], want.col[:E]) and np.array_equal(u32(out.w)[:E], want.w[:E])
