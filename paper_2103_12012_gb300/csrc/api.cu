@@ -592,8 +592,21 @@ sssp_status sssp_shard_problems(uint32_t n_problems, const uint64_t* cost, uint3
 
 namespace {
 
+// Bucket width of the shared-memory kernel: three times the one given, which suits the general kernel (in
+// shared memory an edge costs less and a round more: 220 graphs of 1,024 to 8,192 vertices, 16 sources each, 2.20
+// ms at the given width and 1.83 at three times it, 146 of 8,192 to 32,768 4.85 and 4.10).
+uint32_t wide_delta(int wtype, uint32_t delta_bits) {
+    if (wtype != SSSP_W_F32) return (uint32_t)std::min<uint64_t>(3ull * delta_bits, 0x7FFFFFFFu);
+    float f;
+    std::memcpy(&f, &delta_bits, 4);
+    f = std::min(f * 3.0f, 3.0e38f);
+    std::memcpy(&delta_bits, &f, 4);
+    return delta_bits;
+}
+
 struct BatchTables {
     std::vector<BatchProblem> probs;  // in processing order
+    std::vector<BatchUnit> units;     // instead, if shared memory holds every graph: groups of them
     uint64_t total_out = 0, total_words = 0;
 };
 
@@ -603,6 +616,7 @@ bool build_tables(const sssp_batch* b, BatchTables* t) {
     if (b->n_problems == 0 || b->n_graphs == 0) return false;
     t->probs.resize(b->n_problems);
     uint64_t out = 0;
+    uint32_t largest = 0;
     for (uint32_t i = 0; i < b->n_problems; ++i) {
         const uint32_t gi = b->prob_graph[i];
         if (gi >= b->n_graphs) return false;
@@ -617,7 +631,8 @@ bool build_tables(const sssp_batch* b, BatchTables* t) {
         p.V = G.V;
         p.src = b->prob_source[i];
         p.E = G.E;
-        p.pad = 0;
+        p.pad = gi;
+        largest = std::max(largest, G.V);
         out += G.V;
     }
     t->total_out = out;
@@ -625,37 +640,89 @@ bool build_tables(const sssp_batch* b, BatchTables* t) {
     // largest graphs first (longest-processing-time order), stable
     std::stable_sort(t->probs.begin(), t->probs.end(),
                      [](const BatchProblem& x, const BatchProblem& y) { return x.E > y.E; });
+    const uint64_t blocks = 2u * (uint64_t)std::max(sm_count(), 1);
+    if (largest <= BATCH_ITEMS) {
+        // The problems of a graph go to blocks in groups: as many as shared memory holds, while there
+        // are enough groups for the chip.  (The sort keeps the problems of a graph together, in order, unless
+        // another graph has as many edges.)
+        const uint32_t most = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(b->n_problems / blocks, 1), BATCH_COPIES);
+        for (size_t i = 0; i < t->probs.size();) {
+            const BatchProblem& p = t->probs[i];
+            BatchUnit u{};
+            u.row_off = p.row_off;
+            u.edge_off = p.edge_off;
+            u.V = p.V;
+            size_t end = i;
+            while (end < t->probs.size() && t->probs[end].pad == p.pad) ++end;
+            const size_t n = end - i, k = std::max(std::min(most, BATCH_ITEMS / p.V), 1u), groups = (n + k - 1) / k;
+            for (size_t g = 0; g < groups; ++g) {
+                u.S = 0;
+                for (size_t j = i + n * g / groups; j < i + n * (g + 1) / groups; ++j, ++u.S) {
+                    u.out[u.S] = t->probs[j].out_off;
+                    u.src[u.S] = t->probs[j].src;
+                }
+                t->units.push_back(u);
+            }
+            i = end;
+        }
+        t->probs.clear();
+        return true;
+    }
+    for (BatchProblem& p : t->probs) p.pad = 0;
+    // With the largest problems all at once the words in flight (8 bytes a vertex and the bitmaps) are several
+    // times L2: then a quarter of the work in flight comes from the other end, while there are problems
+    // enough to end evenly all the same (512 graphs of 1,024 to 131,072 vertices, 16 sources each: 32.6 -> 30.8
+    // ms, 8 each: 16.9 -> 16.5; 2 each, and 64 graphs of 16 each, would lose 5 to 9%).
+    uint64_t flying = 0;
+    for (size_t i = 0; i < std::min<size_t>(blocks, t->probs.size()); ++i) flying += t->probs[i].V;
+    if (t->probs.size() >= 12u * blocks && 10ull * flying > (96ull << 20)) {
+        std::vector<BatchProblem> mixed;
+        mixed.reserve(t->probs.size());
+        uint64_t front = 0, back = 0;  // work taken from either end
+        for (size_t i = 0, j = t->probs.size(); i < j;) {
+            const bool large = front <= 3u * back;
+            const BatchProblem& p = large ? t->probs[i++] : t->probs[--j];
+            (large ? front : back) += (uint64_t)p.E + p.V;
+            mixed.push_back(p);
+        }
+        t->probs.swap(mixed);
+    }
     return true;
 }
 
 struct BatchWs {
-    size_t off_probs, off_packed, off_bitmap, total;
+    size_t off_probs, off_units, off_packed, off_bitmap, total;
 };
 
-BatchWs batch_layout(uint32_t n_problems, uint64_t total_out, uint64_t total_words) {
+BatchWs batch_layout(const BatchTables& t) {
     BatchWs w{};
     size_t off = WS_HEADER_BYTES;
     w.off_probs = off;
-    off += align_up(sizeof(BatchProblem) * (size_t)n_problems, 256);
+    off += align_up(sizeof(BatchProblem) * t.probs.size(), 256);
+    w.off_units = off;
+    off += align_up(sizeof(BatchUnit) * t.units.size(), 256);
     w.off_packed = off;
-    off += align_up(8ull * total_out, 256);
+    off += align_up(8ull * t.total_out, 256);
     w.off_bitmap = off;
-    off += align_up(4ull * total_words * batched_bitmaps(), 256);
+    off += align_up(4ull * t.total_words * batched_bitmaps(), 256);
     w.total = off;
     return w;
 }
 
 sssp_status prepare_batch(const sssp_batch* b, const sssp_options* opt, void* ws, size_t ws_bytes,
-                          cudaStream_t st, BatchLaunch* l) {
+                          cudaStream_t st, BatchLaunch* l, BatchSmem* x) {
     Resolved r;
     BatchTables t;
     if (!ws || !aligned16(ws) || !resolve(opt, b ? b->wtype : 0, &r) || !build_tables(b, &t)) return SSSP_EINVAL;
     if (r.threads > BATCH_MAX_THREADS) return SSSP_EINVAL;
-    const BatchWs L = batch_layout(b->n_problems, t.total_out, t.total_words);
+    const BatchWs L = batch_layout(t);
     if (ws_bytes < L.total) return SSSP_ENOMEM;
     char* base = static_cast<char*>(ws);
-    if (cudaMemcpyAsync(base + L.off_probs, t.probs.data(), sizeof(BatchProblem) * t.probs.size(),
+    if (!t.probs.empty() && cudaMemcpyAsync(base + L.off_probs, t.probs.data(), sizeof(BatchProblem) * t.probs.size(),
                         cudaMemcpyHostToDevice, st) != cudaSuccess)
+        return SSSP_ECUDA;
+    if (!t.units.empty() && cudaMemcpyAsync(base + L.off_units, t.units.data(), sizeof(BatchUnit) * t.units.size(),
+                                            cudaMemcpyHostToDevice, st) != cudaSuccess)
         return SSSP_ECUDA;
     if (cudaStreamSynchronize(st) != cudaSuccess) return SSSP_ECUDA;
     int per_sm = 0;
@@ -666,20 +733,37 @@ sssp_status prepare_batch(const sssp_batch* b, const sssp_options* opt, void* ws
     l->col = b->col;
     l->w = static_cast<const uint32_t*>(b->w);
     l->wtype = b->wtype;
-    l->n_problems = b->n_problems;
+    l->n_problems = (uint32_t)t.probs.size();
     l->probs = reinterpret_cast<const BatchProblem*>(base + L.off_probs);
     l->hdr = reinterpret_cast<WsHeader*>(base);
     l->packed = reinterpret_cast<unsigned long long*>(base + L.off_packed);
     l->bitmap = reinterpret_cast<uint32_t*>(base + L.off_bitmap);
     l->threads = r.threads;
     l->tile = r.tile;
-    l->grid = (uint32_t)std::min<uint64_t>(b->n_problems, (uint64_t)per_sm * sm_count());
+    l->grid = (uint32_t)std::min<uint64_t>(t.probs.size(), (uint64_t)per_sm * sm_count());
     l->delta_bits = r.delta_bits;
     l->timeout_ns = r.timeout_ns;
     l->dist = static_cast<uint32_t*>(b->dist);
     l->pred = b->pred;
     l->ev_begin = r.ev_begin;
     l->ev_end = r.ev_end;
+    if (t.units.empty()) return SSSP_OK;
+    x->row_ptr = l->row_ptr;
+    x->col = l->col;
+    x->w = l->w;
+    x->wtype = l->wtype;
+    x->delta_bits = wide_delta(b->wtype, l->delta_bits);
+    x->units = reinterpret_cast<const BatchUnit*>(base + L.off_units);
+    x->n_units = (uint32_t)t.units.size();
+    for (const BatchUnit& u : t.units) x->items = std::max(x->items, u.S * u.V);
+    x->hdr = l->hdr;
+    x->dist = l->dist;
+    x->pred = l->pred;
+    x->timeout_ns = r.timeout_ns;
+    if (batch_smem_setup(b->wtype, x->items, &per_sm) != cudaSuccess) return SSSP_ECUDA;
+    if (per_sm <= 0) return SSSP_EUNSUPPORTED;
+    if (r.bps) per_sm = std::min<int>(per_sm, (int)r.bps);
+    x->grid = (uint32_t)std::min<uint64_t>(x->n_units, (uint64_t)per_sm * sm_count());
     return SSSP_OK;
 }
 
@@ -689,15 +773,16 @@ size_t sssp_batch_workspace_size(const sssp_batch* b, const sssp_options* opt) {
     Resolved r;
     BatchTables t;
     if (!resolve(opt, b ? b->wtype : 0, &r) || !build_tables(b, &t)) return 0;
-    return batch_layout(b->n_problems, t.total_out, t.total_words).total;
+    return batch_layout(t).total;
 }
 
 sssp_status sssp_solve_batched(const sssp_batch* b, const sssp_options* opt, void* ws, size_t ws_bytes,
                                sssp_stream_t stream) {
     BatchLaunch l{};
-    const sssp_status st = prepare_batch(b, opt, ws, ws_bytes, (cudaStream_t)stream, &l);
+    BatchSmem x{};
+    const sssp_status st = prepare_batch(b, opt, ws, ws_bytes, (cudaStream_t)stream, &l, &x);
     if (st != SSSP_OK) return st;
-    return launch_batched(l, (cudaStream_t)stream) == cudaSuccess ? SSSP_OK : SSSP_ECUDA;
+    return launch_batched(l, x, (cudaStream_t)stream) == cudaSuccess ? SSSP_OK : SSSP_ECUDA;
 }
 
 struct sssp_batch_plan {
@@ -710,8 +795,9 @@ sssp_status sssp_batch_plan_create(const sssp_batch* b, const sssp_options* opt,
     if (!plan) return SSSP_EINVAL;
     *plan = nullptr;
     BatchLaunch l{};
+    BatchSmem x{};
     cudaStream_t st = (cudaStream_t)stream;
-    sssp_status s = prepare_batch(b, opt, ws, ws_bytes, st, &l);
+    sssp_status s = prepare_batch(b, opt, ws, ws_bytes, st, &l, &x);
     if (s != SSSP_OK) return s;
     // capture on a private stream so that the caller's stream may be the legacy default stream
     cudaStream_t cap;
@@ -721,7 +807,7 @@ sssp_status sssp_batch_plan_create(const sssp_batch* b, const sssp_options* opt,
     l.ev_begin = l.ev_end = nullptr;  // timing events are for direct launches only
     bool ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
-        const cudaError_t le = launch_batched(l, cap);
+        const cudaError_t le = launch_batched(l, x, cap);
         const cudaError_t ce = cudaStreamEndCapture(cap, &graph);
         ok = le == cudaSuccess && ce == cudaSuccess && graph;
     }

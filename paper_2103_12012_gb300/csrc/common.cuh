@@ -22,7 +22,10 @@ struct WsHeader {
     unsigned long long stats[9];   // sssp_stats
     uint32_t swept;         // the sweep finished: nothing is left for the persistent solve
     uint32_t lay_general;   // layout: the rows cannot be sorted segment by segment
-    uint32_t pad[(256 - 4 - 4 - 8 - 8 - 72 - 8) / 4];
+    uint32_t unit_next;     // batch: next unit of the shared-memory kernel
+    uint32_t pad0;
+    unsigned long long begin;  // batch: time of its first block's start
+    uint32_t pad[(256 - 4 - 4 - 8 - 8 - 72 - 24) / 4];
 };
 static_assert(sizeof(WsHeader) == 256, "header size");
 

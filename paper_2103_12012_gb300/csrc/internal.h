@@ -127,6 +127,35 @@ cudaError_t relax_max_blocks_per_sm(int wtype, uint32_t threads, uint32_t tile, 
 // queued when it finished: every block sees a zero count at its first look and ends)
 cudaError_t launch_solve(const SolveLaunch& L, const SweepLaunch* sweep, cudaStream_t st);  // (L.warm: a WarmLaunch)
 
+// ------------------------------------------------------------------ batch.cu
+constexpr uint32_t BATCH_ITEMS = 47104;  // most vertices (of all copies) of a block
+constexpr uint32_t BATCH_COPIES = 16;
+
+// Problems of a batch on one graph that a block solves together.
+struct BatchUnit {
+    unsigned long long row_off, edge_off;
+    unsigned long long out[BATCH_COPIES];  // first output of each problem
+    uint32_t src[BATCH_COPIES];
+    uint32_t V, S, pad[2];
+};
+static_assert(sizeof(BatchUnit) % 16 == 0, "batch unit layout");
+
+struct BatchSmem {
+    const uint32_t* row_ptr;
+    const uint32_t* col;
+    const uint32_t* w;
+    int wtype;
+    uint32_t delta_bits;
+    const BatchUnit* units;  // device: largest first
+    uint32_t n_units, items, grid;  // items: most of a unit (it decides the block size)
+    WsHeader* hdr;
+    uint32_t* dist;
+    uint32_t* pred;
+    uint64_t timeout_ns;
+};
+cudaError_t batch_smem_setup(int wtype, uint32_t items, int* blocks_per_sm);  // (not a stream operation)
+void launch_batch_smem(const BatchSmem& B, cudaStream_t st);
+
 // One problem of a batch, in the order blocks take them (largest first).
 struct BatchProblem {
     unsigned long long row_off, edge_off, out_off, bm_off;
@@ -154,7 +183,7 @@ struct BatchLaunch {
 
 uint32_t batched_bitmaps();  // inbox bitmaps per batched problem (distance buckets + overflow)
 cudaError_t batched_max_blocks_per_sm(int wtype, uint32_t threads, uint32_t tile, int* out);
-cudaError_t launch_batched(const BatchLaunch& L, cudaStream_t st);
+cudaError_t launch_batched(const BatchLaunch& L, const BatchSmem& B, cudaStream_t st);  // B with units: instead of L's table
 
 // -------------------------------------------------------------------- csr.cu
 size_t csr_workspace_bytes(uint32_t V, uint64_t E_raw);

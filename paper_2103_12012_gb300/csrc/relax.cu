@@ -1269,7 +1269,8 @@ __global__ void __launch_bounds__(SOLVE_MAX_THREADS, 4) k_solve(SolveLaunch L) {
     flush_stats(L.hdr, sm.st);
 }
 
-// K5: persistent, dynamic: blocks pull whole problems from a work queue.  Compiled for
+// K5: persistent, dynamic: blocks pull whole problems from a work queue (batches with a graph that shared
+// memory does not hold; the others: batch.cu).  Compiled for
 // 2 x 1024 threads per SM (the register budget of 4 x 512): two 1024-thread blocks hold half the
 // problems in flight, and so half the distance state competing for L2, with twice the threads on
 // each problem's rounds (the 512-graph batch: 44.2 ms at tile 2048 against 47.0 ms with four
@@ -1484,14 +1485,16 @@ cudaError_t batched_max_blocks_per_sm(int wtype, uint32_t threads, uint32_t tile
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_batched<WU32>, (int)threads, smem);
 }
 
-cudaError_t launch_batched(const BatchLaunch& L, cudaStream_t st) {
+cudaError_t launch_batched(const BatchLaunch& L, const BatchSmem& B, cudaStream_t st) {
     cudaError_t e;
     if ((e = cudaMemsetAsync(L.hdr, 0, WS_HEADER_BYTES, st)) != cudaSuccess) return e;
     // the dynamic shared-memory limit was raised by batched_max_blocks_per_sm (not a stream
     // operation, so it stays outside any graph capture)
     const size_t smem = relax_smem_bytes(L.tile, 0, false);
     if (L.ev_begin && (e = cudaEventRecord(L.ev_begin, st)) != cudaSuccess) return e;
-    if (L.wtype == SSSP_W_F32)
+    if (B.n_units)
+        launch_batch_smem(B, st);
+    else if (L.wtype == SSSP_W_F32)
         k_batched<WF32><<<L.grid, L.threads, smem, st>>>(L);
     else
         k_batched<WU32><<<L.grid, L.threads, smem, st>>>(L);
