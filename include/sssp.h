@@ -324,7 +324,10 @@ sssp_status sssp_update(const sssp_graph* g, uint32_t S, void* dist, uint32_t* p
  * hub_count over {256, 512, 1024} is tried with 1, 1.5, 2 and 3 times that
  * delta under RELATIVE, FIXED and NEAR_FAR; then tile over {1024, 2048, 4096},
  * then split over {1, 2, 4}, then tile once more if the split changed (split
- * only where ws is large enough).  The base options' policy and hub_count are
+ * only where ws is large enough).  Candidates run the persistent solve (what
+ * sssp_update with few tails, sssp_solve_prune and message buffering run too); at the
+ * end the chosen one is timed as sssp_solve makes it, under RELATIVE, which may be a
+ * sweep, and taken if that is faster.  The base options' policy and hub_count are
  * ignored.  Each candidate runs `trials` times (>= 1) after one
  * warm-up, timed with CUDA events on `stream`; candidates that fail are
  * skipped.  Synchronous.  Results do not depend on the schedule, so dist and

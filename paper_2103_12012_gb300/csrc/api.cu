@@ -249,7 +249,8 @@ size_t sssp_solve_workspace_size(const sssp_graph* g, uint32_t S, const sssp_opt
 static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint32_t S, void* dist, uint32_t* pred,
                               const sssp_options* opt, void* ws, size_t ws_bytes, sssp_stream_t stream,
                               const uint32_t* tails, uint32_t n_tails, bool warm, int prune_mode = -1,
-                              uint8_t* keep = nullptr, uint32_t* witness = nullptr, bool least = false) {
+                              uint8_t* keep = nullptr, uint32_t* witness = nullptr, bool least = false,
+                              bool persistent = false) {
     Resolved r;
     if (!graph_ok(g) || S == 0 || (!warm && !sources) || !dist || !ws || !resolve(opt, g->wtype, &r))
         return SSSP_EINVAL;
@@ -265,7 +266,7 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
     // The persistent solve alone keeps its own, tighter layout: behind a gap, 276 doorbells made a solve of
     // 0.71 ms (random graph, 89,656 vertices, 4 sources, 69 partitions) one of 0.84.
     const bool sweep =
-        L.sweep && !prune && r.policy == SSSP_POLICY_RELATIVE && r.msg_buffer == 0 && !(r.flags & SSSP_FLAG_TEST_HOLD_PENDING) &&
+        L.sweep && !persistent && !prune && r.policy == SSSP_POLICY_RELATIVE && r.msg_buffer == 0 && !(r.flags & SSSP_FLAG_TEST_HOLD_PENDING) &&
         (warm ? warm_sweep_wins(S, n_tails, static_cast<char*>(ws) + L.off_packed) : sweep_wins(g, S, L, r.delta_given));
     if (!sweep) L = solve_layout(g, S, r.split, false);
     int per_sm = 0;
@@ -444,15 +445,21 @@ sssp_status sssp_autotune(const sssp_graph* g, const uint32_t* sources, uint32_t
         cudaEventDestroy(e0);
         return SSSP_ECUDA;
     }
-    // time one candidate: warm-up, then `trials` runs; +inf if it fails
-    auto run = [&](const sssp_options& o) -> float {
+    // time one candidate: warm-up, then `trials` runs; +inf if it fails.  The persistent solve alone: the
+    // sweep does not use the schedule, so its times would leave it to chance, and warm starts of few
+    // tails, prunes on idle time and buffered solves go by it.
+    auto run = [&](const sssp_options& o, bool persistent = true) -> float {
+        auto solve = [&]() {
+            return solve_impl(g, sources, S, dist, pred, &o, ws, ws_bytes, stream, nullptr, 0, false, -1, nullptr, nullptr,
+                              false, persistent);
+        };
         if (sssp_solve_workspace_size(g, S, &o) > ws_bytes || sssp_solve_workspace_size(g, S, &o) == 0)
             return INFINITY;
-        if (sssp_solve(g, sources, S, dist, pred, &o, ws, ws_bytes, stream) != SSSP_OK) return INFINITY;
+        if (solve() != SSSP_OK) return INFINITY;
         if (sssp_workspace_status(ws, stream, nullptr) != SSSP_OK) return INFINITY;
         cudaEventRecord(e0, st);
         for (uint32_t t = 0; t < trials; ++t)
-            if (sssp_solve(g, sources, S, dist, pred, &o, ws, ws_bytes, stream) != SSSP_OK) return INFINITY;
+            if (solve() != SSSP_OK) return INFINITY;
         cudaEventRecord(e1, st);
         if (sssp_workspace_status(ws, stream, nullptr) != SSSP_OK) return INFINITY;
         float ms = 0;
@@ -538,6 +545,16 @@ sssp_status sssp_autotune(const sssp_graph* g, const uint32_t* sources, uint32_t
                 cur_ms = ms;
                 cur = o;
             }
+        }
+    }
+    // the solve that the relative policy really makes: swept, where that is the rule
+    {
+        sssp_options o = cur;
+        o.policy = SSSP_POLICY_RELATIVE;
+        const float ms = run(o, false);
+        if (ms < cur_ms) {
+            cur_ms = ms;
+            cur = o;
         }
     }
     cudaEventDestroy(e0);
