@@ -56,8 +56,9 @@ struct RowWalk {
             const uint32_t k = seen + __popc(at & (0xFFFFFFFFu >> (31u - lane)));
             if (k) u = row[k - 1u];
             seen += __popc(at);
-            if (end >= min(eb + 32u, e1) || r0 >= V) return u;  // (r0: a last row that ends before e1)
+            if (end >= min(eb + 32u, e1)) return u;
             r0 += 32u;
+            if (r0 >= V) return u;  // (the last row ends before e1: an edge count that is too large)
             if (!window()) seek(end);
         }
     }
