@@ -328,13 +328,15 @@ struct Worker {
         fence_gpu();  // the lowered distances before the marks
         // Most lowered items are marked already: a mark seen here is cleared, if it is, after the fence,
         // and the distances are read after that.
+        // A short buffer is the last of an iteration: it skips the look, which would only lengthen the
+        // chain (random graph, 65,536 vertices, 8 sources: 529 -> 504 us; 16,384, 1 source: 338 -> 328).
         uint32_t fresh = 0;
 #pragma unroll
         for (uint32_t i = 0; i < MQ; ++i) {
             const uint32_t x = i * 32u + lane;
             if (x < nC) {
                 const uint32_t item = wm.low[x];
-                if (!(ld_relaxed(&L.mark[item >> 5]) >> (item & 31u) & 1u)) fresh |= 1u << i;
+                if (nC <= MARKS / 2u || !(ld_relaxed(&L.mark[item >> 5]) >> (item & 31u) & 1u)) fresh |= 1u << i;
             }
         }
         uint32_t nact = 0;
