@@ -623,7 +623,7 @@ uint32_t wide_delta(int wtype, uint32_t delta_bits) {
 
 struct BatchTables {
     std::vector<BatchProblem> probs;  // in processing order
-    std::vector<BatchUnit> units;     // instead, if shared memory holds every graph: groups of them
+    std::vector<BatchUnit> units;     // groups of those that shared memory takes
     uint64_t total_out = 0, total_words = 0;
 };
 
@@ -633,7 +633,7 @@ bool build_tables(const sssp_batch* b, BatchTables* t) {
     if (b->n_problems == 0 || b->n_graphs == 0) return false;
     t->probs.resize(b->n_problems);
     uint64_t out = 0;
-    uint32_t largest = 0;
+    uint64_t large = 0;  // problems that shared memory does not hold
     for (uint32_t i = 0; i < b->n_problems; ++i) {
         const uint32_t gi = b->prob_graph[i];
         if (gi >= b->n_graphs) return false;
@@ -649,7 +649,7 @@ bool build_tables(const sssp_batch* b, BatchTables* t) {
         p.src = b->prob_source[i];
         p.E = G.E;
         p.pad = gi;
-        largest = std::max(largest, G.V);
+        large += G.V > BATCH_ITEMS;
         out += G.V;
     }
     t->total_out = out;
@@ -658,13 +658,24 @@ bool build_tables(const sssp_batch* b, BatchTables* t) {
     std::stable_sort(t->probs.begin(), t->probs.end(),
                      [](const BatchProblem& x, const BatchProblem& y) { return x.E > y.E; });
     const uint64_t blocks = 2u * (uint64_t)std::max(sm_count(), 1);
-    if (largest <= BATCH_ITEMS) {
+    // Shared memory takes all problems that it holds if it holds every graph, or if the others fill the chip
+    // several times by themselves (the two kernels run one after the other: 512 graphs of 1,024 to 131,072
+    // vertices, 16 sources each, 1,648 large problems, 30.8 -> 29.1 ms, float32 27.9 -> 24.4; 2 each, 206 large ones,
+    // would go from 5.4 to 6.3).
+    if (large == 0 || large >= 4u * blocks) {
         // The problems of a graph go to blocks in groups: as many as shared memory holds, while there
         // are enough groups for the chip.  (The sort keeps the problems of a graph together, in order, unless
         // another graph has as many edges.)
-        const uint32_t most = (uint32_t)std::min<uint64_t>(std::max<uint64_t>(b->n_problems / blocks, 1), BATCH_COPIES);
+        std::vector<BatchProblem> rest;
+        const uint32_t most = (uint32_t)std::min<uint64_t>(std::max<uint64_t>((b->n_problems - large) / blocks, 1), BATCH_COPIES);
         for (size_t i = 0; i < t->probs.size();) {
             const BatchProblem& p = t->probs[i];
+            if (p.V > BATCH_ITEMS) {
+                rest.push_back(p);
+                rest.back().pad = 0;
+                ++i;
+                continue;
+            }
             BatchUnit u{};
             u.row_off = p.row_off;
             u.edge_off = p.edge_off;
@@ -682,14 +693,14 @@ bool build_tables(const sssp_batch* b, BatchTables* t) {
             }
             i = end;
         }
-        t->probs.clear();
+        t->probs.swap(rest);
         return true;
     }
     for (BatchProblem& p : t->probs) p.pad = 0;
     // With the largest problems all at once the words in flight (8 bytes a vertex and the bitmaps) are several
     // times L2: then a quarter of the work in flight comes from the other end, while there are problems
-    // enough to end evenly all the same (512 graphs of 1,024 to 131,072 vertices, 16 sources each: 32.6 -> 30.8
-    // ms, 8 each: 16.9 -> 16.5; 2 each, and 64 graphs of 16 each, would lose 5 to 9%).
+    // enough to end evenly all the same (512 graphs of 1,024 to 131,072 vertices, 8 sources each: 16.9 -> 16.5
+    // ms; 2 each, and 64 graphs of 16 each, would lose 5 to 9%).
     uint64_t flying = 0;
     for (size_t i = 0; i < std::min<size_t>(blocks, t->probs.size()); ++i) flying += t->probs[i].V;
     if (t->probs.size() >= 12u * blocks && 10ull * flying > (96ull << 20)) {

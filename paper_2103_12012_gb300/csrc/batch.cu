@@ -1,4 +1,5 @@
-// K5b: a batch whose graphs all fit in shared memory.  A block takes a unit (one problem, or up to 16 of a
+// K5b: the problems of a batch in shared memory: all of them if every graph fits, or the ones that do of a
+// large batch (api.cu).  A block takes a unit (one problem, or up to 16 of a
 // graph, as copies of it with a source each) from a queue and keeps its distances there, 4 bytes an
 // item: reading a head's distance, lowering it and marking it cost tens of cycles instead of the L2 round
 // trips of the general kernel (k_batched, relax.cu), which stays for larger graphs.

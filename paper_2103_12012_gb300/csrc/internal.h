@@ -183,7 +183,7 @@ struct BatchLaunch {
 
 uint32_t batched_bitmaps();  // inbox bitmaps per batched problem (distance buckets + overflow)
 cudaError_t batched_max_blocks_per_sm(int wtype, uint32_t threads, uint32_t tile, int* out);
-cudaError_t launch_batched(const BatchLaunch& L, const BatchSmem& B, cudaStream_t st);  // B with units: instead of L's table
+cudaError_t launch_batched(const BatchLaunch& L, const BatchSmem& B, cudaStream_t st);  // L's table, then B's units
 
 // -------------------------------------------------------------------- csr.cu
 size_t csr_workspace_bytes(uint32_t V, uint64_t E_raw);

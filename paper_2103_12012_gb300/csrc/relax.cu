@@ -1269,8 +1269,8 @@ __global__ void __launch_bounds__(SOLVE_MAX_THREADS, 4) k_solve(SolveLaunch L) {
     flush_stats(L.hdr, sm.st);
 }
 
-// K5: persistent, dynamic: blocks pull whole problems from a work queue (batches with a graph that shared
-// memory does not hold; the others: batch.cu).  Compiled for
+// K5: persistent, dynamic: blocks pull whole problems from a work queue (graphs that shared memory does not
+// hold, and the others of such a batch unless it is large: batch.cu).  Compiled for
 // 2 x 1024 threads per SM (the register budget of 4 x 512): two 1024-thread blocks hold half the
 // problems in flight, and so half the distance state competing for L2, with twice the threads on
 // each problem's rounds (the 512-graph batch: 44.2 ms at tile 2048 against 47.0 ms with four
@@ -1492,12 +1492,11 @@ cudaError_t launch_batched(const BatchLaunch& L, const BatchSmem& B, cudaStream_
     // operation, so it stays outside any graph capture)
     const size_t smem = relax_smem_bytes(L.tile, 0, false);
     if (L.ev_begin && (e = cudaEventRecord(L.ev_begin, st)) != cudaSuccess) return e;
-    if (B.n_units)
-        launch_batch_smem(B, st);
-    else if (L.wtype == SSSP_W_F32)
+    if (L.n_problems && L.wtype == SSSP_W_F32)
         k_batched<WF32><<<L.grid, L.threads, smem, st>>>(L);
-    else
+    else if (L.n_problems)
         k_batched<WU32><<<L.grid, L.threads, smem, st>>>(L);
+    if (B.n_units) launch_batch_smem(B, st);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (L.ev_end && (e = cudaEventRecord(L.ev_end, st)) != cudaSuccess) return e;
     return cudaSuccess;

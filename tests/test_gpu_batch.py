@@ -103,6 +103,19 @@ def test_large_and_small_ends_together(sssp):
     check(b, graphs, step=9)
 
 
+def test_large_batch_split_over_both_kernels(sssp):
+    """Large problems for several rounds of blocks, and small graphs among them."""
+    rng = np.random.default_rng(12)
+    graphs = [graph(rng, V, 2 * V) for V in (47200, 300, 47104)]
+    sources = [rng.integers(0, g.V, n).tolist() for g, n in zip(graphs, (1300, 70, 9))]
+    b = sssp.Batch(graphs, sources, sssp.options(delta=32.0))
+    b.make_plan()
+    for _ in range(2):
+        b.replay()
+    check(b, graphs, step=23)
+    assert b.status()[1]["vertices"] > 0
+
+
 @pytest.mark.parametrize("V", [38000, 47000])
 def test_hub_rows(sssp, V):
     """Rows of 511, 512 and 513 edges, and three rows of every vertex in one round: more segments than
