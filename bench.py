@@ -11,8 +11,8 @@ value  = GTEPS: edges (after dedupe) whose tail is reached, summed over the
          step's sources, / device time per step (CUDA events, max over ranks).
 e2e    = the same metric through the C ABI with host buffers: pinned host CSR
          and sources copied in, dist/pred copied out, inside the timed region.
-roofline: the persistent relaxation kernel (launch timed alone with events
-         recorded by the library on the launching stream); algorithmic bytes
+roofline: the relaxation (the sweep's launches, or the persistent kernel, timed with
+         events recorded by the library on the launching stream); algorithmic bytes
          per source = 8 per reached edge (col + weight) + 16 per reached vertex
          (row_ptr pair + final packed word).
 --impl reference: the CPU oracle (binary-heap Dijkstra) on the same workload,
@@ -343,14 +343,15 @@ def run_ours(a):
                                "delta": opts.delta or 4, "split": opts.split or 1,
                                "policy": sssp.POLICY_NAMES[opts.policy], "hub_count": opts.hub_count,
                                "autotuned": not (a.no_tune or a.threads or a.tile or a.delta or a.split)}},
-        "roofline": {"bound": "hbm", "kernel": "k_solve (persistent relaxation)", "achieved": round(achieved, 1),
+        "roofline": {"bound": "hbm", "kernel": "k_sweep + k_sweep_out (k_solve if the schedule does not sweep)", "achieved": round(achieved, 1),
                      "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": round(achieved / peak, 4),
                      "traffic": traffic, "traffic_note": traffic_note, "alg_bytes_per_launch": alg_bytes,
                      "kernel_ms": round(relax_avg, 4), "kernel_ms_median": round(statistics.median(relax_ms), 4)},
         "cpu_baseline": cpu,
         "e2e": e2e,
         "clocks": clk,
-        "gpu_launches": 4 * a.steps,
+        # a swept solve: init, k_sweep, k_sweep_out, requeue, pack, k_solve, unpack; else init, seed, k_solve, unpack
+        "gpu_launches": (7 if opts.policy == 0 and opts.msg_buffer == 0 else 4) * a.steps,
         "phases": {"csr_build_ms": round(csr_ms, 3), "partition_ms": round(part_ms, 3),
                    "layout_ms": round(layout_ms, 3),
                    "prune_local_ms": round(prune_ms, 3), "pruned_edges": pruned, "edges": g.E,
