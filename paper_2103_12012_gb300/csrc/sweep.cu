@@ -99,6 +99,11 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
 
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
+__device__ __forceinline__ void and_acquire(uint32_t* p, uint32_t v) {
+    uint32_t old;
+    asm volatile("atom.acquire.gpu.global.and.b32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+}
+
 // The G distances of an item from L2 (rows are aligned to their size, 32 bytes at most): one
 // 256-bit load for eight (two 128-bit ones made twice the L1 and L2 requests).  Not ordered with
 // other accesses by the compiler: what an older value lets through is settled by the atomic.
@@ -109,13 +114,13 @@ __device__ __forceinline__ void load_row(const uint32_t* p, uint32_t (&r)[G]) {
                      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                      : "l"(p));
     } else if constexpr (G == 4) {
-        const uint4 a = __ldcg(reinterpret_cast<const uint4*>(p));
-        r[0] = a.x, r[1] = a.y, r[2] = a.z, r[3] = a.w;
+        asm volatile("ld.relaxed.gpu.global.v4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "l"(p));
     } else if constexpr (G == 2) {
-        const uint2 a = __ldcg(reinterpret_cast<const uint2*>(p));
-        r[0] = a.x, r[1] = a.y;
+        asm volatile("ld.relaxed.gpu.global.v2.b32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "l"(p));
     } else {
-        r[0] = __ldcg(p);
+        asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(r[0]) : "l"(p));
     }
 }
 
@@ -289,13 +294,13 @@ struct Worker {
     }
 
     // Takes the item of each lane with `ok`: its mark is cleared before its distances are read, so a
-    // distance lowered after the read marks it again.
+    // distance lowered after the read marks it again (mark_all).  An atomic with acquire semantics: a
+    // reduction, which has no result, reads nothing that could order the loads after it.
     __device__ __forceinline__ void take(bool ok, uint32_t item, uint32_t (&r)[G]) {
 #pragma unroll
         for (int s = 0; s < G; ++s) r[s] = Dist<W>::INF;
         if (ok) {
-            atomicAnd(&L.mark[item >> 5], ~(1u << (item & 31u)));
-            fence_gpu();
+            and_acquire(&L.mark[item >> 5], ~(1u << (item & 31u)));
             load_dist(item, r);
         }
     }
@@ -321,32 +326,26 @@ struct Worker {
         return fin;
     }
 
-    // Marks the nC buffered items, whose distances this warp has lowered, MQ a lane with their
-    // accesses in flight together; newly marked ones go to the list being filled.
+    // Marks the nC buffered items, whose distances this warp has lowered, MQ a lane; newly marked ones go to
+    // the list being filled.  A mark is always set by a read-modify-write, also where the item has one: it
+    // comes either before the clearing in take, which then sees the lowered distance (the fence here, the
+    // mark, the acquire there), or after it, and lists the item again.  A plain look that left marked items out
+    // would not be ordered so (each side would write one word and read the other's) without a sequentially
+    // consistent fence on both sides, and with them it is no faster: R-MAT scale 22, 8 sources 4.04 ms with
+    // the look, 3.98 without; random graphs of 16,384 vertices, 1 source 333 and 309 us, of 1 M, 8 sources
+    // 2.29 and 2.22 ms.
     __device__ __forceinline__ void mark_all() {
         __syncwarp();
         fence_gpu();  // the lowered distances before the marks
-        // Most lowered items are marked already: a mark seen here is cleared, if it is, after the fence,
-        // and the distances are read after that.
-        // A short buffer is the last of an iteration: it skips the look, which would only lengthen the
-        // chain (random graph, 65,536 vertices, 8 sources: 529 -> 504 us; 16,384, 1 source: 338 -> 328).
-        uint32_t fresh = 0;
-#pragma unroll
-        for (uint32_t i = 0; i < MQ; ++i) {
-            const uint32_t x = i * 32u + lane;
-            if (x < nC) {
-                const uint32_t item = wm.low[x];
-                if (nC <= MARKS / 2u || !(ld_relaxed(&L.mark[item >> 5]) >> (item & 31u) & 1u)) fresh |= 1u << i;
-            }
-        }
         uint32_t nact = 0;
 #pragma unroll
         for (uint32_t i = 0; i < MQ; ++i) {
-            bool f = fresh & (1u << i);
+            const uint32_t x = i * 32u + lane;
+            bool f = x < nC;
             if (!__any_sync(0xFFFFFFFFu, f)) continue;
             uint32_t item = 0, deg = 0;
             if (f) {
-                item = wm.low[i * 32u + lane];
+                item = wm.low[x];
                 const uint32_t v = vertex(item), bit = 1u << (item & 31u);
                 const uint32_t r0 = __ldg(&L.row_ptr[v]), r1 = __ldg(&L.row_ptr[v + 1]);  // in flight with the atomic
                 f = !(atomicOr(&L.mark[item >> 5], bit) & bit);

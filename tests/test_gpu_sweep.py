@@ -222,3 +222,24 @@ def test_warm_start_with_a_bad_tail(sssp):
     dist, pred, st, _ = sssp.update(g, dist, pred, tails, check=False)
     assert st == sssp.SSSP_EINVAL
     assert torch.equal(dist, d0) and torch.equal(pred, p0)
+
+
+@pytest.mark.parametrize("S", [1, 2, 4, 8, 9])
+@pytest.mark.parametrize("f32", [False, True])
+def test_marks_under_contention(sssp, S, f32):
+    """A small dense graph: every iteration lowers most distances several times from many warps while their
+    items are taken, so an item whose mark is set and cleared in the wrong order keeps a distance that
+    is too large.  Repeated, with the same result each time."""
+    rng = np.random.default_rng(70 + S)
+    V = 3001
+    src, dst, w = graph(rng, V, 150 * V, f32, hi=1000000)
+    ref = oracle.csr(V, src, dst, w)
+    g = sssp.build_csr(V, src, dst, w, partitions=5)
+    sources = rng.integers(0, V, S).astype(np.uint32)
+    stats = check(sssp, g, ref, sources.tolist())
+    assert stats["remote_activations"] == 0 and stats["rounds"] > 0  # (swept)
+    first = [t.clone() for t in sssp.solve(g, sources)[:2]]
+    solver = sssp.Solver(g, S)
+    for _ in range(50):
+        dist, pred = solver(sources)
+        assert torch.equal(dist, first[0]) and torch.equal(pred, first[1])
