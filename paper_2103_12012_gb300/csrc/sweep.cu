@@ -142,13 +142,21 @@ __device__ __forceinline__ void load_final(const uint32_t* p, uint32_t (&r)[G]) 
     }
 }
 
-// G packed words of an item: predecessors, distances
+// G packed words of an item: predecessors, distances.  Loaded as 64-bit elements, each of which is whole (the
+// halves of a word read apart could be a new distance with an old, lower label: a candidate of that
+// distance and a label between the two would be dropped).
 template <int G>
 __device__ __forceinline__ void load_keys(const uint32_t* dist, uint32_t item, uint32_t (&lo)[G], uint32_t (&hi)[G]) {
-    uint32_t x[2 * G];
-    load_row<2 * G>(dist + (size_t)item * (2 * G), x);
+    const uint32_t* const p = dist + (size_t)item * (2 * G);
+    unsigned long long x[G];
+    if constexpr (G == 4)
+        asm volatile("ld.relaxed.gpu.global.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(x[0]), "=l"(x[1]), "=l"(x[2]), "=l"(x[3]) : "l"(p));
+    else if constexpr (G == 2)
+        asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(x[0]), "=l"(x[1]) : "l"(p));
+    else
+        asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(x[0]) : "l"(p));
 #pragma unroll
-    for (int s = 0; s < G; ++s) lo[s] = x[2 * s], hi[s] = x[2 * s + 1];
+    for (int s = 0; s < G; ++s) lo[s] = (uint32_t)x[s], hi[s] = (uint32_t)(x[s] >> 32);
 }
 
 template <int G>

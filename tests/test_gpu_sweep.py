@@ -243,3 +243,23 @@ def test_marks_under_contention(sssp, S, f32):
     for _ in range(50):
         dist, pred = solver(sources)
         assert torch.equal(dist, first[0]) and torch.equal(pred, first[1])
+
+
+@pytest.mark.parametrize("S", [1, 2, 3, 4, 8])
+def test_warm_ties_under_contention(sssp, S):
+    """Weights 1 and 2: most vertices have many predecessors of one distance, whose labels several warps lower
+    while others read the packed words; the least label wins each time."""
+    rng = np.random.default_rng(80 + S)
+    V, E = 60011, 20 * 60011
+    src, dst, w = graph(rng, V, E, hi=2)
+    w0 = w + np.where((src < 9000) & (rng.random(E) < 0.05), 2, 0).astype(np.uint32)
+    ref = oracle.csr(V, src, dst, w)
+    g = sssp.build_csr(V, src, dst, w, partitions=5)
+    sources = rng.integers(0, V, S).astype(np.uint32)
+    want = [oracle.dijkstra(ref, int(s)) for s in sources]
+    dist0, pred0 = sssp.solve(sssp.build_csr(V, src, dst, w0, partitions=5), sources)[:2]
+    for _ in range(10):
+        dist, pred, st, stats = sssp.update(g, dist0.clone(), pred0.clone(), np.arange(17000, dtype=np.uint32))
+        assert st == 0 and stats["remote_activations"] == 0  # (swept)
+        for i, (d, p, _) in enumerate(want):
+            assert np.array_equal(u32(dist[i]), d) and np.array_equal(u32(pred[i]), p)
