@@ -348,7 +348,8 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
             x.n_tails = n_tails;
             x.dist = reinterpret_cast<uint32_t*>(l.packed);
             x.mark = l.dist;
-            x.list[0] = l.dist + (x.items + 31u) / 32u;
+            x.over = x.mark + (x.items + 31u) / 32u;
+            x.list[0] = x.over + (x.items + 31u) / 32u;
             const uint32_t cap = (uint32_t)std::min<size_t>((l.dist + (size_t)S * g->V - x.list[0]) / 2, x.items);
             x.list[1] = x.list[0] + cap;
             x.capM = cap / 4u;

@@ -23,7 +23,7 @@ struct WsHeader {
     uint32_t swept;         // the sweep finished: nothing is left for the persistent solve
     uint32_t lay_general;   // layout: the rows cannot be sorted segment by segment
     uint32_t unit_next;     // batch: next unit of the shared-memory kernel
-    uint32_t pad0;
+    uint32_t over;          // sweep: a candidate from a distance on the way did not fit
     unsigned long long begin;  // batch: time of its first block's start
     uint32_t pad[(256 - 4 - 4 - 8 - 8 - 72 - 24) / 4];
 };

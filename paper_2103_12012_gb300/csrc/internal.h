@@ -57,6 +57,7 @@ struct SweepLaunch {
 struct WarmLaunch : SweepLaunch {
     const uint32_t* tails;  // [n_tails] caller's ids
     uint32_t n_tails;
+    uint32_t* over;         // [items] bits: a candidate from the item did not fit
     uint32_t capA, capM;    // items that a list holds of either kind
 };
 

@@ -1053,14 +1053,15 @@ __global__ void k_seed(SolveLaunch L) {
 template <class W>
 __global__ void k_warm_pack(size_t n, uint32_t V, const uint32_t* __restrict__ slots,
                             const uint32_t* __restrict__ dist, const uint32_t* __restrict__ pred,
-                            unsigned long long* __restrict__ packed, const uint32_t* done) {
-    if (done && *done) return;
+                            unsigned long long* __restrict__ packed, const WsHeader* sweep, bool warm) {
+    if (sweep && sweep->swept) return;
+    const bool again = sweep && !warm && sweep->over;  // (from the start: see k_sweep_requeue)
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const size_t s = i / V, j = i - s * V;
         const size_t at = s * V + (slots ? __ldg(&slots[j]) : j);
         const uint32_t d = dist[i];
-        packed[at] = d == W::inf_out() ? INF_KEY : ((unsigned long long)d << 32) | (pred ? pred[i] : NONE);
+        packed[at] = d == W::inf_out() || (again && d) ? INF_KEY : ((unsigned long long)d << 32) | (pred ? pred[i] : NONE);
     }
 }
 
@@ -1427,16 +1428,16 @@ cudaError_t launch_solve(const SolveLaunch& L, const SweepLaunch* sweep, cudaStr
                     return e;
             }
             if (L.wtype == SSSP_W_F32)
-                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, done);
+                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, L.hdr, L.warm);
             else
-                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, done);
+                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, L.hdr, L.warm);
         } else if (L.warm) {
             if ((e = cudaMemsetAsync(L.bitmap, 0, 4 * n_words, st)) != cudaSuccess) return e;
             if ((e = cudaMemsetAsync(L.dirty, 0, 4 * n_dirty, st)) != cudaSuccess) return e;
             if (L.wtype == SSSP_W_F32)
-                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, nullptr);
+                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, nullptr, true);
             else
-                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, nullptr);
+                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, nullptr, true);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             const size_t nt = (size_t)L.S * L.n_tails;
             const unsigned tb = (unsigned)std::min<size_t>(std::max<size_t>((nt + 255) / 256, 1), (size_t)sms * 8);

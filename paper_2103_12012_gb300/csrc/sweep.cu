@@ -407,7 +407,13 @@ struct Worker {
                 } else {
                     const uint4 rw = wm.row[b[j]];
                     uint32_t z;
-                    if (!W::add(rw.z, y[j], z)) bad |= 2u;
+                    if (!W::add(rw.z, y[j], z)) {  // (judged at the end: k_sweep_requeue)
+                        bad |= 2u;
+                        if constexpr (WARM) {
+                            const uint32_t tail = rw.y + (L.slots ? __ldg(&L.slots[rw.w]) : rw.w);
+                            atomicOr(&L.over[tail >> 5], 1u << (tail & 31u));
+                        }
+                    }
                     x[j] += rw.y;
                     if constexpr (WARM)
                         load_keys<G>(L.dist, x[j], pr[j], d[j]);
@@ -691,7 +697,7 @@ __global__ void __launch_bounds__(WT, 2) k_sweep(Launch L) {
             if (wk.s_imp) atomicAdd(&bm.imp, (unsigned long long)wk.s_imp);
             if (wm.edges != before) atomicAdd(&bm.work, wm.edges - before);
             if (wk.bad & 1u) set_status(L.hdr, SSSP_EINVAL);
-            if (wk.bad & 2u) set_status(L.hdr, SSSP_EOVERFLOW);
+            if (wk.bad & 2u) st_relaxed(&L.hdr->over, 1u);
         }
         wk.flush_block();
         if (tid == 0 && bm.work) {
@@ -831,13 +837,52 @@ __global__ void k_warm_out(WarmLaunch L) {
     }
 }
 
+// SSSP_EOVERFLOW if a candidate from an item's final distances does not fit: of all items, or (warm start) of
+// those the sweep noted one of.  One warp per item.
+template <class W, int G, class Launch>
+__device__ __noinline__ void judge_overflow(const Launch& L) {
+    constexpr bool WARM = std::is_same<Launch, WarmLaunch>::value;
+    const uint32_t lane = threadIdx.x & 31u;
+    for (size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < L.items; i += (size_t)gridDim.x * blockDim.x >> 5) {
+        if constexpr (WARM)
+            if (!(L.over[i >> 5] >> (i & 31u) & 1u)) continue;
+        uint32_t most = 0;
+        bool reached = false;
+#pragma unroll
+        for (int s = 0; s < G; ++s) {
+            const uint32_t d = L.dist[WARM ? 2 * (i * G + s) + 1 : i * G + s];
+            if (d < L.inf) reached = true, most = max(most, d);
+        }
+        if (!reached) continue;
+        const uint32_t v = (uint32_t)(i % L.V), end = L.row_ptr[v + 1];
+        bool bad = false;
+        for (uint32_t e = L.row_ptr[v] + lane; e < end; e += 32u) {
+            uint32_t z;
+            bad = bad || (L.col[e] < L.V && W::weight_ok(L.w[e]) && !W::add(most, L.w[e], z));
+        }
+        if (bad) set_status(L.hdr, SSSP_EOVERFLOW);
+    }
+}
+
 // Handed over: the marked vertices become inbox bits of the sources that have reached them, their
 // units' doorbells are rung and they are counted.  One thread per inbox word (G = 1: the marks are
 // the inbox words already).
+// The sweep relaxes vertices at distances far above their final ones, as a solve in bucket order hardly does, so
+// a candidate of its that does not fit says nothing yet.  If it has met one and has finished, the final distances
+// are judged here; if it is handed over, the persistent solve starts again from the sources, as if
+// there had been no sweep (a warm start cannot: it queues the items in question once more).
 template <int G, class Launch>
 __global__ void k_sweep_requeue(Launch L, uint32_t* bitmap, uint32_t words, uint32_t B, uint32_t Bq, uint32_t split,
                                 uint32_t Q) {
-    if (L.hdr->swept) return;
+    constexpr bool WARM = std::is_same<Launch, WarmLaunch>::value;
+    const bool over = L.hdr->over;
+    if (L.hdr->swept) {
+        if (over && L.wtype == SSSP_W_F32)
+            judge_overflow<WF32, G>(L);
+        else if (over)
+            judge_overflow<WU32, G>(L);
+        return;
+    }
     const size_t n = (size_t)L.S * words, stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const uint32_t s = (uint32_t)(i / words), wd = (uint32_t)(i - (size_t)s * words);
@@ -845,8 +890,12 @@ __global__ void k_sweep_requeue(Launch L, uint32_t* bitmap, uint32_t words, uint
         for (uint32_t j = 0; j < 32u && wd * 32u + j < L.V; ++j) {
             const uint32_t item = s / G * L.V + wd * 32u + j;
             size_t d = (size_t)item * G + s % G;
-            if (std::is_same<Launch, WarmLaunch>::value) d = 2 * d + 1;
-            if ((L.mark[item >> 5] >> (item & 31u) & 1u) && L.dist[d] < L.inf) bits |= 1u << j;
+            uint32_t m = L.mark[item >> 5];
+            if constexpr (WARM) {
+                d = 2 * d + 1;
+                m |= L.over[item >> 5];
+            }
+            if (!WARM && over ? L.dist[d] == 0u : (m >> (item & 31u) & 1u) && L.dist[d] < L.inf) bits |= 1u << j;
         }
         bitmap[i] = bits;
         if (!bits) continue;
@@ -915,7 +964,7 @@ cudaError_t launch_warm_sweep(const WarmLaunch& L, int sms, cudaStream_t st) {
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     // (the previous result has been read: its place holds the marks and the lists)
-    if ((e = cudaMemsetAsync(L.mark, 0, 4 * (((size_t)L.items + 31) / 32), st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(L.mark, 0, 8 * (((size_t)L.items + 31) / 32), st)) != cudaSuccess) return e;  // (and over)
     const void* k = L.wtype == SSSP_W_F32 ? sweep_kernel<WF32, WarmLaunch>(L.G) : sweep_kernel<WU32, WarmLaunch>(L.G);
     void* args[] = {const_cast<WarmLaunch*>(&L)};
     return cudaLaunchCooperativeKernel(k, dim3(L.grid), dim3(WT), args, sweep_smem(L.G), st);

@@ -263,3 +263,119 @@ def test_warm_ties_under_contention(sssp, S):
         assert st == 0 and stats["remote_activations"] == 0  # (swept)
         for i, (d, p, _) in enumerate(want):
             assert np.array_equal(u32(dist[i]), d) and np.array_equal(u32(pred[i]), p)
+
+
+def fits(ref, sources):
+    """Every candidate from a final distance can be represented (else the status is SSSP_EOVERFLOW)."""
+    tail = np.repeat(np.arange(ref.row_ptr.size - 1), np.diff(ref.row_ptr.astype(np.int64)))
+    for s in sources:
+        d = oracle.dijkstra(ref, int(s))[0]
+        if ref.w.dtype == np.float32:
+            d, w = d.view(np.float32), ref.w
+            on = np.isfinite(d[tail])
+            with np.errstate(over="ignore"):
+                c, top = d[tail][on] + w[on], np.float32(np.inf)
+        else:
+            on = d[tail] != 0xFFFFFFFF
+            c, top = d[tail][on].astype(np.uint64) + ref.w[on], 0xFFFFFFFF
+        if (c >= top).any():
+            return False
+    return True
+
+
+@pytest.mark.parametrize("S", [1, 2, 4, 9])
+@pytest.mark.parametrize("f32", [False, True])
+def test_overflow_is_of_final_distances(sssp, S, f32):
+    """Weights up to a quarter of the range: distances on the way are past its end, final ones not; then one
+    edge from a reached vertex whose final candidate is."""
+    rng = np.random.default_rng(90 + S)
+    V = 16384
+    src, dst, w = graph(rng, V, 8 * V, hi=(1 << 30) - 1)
+    if f32:
+        w = (w * 8e28).astype(np.float32)
+    sources = rng.integers(0, V, S)
+    ref = oracle.csr(V, src, dst, w)
+    assert fits(ref, sources)
+    stats = check(sssp, sssp.build_csr(V, src, dst, w, partitions=5), ref, sources.tolist())
+    assert stats["remote_activations"] == 0  # (swept)
+    u = int(oracle.dijkstra(ref, int(sources[0]))[0].view(np.float32 if f32 else np.uint32).argsort()[V // 2])
+    w[np.nonzero(src == u)[0][0]] = np.float32(3.4e38) if f32 else 0xFFFFFFFE
+    ref = oracle.csr(V, src, dst, w)
+    assert not fits(ref, sources)
+    check(sssp, sssp.build_csr(V, src, dst, w, partitions=5), ref, sources.tolist(), status=sssp.SSSP_EOVERFLOW)
+
+
+@pytest.mark.parametrize("S", [1, 3, 8])
+@pytest.mark.parametrize("final", [False, True])
+def test_overflow_when_handed_over(sssp, S, final):
+    """A band graph, which the persistent solve finishes.  A long cut makes candidates on the way that do not
+    fit; or a vertex that the sweep is done with has one."""
+    rng = np.random.default_rng(6)
+    V = 30000
+    v = np.repeat(np.arange(V), 7)
+    t = v + np.tile(np.arange(1, 8), V)
+    keep = t < V
+    src = np.concatenate([v[keep], t[keep], [0]]).astype(np.uint32)
+    dst = np.concatenate([t[keep], v[keep], [15000]]).astype(np.uint32)
+    w = rng.integers(1, 50, src.size).astype(np.uint32)
+    w[-1] = 3000000000
+    w[(src == 15000) & (dst == 15001)] = 2000000000
+    if final:
+        w[(src == 12) & (dst == 13)] = 0xFFFFFFFE
+    sources = [0, 3, 1, 2, 4, 5, 6, 7][:S]
+    ref = oracle.csr(V, src, dst, w)
+    assert fits(ref, sources) == (not final)
+    check(sssp, sssp.build_csr(V, src, dst, w), ref, sources, status=sssp.SSSP_EOVERFLOW if final else 0)
+
+
+@pytest.mark.parametrize("S", [1, 2, 4])
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("kind", ["on the way", "final", "not touched"])
+def test_overflow_in_a_warm_start(sssp, S, f32, kind):
+    """The changed edges' heads get distances that a shorter way replaces; one vertex that is reached anew has
+    a candidate that does not fit; or one that the change does not reach."""
+    rng = np.random.default_rng(95 + S)
+    V = 60011
+    dt, unit = (np.float32, 1e38) if f32 else (np.uint32, 1200000000)  # (3 units fit, 4 do not)
+    src, dst, w = graph(rng, V, 8 * V, f32)
+    keep = (dst >= 10) & (src >= 10)
+    extra = [(0, 1, 3), (0, 2, 1), (2, 1, 1), (1, 3, 3 if kind == "final" else 1), (0, 20, 1 / unit), (0, 6, 2)]
+    if kind == "not touched":
+        extra.append((6, 9, 3))
+    src = np.concatenate([src[keep], [a for a, _, _ in extra]]).astype(np.uint32)
+    dst = np.concatenate([dst[keep], [b for _, b, _ in extra]]).astype(np.uint32)
+    w = np.concatenate([w[keep], [c * unit for _, _, c in extra]]).astype(dt)
+    before = ~((src == 0) & (dst < 3))  # the edges 0 -> 1 and 0 -> 2 are added
+    sources = np.zeros(S, np.uint32)
+    dist, pred = sssp.solve(sssp.build_csr(V, src[before], dst[before], w[before], partitions=5), sources, check=False)[:2]
+    ref = oracle.csr(V, src, dst, w)
+    assert fits(ref, sources) == (kind == "on the way")
+    dist, pred, st, stats = sssp.update(sssp.build_csr(V, src, dst, w, partitions=5), dist, pred,
+                                        np.zeros(17000, np.uint32), check=False)
+    assert stats["remote_activations"] == 0  # (swept)
+    assert st == (sssp.SSSP_EOVERFLOW if kind == "final" else 0)
+    d, p, _ = oracle.dijkstra(ref, 0)
+    for i in range(S):
+        assert np.array_equal(u32(dist[i]), d.view(np.uint32)) and np.array_equal(u32(pred[i]), p)
+
+
+@pytest.mark.parametrize("S", [1, 4])
+def test_overflow_in_a_warm_start_that_is_handed_over(sssp, S):
+    """An item of the first iterations has a candidate that does not fit; the persistent solve finishes."""
+    rng = np.random.default_rng(S)
+    V = 20000
+    src = np.repeat(np.arange(V - 6), 6).astype(np.uint32)
+    dst = src + np.tile(np.arange(1, 7), V - 6).astype(np.uint32)
+    w = rng.integers(50, 60, src.size).astype(np.uint32)
+    src, dst, w = np.append(src, 9).astype(np.uint32), np.append(dst, 900).astype(np.uint32), np.append(w, np.uint32(0xFFFFFFFE))
+    w2 = w.copy()
+    w2[:12] = 1
+    sources = np.arange(S).astype(np.uint32)
+    dist, pred = sssp.solve(sssp.build_csr(V, src, dst, w), sources, check=False)[:2]
+    dist, pred, st, _ = sssp.update(sssp.build_csr(V, src, dst, w2), dist, pred,
+                                    np.concatenate([src[:12], np.full(20000, V - 1, np.uint32)]), check=False)
+    assert st == sssp.SSSP_EOVERFLOW
+    ref = oracle.csr(V, src, dst, w2)
+    for i, s in enumerate(sources):
+        d, p, _ = oracle.dijkstra(ref, int(s))
+        assert np.array_equal(u32(dist[i]), d) and np.array_equal(u32(pred[i]), p)
