@@ -39,8 +39,9 @@
  *  - uint32 distances: a candidate d(u)+w that does not fit below 0xFFFFFFFF
  *    is discarded and the status becomes SSSP_EOVERFLOW; vertices whose true
  *    distance does not fit are then reported unreachable.  A swept solve
- *    (sssp_solve) counts the candidates from final distances only; the
- *    persistent solve also one from a distance that a later one replaced.
+ *    (sssp_solve) and a batch in shared memory count the candidates from
+ *    final distances only; the others also one from a distance that a
+ *    later one replaced.
  */
 #ifndef SSSP_H
 #define SSSP_H

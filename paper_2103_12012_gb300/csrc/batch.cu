@@ -230,6 +230,29 @@ struct Round {
     }
 };
 
+// SSSP_EOVERFLOW if a candidate from a final distance does not fit.  (One that was met on the way may be from
+// a distance that was lowered later: more of them than in the general kernel, whose buckets are narrower.)
+// Inlined: a call's stack costs the launch 13 us.
+template <class W>
+__device__ __forceinline__ void judge_overflow(const uint32_t* dist, uint32_t V, uint32_t S, const uint32_t* row_ptr,
+                                            const uint32_t* col, const uint32_t* w, WsHeader* hdr) {
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t u = threadIdx.x >> 5; u < V; u += blockDim.x >> 5) {
+        uint32_t most = 0;
+        bool reached = false, bad = false;
+        for (uint32_t s = 0; s < S; ++s) {
+            const uint32_t d = dist[s * V + u];
+            if (d < W::inf_out()) reached = true, most = max(most, d);
+        }
+        if (!reached) continue;
+        for (uint32_t e = row_ptr[u] + lane; e < row_ptr[u + 1u]; e += 32u) {
+            uint32_t z;
+            bad = bad || (col[e] < V && W::weight_ok(w[e]) && !W::add(most, w[e], z));
+        }
+        if (bad) set_status(hdr, SSSP_EOVERFLOW);
+    }
+}
+
 // One unit, by the block.
 template <class W, uint32_t BT>
 __device__ __forceinline__ void solve_unit(const BatchSmem& B, Mem<BT / 32>& M, uint32_t* dsm, uint64_t deadline) {
@@ -292,7 +315,7 @@ __device__ __forceinline__ void solve_unit(const BatchSmem& B, Mem<BT / 32>& M, 
             B.dist[U.out[s] + v] = I.dist[s * V + v];
             if (B.pred) B.pred[U.out[s] + v] = NONE;
         }
-    __syncthreads();
+    const bool over = __syncthreads_or((int)(R.bad & 2u));
     if (B.pred && !stopped) {
         uint32_t* const rows = reinterpret_cast<uint32_t*>(M.row[wid]);
         RowWalk walk{R.row_ptr, V, rows, rows + 32};
@@ -327,11 +350,8 @@ __device__ __forceinline__ void solve_unit(const BatchSmem& B, Mem<BT / 32>& M, 
             }
         }
     }
-    R.bad = __reduce_or_sync(0xFFFFFFFFu, R.bad);
-    if (lane == 0) {
-        if (R.bad & 1u) set_status(B.hdr, SSSP_EINVAL);
-        if (R.bad & 2u) set_status(B.hdr, SSSP_EOVERFLOW);
-    }
+    if (__any_sync(0xFFFFFFFFu, R.bad & 1u) && lane == 0) set_status(B.hdr, SSSP_EINVAL);
+    if (over && !stopped) judge_overflow<W>(I.dist, V, S, R.row_ptr, R.col, R.w, B.hdr);
     // edges_scanned, atomics, improved, activations (but for the sources, an item is relaxed as often as
     // it is marked), rounds, vertices
     R.n_at = __reduce_add_sync(0xFFFFFFFFu, R.n_at);

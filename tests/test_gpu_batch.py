@@ -168,3 +168,29 @@ def test_bad_edges_are_reported(sssp, V, what):
     b = sssp.Batch([g], [[17, int(rng.integers(100, V)), 5]], sssp.options(delta=16.0))
     b.solve()
     assert b.status()[0] == (sssp.SSSP_EOVERFLOW if what == "overflow" else sssp.SSSP_EINVAL)
+
+
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("preds", [False, True])
+@pytest.mark.parametrize("V", [2000, 40000])
+def test_overflow_is_of_final_distances(sssp, V, preds, f32):
+    """1 is lowered within a bucket, after it has been relaxed; its candidate for 3 fits only then, or not at
+    all."""
+    rng = np.random.default_rng(V)
+    dt, unit, way, fits, not_fits = (np.float32, 1e38, 2.9, 1, 3) if f32 else (np.uint32, 1000000000, 2, 2.5, 4)
+    src, dst = rng.integers(10, V, (2, 4 * V)).astype(np.uint32)
+    w = rng.integers(1, 256, src.size)
+    for last in (fits, not_fits):
+        extra = [(0, 1, way), (0, 2, 0.5), (2, 1, 0.5), (1, 3, last), (0, 10, 1 / unit)]
+        g = oracle.csr(V, np.append(src, [a for a, _, _ in extra]).astype(np.uint32),
+                       np.append(dst, [b for _, b, _ in extra]).astype(np.uint32),
+                       np.append(w, [c * unit for _, _, c in extra]).astype(dt))
+        b = sssp.Batch([g], [[0, 10]], sssp.options(delta=unit))
+        if not preds:
+            b.c.pred = None
+        b.solve()
+        assert b.status()[0] == (0 if last == fits else sssp.SSSP_EOVERFLOW)
+        for i in range(2):
+            d, p, _ = oracle.dijkstra(g, 10 * i)
+            bd, bp = b.result(i)
+            assert np.array_equal(u32(bd), d.view(np.uint32)) and (not preds or np.array_equal(u32(bp), p))
