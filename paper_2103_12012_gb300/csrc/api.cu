@@ -51,6 +51,16 @@ uint32_t delta_bits_for(int wtype, double delta) {
     return (uint32_t)std::min(4294967294.0, std::max(1.0, std::floor(delta)));
 }
 
+// a bucket width times a small factor
+uint32_t times_delta(int wtype, uint32_t delta_bits, uint32_t times) {
+    if (wtype != SSSP_W_F32) return (uint32_t)std::min<uint64_t>((uint64_t)times * delta_bits, 0x7FFFFFFFu);
+    float f;
+    std::memcpy(&f, &delta_bits, 4);
+    f = std::min(f * (float)times, 3.0e38f);
+    std::memcpy(&delta_bits, &f, 4);
+    return delta_bits;
+}
+
 // bucket width of hubs: the round's over 2^shift (at least one unit for uint32 distances)
 uint32_t hub_delta_bits_for(int wtype, uint32_t delta_bits, int shift) {
     if (wtype == SSSP_W_F32) {
@@ -101,14 +111,15 @@ bool sweep_graph(const sssp_graph* g, uint32_t S) {
            groups * g->E < 0xF0000000ull;
 }
 
-// Workspace of sssp_solve: header | counters of the sweep | packed[S][V] | bitmap[S][words] | hub
-// entries[2] of the sweep | dirty[S*Q] | nfsplit[S*Q].  The sweep keeps dist[items][G] at the start
-// of packed.  For S > 1 its marks are in the rest of packed and its lists in the caller's dist array
-// (written only at the end); for S = 1 its marks are the bitmap, one list is the rest of packed and
-// the other the caller's dist.  A warm start keeps rows of packed words in packed, and marks and lists
-// in the caller's dist (read at the start, written at the end).
+// Workspace of sssp_solve: header | packed[S][V] | bitmap[S][words] | dirty[S*Q] | nfsplit[S*Q], then
+// what the sweep has besides: counters | hub entries[2].  (Behind them, the doorbells made the persistent solve up to
+// a fifth slower: random graph, 89,656 vertices, 4 sources, 69 partitions, 0.71 and 0.84 ms.)  The sweep
+// keeps dist[items][G] at the start of packed.  For S > 1 its marks are in the rest of packed and its lists in the
+// caller's dist array (written only at the end); for S = 1 its marks are the bitmap, one list is the rest of packed
+// and the other the caller's dist.  A warm start keeps rows of packed words in packed, and marks and lists in the
+// caller's dist (read at the start, written at the end).
 struct SolveWs {
-    size_t off_ctl, off_packed, off_bitmap, off_ex, ex_bytes, off_dirty, off_nf, total;
+    size_t off_packed, off_bitmap, off_dirty, off_nf, off_ctl, off_ex, ex_bytes, total;
     uint32_t words, B, Bq, Q;
     bool sweep;
 };
@@ -121,36 +132,65 @@ SolveWs solve_layout(const sssp_graph* g, uint32_t S, uint32_t split, bool sweep
     w.Bq = (w.B + split - 1u) / split;
     w.Q = g->partitions * split;
     size_t off = WS_HEADER_BYTES;
-    w.off_ctl = off;
-    if (w.sweep) off += align_up(sizeof(SweepCtl), 256);
     w.off_packed = off;
     off += align_up(8ull * S * g->V, 256);
     w.off_bitmap = off;
     off += align_up(4ull * S * w.words, 256);
-    w.off_ex = off;
-    w.ex_bytes = 8ull * ((uint64_t)S * g->E / SWEEP_HUB + 1);
-    if (w.sweep) off += align_up(2 * w.ex_bytes, 256);
     w.off_dirty = off;
     off += align_up(4ull * S * w.Q, 256);
     w.off_nf = off;
     off += align_up(4ull * S * w.Q, 256);
+    if (w.sweep) {
+        w.off_ctl = off;
+        off += align_up(sizeof(SweepCtl), 256);
+        w.off_ex = off;
+        w.ex_bytes = 8ull * ((uint64_t)S * g->E / SWEEP_HUB + 1);
+        off += align_up(2 * w.ex_bytes, 256);
+    }
     w.total = off;
     return w;
 }
 
-// Whether the sweep is the faster one (ms, uint32 weights; V, edges per vertex, P, S, given width):
-//   5 sources or more share rows: R-MAT 4.2 M, 16, 148, 8, tuned: 4.1 against 7.5; 1 M, 16, 148, 16:
-//     2.1 / 6.8; ER 262144, 16, 148, 16, default: 1.7 / 5.4; but ER 256, 16, 32, 16: 0.23 / 0.17
-//   few blocks (units) for the persistent solve: ER 16384, 8, 4, 1, default: 0.24 / 1.6; R-MAT 1 M,
-//     16, 4, 1: 0.6 / 35
-//   small sub-blocks make its rounds cheap: ER 4096, 40, 148, 4 (28 vertices each): 0.29 / 0.24,
-//     R-MAT 1024, 16, 148, 4: 0.21 / 0.14
-//   1 to 4 sources, many units and a given (tuned) width, on graphs without hubs: ER 1 M, 16, 148, 4:
-//     2.3 / 1.8, ER 16384, 16, 148, 1: 0.29 / 0.26; with hubs (those that are worth a layout) R-MAT
-//     1 M, 16, 148, 1: 0.6 / 1.2
+// Whether the sweep is the faster one, on random (ER) and power-law (R-MAT) graphs (ms, persistent / sweep, uint32
+// weights; V, edges per vertex, P, S, given width).  At the default width nearly always: ER 16,384, 8, 4, 1: 1.6 /
+// 0.31; 64, 6, 1, 1: 0.34 / 0.11; 8,192, 6, 148, 8: 0.84 / 0.28.  A given (tuned) width makes the persistent solve
+// several times faster, and then the sweep wins
+//   over units of many vertices, more of them the more sources share a row: ER 4,096, 12, 4, 1: 0.31 / 0.19;
+//     R-MAT 65,536, 15, 64, 5: 1.4 times; but R-MAT 8,192, 6, 16, 8, float32: 0.14 / 0.20
+//   over more units than the persistent solve has blocks: R-MAT 4.2 M, 16, 148, 8: 7.2 / 4.0; but ER 1 M, 13, 100,
+//     5 (500 units): 1.5 / 1.9; R-MAT has hubs, and a layout if they are large: 400,000, 16, 64, 5: 1.4 / 0.9
+//   with 1 to 4 sources over many units, only on graphs with hubs: ER 1 M, 16, 148, 4: 1.8 / 2.3; R-MAT 1 M, 16,
+//     148, 1: 1.2 / 0.6
 bool sweep_wins(const sssp_graph* g, uint32_t S, const SolveWs& L, bool delta_given) {
-    if (S >= 5) return g->V >= 2048 || L.Bq >= 64;
-    return L.Bq >= 64 && (!delta_given || g->ids || (uint64_t)S * L.Q < 128);
+    const uint64_t units = (uint64_t)S * L.Q;
+    if (!delta_given) return L.Bq >= 64 || (S >= 5 && g->V >= 2048);
+    if (S < 5) return L.Bq >= 256u * (S + 1u) && (g->ids || units < 128);
+    if (units >= 608) return g->V >= 16384;
+    return (g->ids || units < 256) && L.Bq >= (g->V >= 32768 ? 512u : S >= 7 ? 2048u : 256u * (S + 1u));
+}
+
+// When a sweep stops after its first iterations, in favour of the persistent solve, which then starts from the
+// sources.  On a graph of many hops the sweep's iterations (10 us and more) are as many as the hops and half as
+// many again, and it relaxes an edge several times.
+//   few: such a graph has relaxed less after five iterations than D^4 edges a source (D edges per vertex) or than it
+//     has in all.  Measured on the CPU, per source: 3-D lattices of 6 neighbours 450 to 860 (D^4 1,055 to 1,210), grids of
+//     8 and 24 980 and 11,400 (4,000 and 320,000), rings with short cuts 700; random graphs of 5 and 8 edges 1,400
+//     and more and 14,700 (730 and 4,070), R-MAT from 12,000 on.
+//   narrow: the sweep goes on all the same where the persistent solve is far slower: one source with
+//     65,536 vertices a unit (lattice of 100^3, 4 partitions, width 64: 33 / 2.7 ms), or few units at the default width,
+//     if that is narrow, most weights being above 8 times the width (lattice of 64^3, 4 partitions, 4 sources: 32 / 2.8
+//     ms; with all weights 1 2.7 / 2.8).
+// Else the sweep has cost 0.06 ms: lattice of 100^3, 148 partitions, 8 sources, width 64 8.3 / 8.4 ms (14.1 when it was
+// handed over late), grid of 1000^2 with 24 neighbours 14.0 / 14.2 (47.7), lattice of 20^3, 4 partitions, 1 source 0.42 /
+// 0.47.
+void sweep_keeps(const sssp_graph* g, uint32_t S, const SolveWs& L, const Resolved& r, SweepLaunch* x) {
+    const double D = (double)g->E / g->V;
+    x->few = (unsigned long long)std::min(D * D * D * D * S, (double)g->E);
+    x->narrow = 0xFFFFFFFFu;
+    if (S == 1 && L.Bq >= 65536)
+        x->narrow = 0u;
+    else if (!r.delta_given && (S == 1 || (uint64_t)S * L.Q < 128))
+        x->narrow = times_delta(g->wtype, r.delta_bits, 8);
 }
 
 // A warm start by the sweep: from about ten thousand tails on its passes over the vertices and its grid
@@ -263,12 +303,9 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
     if (smem > 200 * 1024) return SSSP_EINVAL;
     const bool prune = prune_mode >= 0;
     // The sweep takes solves in the default policy (the others ask for a schedule of the persistent solve).
-    // The persistent solve alone keeps its own, tighter layout: behind a gap, 276 doorbells made a solve of
-    // 0.71 ms (random graph, 89,656 vertices, 4 sources, 69 partitions) one of 0.84.
     const bool sweep =
         L.sweep && !persistent && !prune && r.policy == SSSP_POLICY_RELATIVE && r.msg_buffer == 0 && !(r.flags & SSSP_FLAG_TEST_HOLD_PENDING) &&
         (warm ? warm_sweep_wins(S, n_tails, static_cast<char*>(ws) + L.off_packed) : sweep_wins(g, S, L, r.delta_given));
-    if (!sweep) L = solve_layout(g, S, r.split, false);
     int per_sm = 0;
     const uint32_t hubs = g->ids ? std::min(r.hub_count, L.B) : 0u;  // layout graphs only
     if (relax_max_blocks_per_sm(g->wtype, r.threads, r.tile, L.Q, &per_sm, prune, r.msg_buffer != 0, hubs != 0) !=
@@ -364,6 +401,7 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
         x.pred = pred;
         x.inf = g->wtype == SSSP_W_F32 ? F32_INF_BITS : INF32;
         x.timeout_ns = r.timeout_ns;
+        sweep_keeps(g, S, L, r, &x);
         if (sweep_max_blocks_per_sm(g->wtype, x.G, warm, &per_sm) != cudaSuccess) return SSSP_ECUDA;
         if (r.bps) per_sm = std::min<int>(per_sm, (int)r.bps);
         x.grid = (uint32_t)std::min<uint64_t>((uint64_t)std::max(per_sm, 0) * sm_count(),
@@ -610,18 +648,6 @@ sssp_status sssp_shard_problems(uint32_t n_problems, const uint64_t* cost, uint3
 
 namespace {
 
-// Bucket width of the shared-memory kernel: three times the one given, which suits the general kernel (in
-// shared memory an edge costs less and a round more: 220 graphs of 1,024 to 8,192 vertices, 16 sources each, 2.20
-// ms at the given width and 1.83 at three times it, 146 of 8,192 to 32,768 4.85 and 4.10).
-uint32_t wide_delta(int wtype, uint32_t delta_bits) {
-    if (wtype != SSSP_W_F32) return (uint32_t)std::min<uint64_t>(3ull * delta_bits, 0x7FFFFFFFu);
-    float f;
-    std::memcpy(&f, &delta_bits, 4);
-    f = std::min(f * 3.0f, 3.0e38f);
-    std::memcpy(&delta_bits, &f, 4);
-    return delta_bits;
-}
-
 struct BatchTables {
     std::vector<BatchProblem> probs;  // in processing order
     std::vector<BatchUnit> units;     // groups of those that shared memory takes
@@ -781,7 +807,10 @@ sssp_status prepare_batch(const sssp_batch* b, const sssp_options* opt, void* ws
     x->col = l->col;
     x->w = l->w;
     x->wtype = l->wtype;
-    x->delta_bits = wide_delta(b->wtype, l->delta_bits);
+    // Buckets of the shared-memory kernel are three times as wide as given, which suits the general kernel (in
+    // shared memory an edge costs less and a round more: 220 graphs of 1,024 to 8,192 vertices, 16 sources each,
+    // 2.20 ms at the given width and 1.83 at three times it, 146 of 8,192 to 32,768 4.85 and 4.10).
+    x->delta_bits = times_delta(b->wtype, l->delta_bits, 3);
     x->units = reinterpret_cast<const BatchUnit*>(base + L.off_units);
     x->n_units = (uint32_t)t.units.size();
     for (const BatchUnit& u : t.units) x->items = std::max(x->items, u.S * u.V);

@@ -20,7 +20,7 @@ struct WsHeader {
     unsigned long long pending;  // queued-but-unprocessed vertices (Sec. III.D counter)
     unsigned long long work_next;  // batched work-queue cursor
     unsigned long long stats[9];   // sssp_stats
-    uint32_t swept;         // the sweep finished: nothing is left for the persistent solve
+    uint32_t swept;         // sweep: SWEPT_*
     uint32_t lay_general;   // layout: the rows cannot be sorted segment by segment
     uint32_t unit_next;     // batch: next unit of the shared-memory kernel
     uint32_t over;          // sweep: a candidate from a distance on the way did not fit

@@ -15,13 +15,16 @@ struct WsHeader;
 // ------------------------------------------------------------------ sweep.cu
 constexpr uint32_t SWEEP_HUB = 512;  // rows of at least this many edges are cut into segments
 
+// WsHeader::swept: the persistent solve goes on from what the sweep left, has nothing to do, starts from the sources
+constexpr uint32_t SWEPT_HANDED = 0, SWEPT_DONE = 1, SWEPT_AGAIN = 2;
+
 struct SweepIter {            // counters of one iteration
     uint32_t nA, nM;          // items in list A (from the front) and list M (from the back)
     unsigned long long ex;    // hubs << 32 | their segments
     unsigned long long work;  // relaxations of the iteration before
     uint32_t stop, pad[25];   // (warm) a list was full
 };
-struct SweepCtl {  // zero before the launch
+struct SweepCtl {
     uint32_t bar, pad[31];
     SweepIter it[3];
 };
@@ -50,6 +53,8 @@ struct SweepLaunch {
     uint32_t inf;
     uint64_t timeout_ns;
     uint32_t grid;
+    unsigned long long few;  // fewer relaxations than this in the first iterations: a graph of many hops,
+    uint32_t narrow;         // which the sweep keeps if most weights are above `narrow`
 };
 
 // A warm start: out and pred hold a previous result, which is brought up to date.  The rows are of packed

@@ -1053,15 +1053,20 @@ __global__ void k_seed(SolveLaunch L) {
 template <class W>
 __global__ void k_warm_pack(size_t n, uint32_t V, const uint32_t* __restrict__ slots,
                             const uint32_t* __restrict__ dist, const uint32_t* __restrict__ pred,
-                            unsigned long long* __restrict__ packed, const WsHeader* sweep, bool warm) {
-    if (sweep && sweep->swept) return;
-    const bool again = sweep && !warm && sweep->over;  // (from the start: see k_sweep_requeue)
+                            unsigned long long* __restrict__ packed, const WsHeader* sweep,
+                            const uint32_t* __restrict__ sources) {
+    if (sweep && sweep->swept == SWEPT_DONE) return;
+    const bool again = sweep && sources && (sweep->over || sweep->swept == SWEPT_AGAIN);  // (see k_sweep_requeue)
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         const size_t s = i / V, j = i - s * V;
         const size_t at = s * V + (slots ? __ldg(&slots[j]) : j);
+        if (again) {
+            packed[at] = j == __ldg(&sources[s]) ? SRC_KEY : INF_KEY;
+            continue;
+        }
         const uint32_t d = dist[i];
-        packed[at] = d == W::inf_out() || (again && d) ? INF_KEY : ((unsigned long long)d << 32) | (pred ? pred[i] : NONE);
+        packed[at] = d == W::inf_out() ? INF_KEY : ((unsigned long long)d << 32) | (pred ? pred[i] : NONE);
     }
 }
 
@@ -1097,7 +1102,7 @@ template <class W>
 __global__ void k_unpack(const unsigned long long* __restrict__ packed, size_t n, uint32_t V,
                          const uint32_t* __restrict__ slots, uint32_t* __restrict__ dist, uint32_t* __restrict__ pred,
                          const uint32_t* done) {
-    if (done && *done) return;
+    if (done && *done == SWEPT_DONE) return;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         size_t at = i;
@@ -1405,9 +1410,7 @@ cudaError_t launch_solve(const SolveLaunch& L, const SweepLaunch* sweep, cudaStr
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const uint32_t* const done = sweep ? &L.hdr->swept : nullptr;
-    const size_t hdr_bytes =  // (also the prune cursor; with the sweep its counters, which follow)
-        sweep ? (size_t)(reinterpret_cast<char*>(L.packed) - reinterpret_cast<char*>(L.hdr)) : WS_HEADER_BYTES;
-    if ((e = cudaMemsetAsync(L.hdr, 0, hdr_bytes, st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(L.hdr, 0, WS_HEADER_BYTES, st)) != cudaSuccess) return e;  // (also the prune cursor)
     if (!sweep && (e = cudaMemsetAsync(L.nfsplit, 0, 4 * n_dirty, st)) != cudaSuccess) return e;
     if (L.prune_on && (e = trishla_init(L.prune, st)) != cudaSuccess) return e;
     {
@@ -1428,16 +1431,18 @@ cudaError_t launch_solve(const SolveLaunch& L, const SweepLaunch* sweep, cudaStr
                     return e;
             }
             if (L.wtype == SSSP_W_F32)
-                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, L.hdr, L.warm);
+                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, L.hdr,
+                                                         L.warm ? nullptr : L.sources);
             else
-                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, L.hdr, L.warm);
+                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, L.hdr,
+                                                         L.warm ? nullptr : L.sources);
         } else if (L.warm) {
             if ((e = cudaMemsetAsync(L.bitmap, 0, 4 * n_words, st)) != cudaSuccess) return e;
             if ((e = cudaMemsetAsync(L.dirty, 0, 4 * n_dirty, st)) != cudaSuccess) return e;
             if (L.wtype == SSSP_W_F32)
-                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, nullptr, true);
+                k_warm_pack<WF32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, nullptr, nullptr);
             else
-                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, nullptr, true);
+                k_warm_pack<WU32><<<blocks, 256, 0, st>>>(n_packed, L.V, L.slots, L.dist, L.pred, L.packed, nullptr, nullptr);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             const size_t nt = (size_t)L.S * L.n_tails;
             const unsigned tb = (unsigned)std::min<size_t>(std::max<size_t>((nt + 255) / 256, 1), (size_t)sms * 8);

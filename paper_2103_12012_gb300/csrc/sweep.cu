@@ -34,8 +34,8 @@
 // packed words (up to four), so that predecessors come along and no pass over all edges is needed, and
 // the lists and marks take the caller's dist.  R-MAT, 1 M vertices, 15 M edges, 4 sources, 15,000 tails: 0.39 ->
 // 0.27 ms; k_sweep has 0.19 of it, most in the first iteration (the tails' rows are a third of the edges).
-// A graph that is not of that kind (tiny frontiers, many iterations, or many more relaxations than
-// edges) is handed over: marks become inbox bits, distances packed words, and k_solve goes on.
+// A graph of many hops is left to k_solve after a few iterations (api.cu says when), and so is a long tail: marks become
+// inbox bits, distances packed words, and k_solve goes on from them.
 // Waits: the grid barrier is bounded by the idle limit, the kernel by LIMIT_FACTOR times it.
 #include <algorithm>
 #include <type_traits>
@@ -54,11 +54,12 @@ constexpr uint32_t BUF = 64;                // a warp's buffer of newly marked i
 constexpr uint32_t MQ = 4, MARKS = MQ * 32;  // items a lane, a warp marks at a time
 constexpr uint32_t OUT_EDGES = 1024;        // most edges a warp of k_sweep_out takes
 constexpr uint64_t LIMIT_FACTOR = 3;
-// Hand-over, looked at every HAND_EVERY iterations: fewer than HAND_EDGES relaxations an iteration,
-// a pace that predicts more than HAND_ITERS iterations, or more than HAND_INFL relaxations per edge
-// and source (random and power-law graphs: 2 to 10).
 constexpr uint32_t WARM_ITERS = 32;  // a warm start is handed over
-constexpr uint32_t HAND_EVERY = 32, HAND_EDGES = 2048, HAND_ITERS = 1024, HAND_INFL = 24;
+// When a sweep stops.  At HOPS_ITERS: a graph of many hops (SweepLaunch::few), unless it is kept.  Every HAND_EVERY
+// iterations: a kept one at a pace that predicts more than HAND_ITERS iterations at the first look (a band of
+// 30,000 vertices, 7 a hop: 840 to 1,670; a lattice of 64^3: 170 to 290; a ring with short cuts: 320), later four times as
+// many; else a tail, fewer than HAND_EDGES relaxations an iteration.
+constexpr uint32_t HOPS_ITERS = 5, HAND_EVERY = 32, HAND_EDGES = 256, HAND_ITERS = 512;
 
 template <class W>
 struct Dist;
@@ -89,7 +90,11 @@ struct BlockMem {
     unsigned long long work, at, imp;
     uint32_t next;  // the block's next unit of work
     int ok;
+    // the iterations made, their relaxations, those at the last look, many hops and kept all the same; what is next
+    uint32_t iters, slow, then;
+    unsigned long long total, looked;
 };
+constexpr uint32_t GO_ON = ~0u, ASK = ~1u;  // BlockMem::then, or how the sweep ends (SWEPT_*)
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
     uint32_t v;
@@ -371,9 +376,11 @@ struct Worker {
     // (ascending, every row has an edge; lanes without a row: none), so the rows that start within
     // the 32 edges of a step are a bit mask, and a lane's row is the count of starts up to it.
     // A pipeline of three: the (col, w) of the steps after next, the distances of the next ones and
-    // the atomics of these are in flight together (EB steps each: eight distances a lane).
+    // the atomics of these are in flight together (EB steps each; four of them for one or two sources, or three, spill
+    // registers: R-MAT scale 18, 1 source 0.65 and 0.63 against 0.59 ms, scale 20, 2 sources 1.11 and 0.98
+    // against 0.93 ms).
     __device__ __forceinline__ void relax(uint32_t total, uint32_t p) {
-        constexpr int EB = G >= 8 || (WARM && G >= 4) ? 1 : G == 4 || (WARM && G == 2) ? 2 : 4;
+        constexpr int EB = G >= 8 || (WARM && G >= 4) ? 1 : 2;
         uint32_t v[EB], w[EB], a[EB];              // steps after next: head, weight, row
         uint32_t x[EB], y[EB], b[EB], d[EB][G];    // next steps: item, weight, row, its distances
         uint32_t pr[EB][WARM ? G : 1];             // (warm) and predecessors
@@ -572,7 +579,7 @@ struct Worker {
     }
 };
 
-// Every distance to INF, marks to zero, predecessors to NONE.
+// Every distance to INF, marks and counters to zero, predecessors to NONE.
 __global__ void k_sweep_init(SweepLaunch L, uint32_t inf) {
     const size_t stride = (size_t)gridDim.x * blockDim.x, i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t nd = (size_t)L.items * L.G;
@@ -580,9 +587,28 @@ __global__ void k_sweep_init(SweepLaunch L, uint32_t inf) {
     for (size_t i = i0; i < nd / 4; i += stride) d4[i] = make_uint4(inf, inf, inf, inf);
     if (i0 < (nd & 3u)) L.dist[(nd & ~(size_t)3) + i0] = inf;
     for (size_t i = i0; i < ((size_t)L.items + 31) / 32; i += stride) L.mark[i] = 0u;
+    for (size_t i = i0; i < sizeof(SweepCtl) / 4; i += stride) reinterpret_cast<uint32_t*>(L.ctl)[i] = 0u;
     for (size_t i = i0; i < L.n_dirty; i += stride) L.dirty[i] = 0u, L.nfsplit[i] = 0u;
     if (L.pred)
         for (size_t i = i0; i < (size_t)L.S * L.V; i += stride) L.pred[i] = NONE;
+}
+
+// What is next, from the counters of the iteration to come (one thread; the same answer in every block).
+template <class Launch>
+__device__ __forceinline__ uint32_t decide(const Launch& L, BlockMem& bm) {
+    constexpr bool WARM = std::is_same<Launch, WarmLaunch>::value;
+    if (!(bm.c[0] | bm.c[1] | bm.c[3])) return SWEPT_DONE;
+    if (WARM) return bm.c[6] || bm.iters == WARM_ITERS ? SWEPT_HANDED : GO_ON;
+    if (bm.iters == HOPS_ITERS && bm.total < L.few) return ASK;
+    if (bm.iters == 0u || bm.iters % HAND_EVERY != 0u) return GO_ON;
+    if (bm.slow) {
+        const float done = (float)bm.total / ((float)L.E * (float)L.S);
+        const uint32_t most = bm.iters == HAND_EVERY ? HAND_ITERS : 4u * HAND_ITERS;  // (those begun are finished)
+        return done * (float)most >= (float)bm.iters ? GO_ON : done < 1.0f ? SWEPT_AGAIN : SWEPT_HANDED;
+    }
+    if (bm.total - bm.looked < HAND_EVERY * HAND_EDGES) return SWEPT_HANDED;
+    bm.looked = bm.total;
+    return GO_ON;
 }
 
 template <class W, int G, class Launch>
@@ -595,7 +621,11 @@ __global__ void __launch_bounds__(WT, 2) k_sweep(Launch L) {
     WarpMem& wm = wmem[wid];
     const uint64_t t_begin = globaltimer_ns();
     uint32_t nbar = 0;
-    if (tid == 0) bm.work = bm.at = bm.imp = 0ull;
+    if (tid == 0) {
+        bm.work = bm.at = bm.imp = bm.total = bm.looked = 0ull;
+        bm.iters = bm.slow = 0u;
+        bm.then = SWEPT_HANDED;  // (a limit has run out)
+    }
     if (lane == 0) {
         wm.edges = 0ull;
         wm.act = wm.vert = 0u;
@@ -646,24 +676,26 @@ __global__ void __launch_bounds__(WT, 2) k_sweep(Launch L) {
             }
         }
     }
-    uint32_t slot = 0, par = 0, iters = 0;
-    unsigned long long work = 0;
-    const unsigned long long all = (unsigned long long)L.E * L.S;
-    bool done = false;
+    uint32_t slot = 0, par = 0;
     while (grid_barrier(L, bm, nbar, t_begin)) {
-        if (tid < 2u) {  // the counters of this iteration (nobody adds to them any more)
-            const uint4 x = __ldcg(reinterpret_cast<const uint4*>(&L.ctl->it[slot]) + tid);
+        if (tid == 0) {  // the counters of this iteration (nobody adds to them any more)
+            const uint4* const it = reinterpret_cast<const uint4*>(&L.ctl->it[slot]);
+            const uint4 x = __ldcg(it), y = __ldcg(it + 1);
             bm.next = 0u;
-            bm.c[tid * 4] = x.x, bm.c[tid * 4 + 1] = x.y, bm.c[tid * 4 + 2] = x.z, bm.c[tid * 4 + 3] = x.w;
+            bm.c[0] = x.x, bm.c[1] = x.y, bm.c[2] = x.z, bm.c[3] = x.w, bm.c[6] = y.z;
+            bm.total += ((unsigned long long)y.y << 32) | y.x;
+            bm.then = decide(L, bm);
+            bm.iters += bm.then >= ASK;
         }
         __syncthreads();
         const uint32_t cA = bm.c[0], cM = bm.c[1], segs = bm.c[2], cX = bm.c[3];
-        work += ((unsigned long long)bm.c[5] << 32) | bm.c[4];
-        if (!(cA | cM | cX)) {
-            done = true;
-            break;
+        if (!WARM && bm.then == ASK) {  // (the same weights in every block)
+            const uint32_t e = (uint32_t)((unsigned long long)tid * L.E / WT);
+            const bool keep = __syncthreads_count(__ldg(&L.w[e]) > L.narrow) > (int)WT / 2;
+            if (tid == 0) bm.slow = keep, bm.then = keep ? GO_ON : SWEPT_AGAIN;
+            __syncthreads();
         }
-        if (WARM && bm.c[6]) break;
+        if (bm.then != GO_ON) break;
         const uint32_t next = slot == 2u ? 0u : slot + 1u, after = next == 2u ? 0u : next + 1u;
         if (blockIdx.x == 0 && tid == 0) {  // its counters were last read before this barrier
             SweepIter& z = L.ctl->it[after];
@@ -671,12 +703,6 @@ __global__ void __launch_bounds__(WT, 2) k_sweep(Launch L) {
             if (WARM) z.stop = 0u;
             z.ex = z.work = 0ull;
         }
-        ++iters;
-        if (WARM && iters == WARM_ITERS) break;
-        if (!WARM && iters % HAND_EVERY == 0u &&
-            (work < (unsigned long long)iters * HAND_EDGES || all / (work + 1ull) * iters > HAND_ITERS ||
-             work / HAND_INFL > all))
-            break;  // the listed items keep their marks
         if (cX) {
             // hubs are taken before the iteration, since several warps relax one: a distance that
             // falls from here on marks it again
@@ -718,8 +744,8 @@ __global__ void __launch_bounds__(WT, 2) k_sweep(Launch L) {
         if (bm.imp) atomicAdd(&L.hdr->stats[2], bm.imp);
     }
     if (blockIdx.x == 0 && tid == 0) {
-        atomicAdd(&L.hdr->stats[4], (unsigned long long)iters);
-        L.hdr->swept = done ? 1u : 0u;
+        atomicAdd(&L.hdr->stats[4], (unsigned long long)bm.iters);
+        L.hdr->swept = bm.then == GO_ON ? SWEPT_HANDED : bm.then;
     }
 }
 
@@ -730,6 +756,7 @@ template <class W, int G>
 __global__ void __launch_bounds__(256) k_sweep_out(SweepLaunch L, uint32_t per) {
     __shared__ uint32_t rows[8][32], starts[8][32];
     using D = Dist<W>;
+    if (L.hdr->swept == SWEPT_AGAIN) return;
     const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
     for (uint32_t g = 0; g < L.groups; ++g) {
         for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < L.V; c += gridDim.x * blockDim.x) {
@@ -794,6 +821,7 @@ template <int G>
 __global__ void k_warm_rows(WarmLaunch L) {
     const size_t stride = (size_t)gridDim.x * blockDim.x, i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (size_t i = i0; i < L.n_dirty; i += stride) L.dirty[i] = 0u, L.nfsplit[i] = 0u;
+    for (size_t i = i0; i < sizeof(SweepCtl) / 4; i += stride) reinterpret_cast<uint32_t*>(L.ctl)[i] = 0u;
     for (size_t c = i0; c < L.V; c += stride) {
         const uint32_t at = L.slots ? __ldg(&L.slots[c]) : (uint32_t)c;
         for (uint32_t g = 0; g < L.groups; ++g) {
@@ -875,8 +903,8 @@ template <int G, class Launch>
 __global__ void k_sweep_requeue(Launch L, uint32_t* bitmap, uint32_t words, uint32_t B, uint32_t Bq, uint32_t split,
                                 uint32_t Q) {
     constexpr bool WARM = std::is_same<Launch, WarmLaunch>::value;
-    const bool over = L.hdr->over;
-    if (L.hdr->swept) {
+    const bool over = L.hdr->over, again = !WARM && (over || L.hdr->swept == SWEPT_AGAIN);
+    if (L.hdr->swept == SWEPT_DONE) {
         if (over && L.wtype == SSSP_W_F32)
             judge_overflow<WF32, G>(L);
         else if (over)
@@ -895,7 +923,7 @@ __global__ void k_sweep_requeue(Launch L, uint32_t* bitmap, uint32_t words, uint
                 d = 2 * d + 1;
                 m |= L.over[item >> 5];
             }
-            if (!WARM && over ? L.dist[d] == 0u : (m >> (item & 31u) & 1u) && L.dist[d] < L.inf) bits |= 1u << j;
+            if (again ? L.dist[d] == 0u : (m >> (item & 31u) & 1u) && L.dist[d] < L.inf) bits |= 1u << j;
         }
         bitmap[i] = bits;
         if (!bits) continue;

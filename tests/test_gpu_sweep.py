@@ -379,3 +379,43 @@ def test_overflow_in_a_warm_start_that_is_handed_over(sssp, S):
     for i, s in enumerate(sources):
         d, p, _ = oracle.dijkstra(ref, int(s))
         assert np.array_equal(u32(dist[i]), d) and np.array_equal(u32(pred[i]), p)
+
+
+@pytest.mark.parametrize("S", [1, 3, 8])
+@pytest.mark.parametrize("f32", [False, True])
+def test_tail_is_handed_over(sssp, S, f32):
+    """A random graph, which the sweep is done with in some iterations, with a path of thousands of hops behind
+    it, which the persistent solve follows from what the sweep leaves."""
+    rng = np.random.default_rng(3)
+    V, n = 30000, 6000
+    src, dst, w = graph(rng, V, 9 * V, f32)
+    src = np.concatenate([src, [7], np.arange(V, V + n - 1)]).astype(np.uint32)
+    dst = np.concatenate([dst, np.arange(V, V + n)]).astype(np.uint32)
+    w = np.concatenate([w, np.full(n, 3, w.dtype)])
+    ref = oracle.csr(V + n, src, dst, w)
+    g = sssp.build_csr(V + n, src, dst, w, partitions=19)
+    stats = check(sssp, g, ref, rng.integers(0, V, S).tolist())
+    assert stats["remote_activations"] > 0  # messages between the persistent solve's units
+
+
+@pytest.mark.parametrize("S,delta", [(1, 0.0), (1, 48.0), (3, 0.0), (3, 48.0), (8, 0.0)])
+@pytest.mark.parametrize("kind", ["u32", "f32", "units"])
+def test_graphs_of_many_hops(sssp, S, delta, kind):
+    """A lattice: after the first iterations the persistent solve takes over from the sources, or the sweep
+    goes on (few units and buckets far below the weights)."""
+    rng = np.random.default_rng(4)
+    n = 24
+    at = np.arange(n ** 3).reshape(n, n, n)
+    pairs = [(at[1:].ravel(), at[:-1].ravel()), (at[:, 1:].ravel(), at[:, :-1].ravel()),
+             (at[:, :, 1:].ravel(), at[:, :, :-1].ravel())]
+    src = np.concatenate([a for a, _ in pairs] + [b for _, b in pairs]).astype(np.uint32)
+    dst = np.concatenate([b for _, b in pairs] + [a for a, _ in pairs]).astype(np.uint32)
+    if kind == "f32":
+        w, delta = rng.uniform(0.5, 2.0, src.size).astype(np.float32), delta / 100
+    else:
+        w = rng.integers(1, 256 if kind == "u32" else 2, src.size).astype(np.uint32)
+    ref = oracle.csr(n ** 3, src, dst, w)
+    stats = check(sssp, sssp.build_csr(n ** 3, src, dst, w, partitions=7), ref, rng.integers(0, n ** 3, S).tolist(),
+                  sssp.options(delta=delta))
+    kept = delta == 0.0 and kind != "units"
+    assert (stats["remote_activations"] == 0) == kept
