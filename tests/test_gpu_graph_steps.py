@@ -115,6 +115,18 @@ def test_build_runs_across_tiles(sssp, f32):
             check_build(sssp, V, src, dst, w)
 
 
+@pytest.mark.parametrize("gap", [0, 1, 15, 16, 17, 31, 33, 70, 5000, 1000003])
+def test_build_rows_without_edges(sssp, gap):
+    """Runs of rows without an edge before the first edge, between edges that are neighbours in a warp's step,
+    in two steps and in two tiles, and after the last."""
+    tails = np.concatenate([[gap], gap + 1 + np.arange(40) * (gap + 1)])
+    V = int(tails[-1]) + 1 + gap + 1
+    for reps in (1, 3, 200):  # edges of a row
+        src = np.repeat(tails, reps).astype(np.uint32)
+        dst = ((src + 1 + np.tile(np.arange(reps), tails.size)) % V).astype(np.uint32)
+        check_build(sssp, V, src, dst, np.full(src.size, 7, np.uint32))
+
+
 def test_build_without_an_edge_left_and_bad_edges_reported(sssp):
     v = np.arange(9000, dtype=np.uint32)
     g = sssp.build_csr(9000, v, v, np.ones(9000, np.uint32))  # loops only
