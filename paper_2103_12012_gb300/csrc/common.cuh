@@ -25,7 +25,8 @@ struct WsHeader {
     uint32_t unit_next;     // batch: next unit of the shared-memory kernel
     uint32_t over;          // sweep: a candidate from a distance on the way did not fit
     unsigned long long begin;  // batch: time of its first block's start
-    uint32_t pad[(256 - 4 - 4 - 8 - 8 - 72 - 24) / 4];
+    uint32_t lay_deep;         // layout: edges far into their segments
+    uint32_t pad[(256 - 4 - 4 - 8 - 8 - 72 - 28) / 4];
 };
 static_assert(sizeof(WsHeader) == 256, "header size");
 

@@ -357,6 +357,7 @@ __global__ void __launch_bounds__(256) k_compact(uint32_t V, uint32_t E, const u
 
 constexpr uint32_t COO_RANGE = 1024;
 constexpr uint32_t LAY_TILE = 1024, LAY_SEG = 2048;     // stored edges of a block; longest segment
+constexpr uint32_t LAY_DEEP = 256;                      // edges this far into their segments are counted
 constexpr uint32_t LAY_CAP = LAY_TILE + LAY_SEG + 32u;  // stored edges that a block holds
 
 __global__ void k_lay_deg(uint32_t V, const uint32_t* __restrict__ row_ptr, uint32_t* deg) {
@@ -365,7 +366,7 @@ __global__ void k_lay_deg(uint32_t V, const uint32_t* __restrict__ row_ptr, uint
 }
 
 // In-degrees; and whether the rows can be sorted segment by segment (k_lay_rows): they are as sssp_build_csr
-// makes them, and no segment is longer than LAY_SEG.
+// makes them, no segment is longer than LAY_SEG, and (k_lay_keys) few edges are LAY_DEEP or more into theirs.
 __global__ void __launch_bounds__(256) k_lay_check(uint32_t V, uint32_t E, uint32_t B, const uint32_t* __restrict__ row_ptr,
                                                    const uint32_t* __restrict__ col, const uint32_t* __restrict__ w, int wtype,
                                                    uint32_t* deg, WsHeader* hdr) {
@@ -378,6 +379,7 @@ __global__ void __launch_bounds__(256) k_lay_check(uint32_t V, uint32_t E, uint3
     walk.seek(e0);
     uint32_t before = e0 ? __ldg(&col[e0 - 1u]) : 0u;  // head of the edge before the step
     bool odd = false;
+    uint32_t deep = 0;
     uint32_t v = e0 + lane < e1 ? __ldg(&col[e0 + lane]) : 0u;
     for (uint32_t eb = e0; eb < e1 && eb >= e0; eb += 32u) {
         const uint32_t e = eb + lane, u = walk.step(eb, e1), x = v;
@@ -388,12 +390,17 @@ __global__ void __launch_bounds__(256) k_lay_check(uint32_t V, uint32_t E, uint3
         if (e < e1) {
             const uint32_t at = e - __ldg(&row_ptr[u]), wt = __ldg(&w[e]);
             odd = odd || x >= V || x == u || (at && y >= x) || !(wtype == SSSP_W_F32 ? WF32::weight_ok(wt) : WU32::weight_ok(wt));
-            if (at >= LAY_SEG && __ldg(&col[e - LAY_SEG]) / B == x / B) odd = true;
+            if (at >= LAY_DEEP && __ldg(&col[e - LAY_DEEP]) / B == x / B) {
+                ++deep;
+                if (at >= LAY_SEG && __ldg(&col[e - LAY_SEG]) / B == x / B) odd = true;
+            }
             if (x < V) atomicAdd(&deg[x], 1u);
         }
     }
     if (first == 0 && (row_ptr[0] != 0u || row_ptr[V] != E)) odd = true;
     if (__any_sync(0xFFFFFFFFu, odd) && lane == 0) hdr->lay_general = 1u;
+    deep = __reduce_add_sync(0xFFFFFFFFu, deep);
+    if (deep && lane == 0) atomicAdd(&hdr->lay_deep, deep);
 }
 
 // Degrees of the stored vertices (and a last word for the scan).
@@ -423,7 +430,10 @@ __global__ void k_lay_starts(uint32_t V, const uint32_t* __restrict__ row_ptr, c
 // edge list and its sort took 4.1; the whole layout 10.7 -> 4.87 -> 2.06 ms.  Tiles of 512, 1,024, 2,048 and 4,096
 // edges: 2.11, 2.08, 2.12, 2.19; two, four and eight steps of a warp in flight: 2.12, 2.19, 2.37.
 // A row with a longer segment (hubs, few partitions) sends the whole graph to the builder, whose launches
-// otherwise find an empty list (0.11 ms): 1 M vertices, one partition 3.68 -> 3.74 ms.
+// otherwise find an empty list (0.11 ms): 1 M vertices, one partition 3.68 -> 3.74 ms.  So does a share of
+// 1/8 of the edges that are LAY_DEEP or more into their segments, where the counts cost more than the builder's
+// passes: random graphs of 8,192 vertices, one partition, segments of 1,370 2.78 -> 0.92 ms, four, 342 1.06 -> 0.92;
+// of 65,536, one, 299 1.48 and 1.50; of 8,192, eight, 171 (here) 0.78 against 0.92.
 __global__ void __launch_bounds__(256) k_lay_rows(uint32_t V, uint32_t E, uint32_t B, const uint32_t* __restrict__ start,
                                                   const uint32_t* __restrict__ from, const uint32_t* __restrict__ col,
                                                   const uint32_t* __restrict__ w, const uint32_t* __restrict__ slots,
@@ -486,8 +496,9 @@ __global__ void __launch_bounds__(256) k_lay_rows(uint32_t V, uint32_t E, uint32
     }
 }
 
-__global__ void k_lay_keys(uint32_t V, unsigned long long B, const uint32_t* __restrict__ deg,
-                           uint32_t bits, unsigned long long* keys, uint32_t* vals) {
+__global__ void k_lay_keys(uint32_t V, uint32_t E, unsigned long long B, const uint32_t* __restrict__ deg,
+                           uint32_t bits, unsigned long long* keys, uint32_t* vals, WsHeader* hdr) {
+    if (blockIdx.x == 0 && threadIdx.x == 0 && hdr->lay_deep > E / 8u) hdr->lay_general = 1u;
     for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < V; v += gridDim.x * blockDim.x) {
         keys[v] = ((unsigned long long)(v / B) << bits) | ((0xFFFFFFFFu >> (32u - bits)) - deg[v]);
         vals[v] = v;
@@ -649,7 +660,7 @@ sssp_status layout_build(const sssp_graph* g, uint32_t* row_ptr_out, uint32_t* c
         CK(cudaGetLastError());
     }
     const uint32_t bits = std::min(std::max(bits_for(g->E) + 1u, 1u), 32u);  // of a degree (in + out: at most 2 E)
-    k_lay_keys<<<gv, 256, 0, st>>>(g->V, B, deg, bits, kin, vin);
+    k_lay_keys<<<gv, 256, 0, st>>>(g->V, g->E, B, deg, bits, kin, vin, hdr);
     CK(cudaGetLastError());
     bool second = false;
     CK(sort_pairs_u64(p + L.off_tmp, kin, kout, vin, vout, g->V, (int)(bits + bits_for(g->partitions - 1u)), hdr, st, &second));

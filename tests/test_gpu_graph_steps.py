@@ -206,6 +206,29 @@ def test_layout_segments(sssp, V, P, deg, f32):
     assert np.array_equal(slots[ref.col[:h.E]][e], lay.col[:h.E]) and np.array_equal(ref.w[:h.E].view(np.uint32)[e], u32(h.w)[:h.E])
 
 
+@pytest.mark.parametrize("P,deg,hubs,rest", [(1, 2048, 2, 60000), (1, 2049, 2, 60000), (2, 1300, 6, 60000), (1, 256, 500, 9000),
+                                             (1, 257, 500, 9000), (1, 280, 500, 9000), (1, 330, 500, 9000), (1, 1500, 40, 40),
+                                             (3, 4000, 9, 20)])
+def test_layout_share_of_long_segments(sssp, P, deg, hubs, rest):
+    """Long segments that are few of the edges (their heads are counted), or more than an eighth of them (the
+    builder sorts)."""
+    V = 5003
+    rng = np.random.default_rng(deg + hubs)
+    src, dst, w = edges(deg, V, rest)
+    at = rng.choice(V, hubs, replace=False)
+    src = np.concatenate([src] + [np.full(deg, h) for h in at]).astype(np.uint32)
+    dst = np.concatenate([dst] + [rng.choice(np.delete(np.arange(V), h), deg, replace=False) for h in at]).astype(np.uint32)
+    w = rng.integers(1, 99, src.size).astype(np.uint32)
+    ref = oracle.csr(V, src, dst, w)
+    h = sssp.layout(sssp.build_csr(V, src, dst, w, partitions=P))
+    ids, slots, lay = oracle.layout(ref, P)
+    assert np.array_equal(u32(h.ids), ids) and np.array_equal(u32(h.slots), slots)
+    assert np.array_equal(u32(h.row_ptr), lay.row_ptr)
+    assert np.array_equal(u32(h.col)[:h.E], lay.col[:h.E]) and np.array_equal(u32(h.w)[:h.E], lay.w[:h.E])
+    e = u32(h.eid)[:h.E]
+    assert np.array_equal(np.sort(e), np.arange(h.E)) and np.array_equal(slots[ref.col[:h.E]][e], lay.col[:h.E])
+
+
 @pytest.mark.parametrize("what", ["order", "twice", "loop", "head", "weight"])
 def test_layout_of_rows_that_are_not_canonical(sssp, what):
     """Rows out of order, repeated heads and loops go through the builder, as an edge list would; bad heads
