@@ -15,7 +15,7 @@
 // for the lane that brings it to zero, every sibling's contributions before it
 // reads the parent's sum.  Accumulation is float64.
 //
-// The state has a vertex's sources side by side (item v * S + s).  The trees of
+// The state has a vertex's sources side by side, and warps take items v * S + s.  The trees of
 // different sources share most of their edges (far from the sources the
 // shortest paths are the same), so neighbouring lanes have one parent: their
 // counts and sums are neighbouring words, which an atomic takes a sector at a
@@ -24,6 +24,9 @@
 // 45 -> 26, searches 117 -> 67, walks 255 -> 107 us (153 with the shared edges summed one after another);
 // the transposition costs 8 us more than the copy it replaces.  Bound by the
 // atomics' latency and throughput (four leaves of a thread together: 396 us).
+// Sixteen sources are side by side, so that the sums of a vertex with very many children, which all come to
+// a few cache lines, are in several of them (star of 1 M leaves, 32 sources: 11.2 ms with all side by side, 6.0 with
+// sixteen, 3.7 with eight; random graph of 1 M vertices, 32 sources: 3.1, 3.5 and 3.9).
 #include <algorithm>
 
 #include "common.cuh"
@@ -31,6 +34,9 @@
 
 namespace sssp {
 namespace {
+
+constexpr uint32_t REFILL = 24;  // lanes of a warp (k_bw_walk)
+constexpr uint32_t FEW = 8;      // sources that are transposed without shared memory (1 M vertices, 2: 216 -> 196 us)
 
 struct BwWs {
     uint32_t* nchild;  // [S*V]
@@ -76,7 +82,40 @@ __device__ __forceinline__ int64_t find_edge(const uint32_t* row_ptr, const uint
     return (lo < end && __ldg(&col[lo]) == b) ? (int64_t)lo : -1;
 }
 
-// Item v * S + s of the state from element s * V + v of the caller's arrays, 32 by 32 through shared memory.
+// an item's vertex
+__device__ __forceinline__ uint32_t vertex_of(size_t i, size_t n, uint32_t S) {
+    return n >> 32 ? (uint32_t)(i / S) : (uint32_t)i / S;
+}
+
+// Where the state has (v, s): the sources of a block of sixteen side by side.
+struct Place {
+    size_t base;
+    uint32_t wide;
+    __device__ __forceinline__ Place(uint32_t V, uint32_t S, uint32_t s)
+        : base((size_t)(s & ~15u) * V + (s & 15u)), wide(min(16u, S - (s & ~15u))) {}
+    __device__ __forceinline__ size_t operator()(uint32_t v) const { return base + (size_t)v * wide; }
+};
+
+__device__ __forceinline__ void clear_grad(uint32_t E, double* grad) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < E; i += (size_t)gridDim.x * blockDim.x) grad[i] = 0.0;
+}
+
+// Item v * S + s of the state from element s * V + v of the caller's arrays: a thread per item (a few sources; pred_t
+// NULL: one), or 32 by 32 through shared memory.
+__global__ void __launch_bounds__(256) k_bw_init_few(uint32_t V, uint32_t S, uint32_t E, const float* __restrict__ g,
+                                                     const uint32_t* __restrict__ pred, uint32_t* nchild, double* acc,
+                                                     uint32_t* pred_t, double* grad) {
+    const size_t n = (size_t)S * V;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const uint32_t v = vertex_of(i, n, S);
+        const size_t at = (i - (size_t)v * S) * V + v;
+        nchild[i] = 0u;
+        acc[i] = (double)__ldg(&g[at]);
+        if (pred_t) pred_t[i] = __ldg(&pred[at]);
+    }
+    clear_grad(E, grad);
+}
+
 __global__ void __launch_bounds__(256) k_bw_init(uint32_t V, uint32_t S, uint32_t E, const float* __restrict__ g,
                                                  const uint32_t* __restrict__ pred, uint32_t* nchild, double* acc,
                                                  uint32_t* pred_t, double* grad) {
@@ -96,7 +135,7 @@ __global__ void __launch_bounds__(256) k_bw_init(uint32_t V, uint32_t S, uint32_
             __syncthreads();
             for (uint32_t k = threadIdx.x; k < nv * ns; k += 256u) {
                 const uint32_t v = k / ns, s = k - v * ns;
-                const size_t i = (size_t)(v0 + v) * S + s0 + s;
+                const size_t i = Place(V, S, s0 + s)(v0 + v);
                 nchild[i] = 0u;
                 acc[i] = (double)gs[s][v];
                 pred_t[i] = ps[s][v];
@@ -104,24 +143,21 @@ __global__ void __launch_bounds__(256) k_bw_init(uint32_t V, uint32_t S, uint32_
             __syncthreads();
         }
     }
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < E; i += (size_t)gridDim.x * blockDim.x) grad[i] = 0.0;
-}
-
-// an item's vertex
-__device__ __forceinline__ uint32_t vertex_of(size_t i, size_t n, uint32_t S) {
-    return n >> 32 ? (uint32_t)(i / S) : (uint32_t)i / S;
+    clear_grad(E, grad);
 }
 
 __global__ void k_bw_count(uint32_t V, uint32_t S, size_t n, const uint32_t* __restrict__ pred, uint32_t* nchild, WsHeader* hdr) {
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const uint32_t p = pred[i];
+        const uint32_t v = vertex_of(i, n, S);
+        const Place at(V, S, (uint32_t)(i - (size_t)v * S));
+        const uint32_t p = pred[at(v)];
         if (p == NONE) continue;
         if (p >= V) {
             set_status(hdr, SSSP_EINVAL);
             continue;
         }
-        atomicAdd(&nchild[(size_t)p * S + (i - (size_t)vertex_of(i, n, S) * S)], 1u);
+        atomicAdd(&nchild[at(p)], 1u);
     }
 }
 
@@ -131,10 +167,12 @@ __global__ void k_bw_leaves(uint32_t V, uint32_t S, size_t n, const uint32_t* __
                             const uint32_t* __restrict__ nchild, uint8_t* leaf, uint32_t* eidx) {
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const uint32_t p = pred[i];
-        leaf[i] = (p != NONE && nchild[i] == 0u) ? 1u : 0u;
-        const int64_t e = (p != NONE && p < V) ? find_edge(row_ptr, col, p, vertex_of(i, n, S)) : -1;
-        eidx[i] = e < 0 ? NONE : (uint32_t)e;
+        const uint32_t v = vertex_of(i, n, S);
+        const size_t at = Place(V, S, (uint32_t)(i - (size_t)v * S))(v);
+        const uint32_t p = pred[at];
+        leaf[at] = (p != NONE && nchild[at] == 0u) ? 1u : 0u;
+        const int64_t e = (p != NONE && p < V) ? find_edge(row_ptr, col, p, v) : -1;
+        eidx[at] = e < 0 ? NONE : (uint32_t)e;
     }
 }
 
@@ -145,52 +183,82 @@ __device__ __forceinline__ uint32_t dec_acq_rel(uint32_t* p) {
     return old;
 }
 
-// A warp walks its 32 items up together; the lanes on one tree edge add to its gradient once.
-__global__ void __launch_bounds__(256) k_bw_walk(uint32_t V, uint32_t S, size_t n, const uint32_t* __restrict__ pred,
+// A warp walks the leaves among its items up.  A lane whose walk has ended takes another item while others go on (once
+// REFILL lanes or fewer do): walks are as long as the tree is deep, and a warp that waited for its longest one left
+// the other lanes idle.  Grid of 1000 x 1000, 8 sources: 17.2 -> 3.5 ms (7.2 with an array per source and a thread
+// per leaf); random graph of 1 M vertices, 32 sources: 2.5 -> 2.9 (3.7), since fewer lanes share an edge; with 4 lanes
+// for REFILL 4.0 and 2.8, with 31 3.6 and 2.9.
+// SHARED: the lanes on one tree edge add to its gradient once.
+template <bool SHARED>
+__global__ void __launch_bounds__(256) k_bw_walk(uint32_t V, uint32_t S, size_t n, size_t per, const uint32_t* __restrict__ pred,
                                                  const uint32_t* __restrict__ eidx, const uint8_t* __restrict__ leaf,
                                                  uint32_t* nchild, double* acc, double* grad, WsHeader* hdr) {
     const uint32_t lane = threadIdx.x & 31u;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (size_t i0 = (size_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += stride) {
-        size_t at = i0 + lane;  // the item
-        const uint32_t s = (uint32_t)(at - (size_t)vertex_of(at, n, S) * S);
-        bool on = at < n && leaf[at];  // walks start at leaves only
-        // bounded by V steps: a tree path has fewer than V edges
-        for (uint32_t step = 0; step < V && __any_sync(0xFFFFFFFFu, on); ++step) {
-            uint32_t p = NONE, e = NONE;
-            double a = 0.0;
-            if (on) {
-                p = __ldg(&pred[at]);
-                e = __ldg(&eidx[at]);
-                a = ld_relaxed(&acc[at]);
-                if (p >= V) {  // reached the source
-                    on = false;
-                } else if (e == NONE) {  // (pred(x), x) is not an edge
-                    set_status(hdr, SSSP_EINVAL);
-                    on = false;
+    size_t next = (((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per;  // first item not taken yet
+    const size_t end = min(next + per, n);
+    size_t at = 0;  // where the lane is
+    Place place(V, S, 0);
+    uint32_t steps = 0;
+    bool on = false;
+    for (;;) {
+        const uint32_t live = __ballot_sync(0xFFFFFFFFu, on);
+        bool fresh = false;  // (walks start at leaves only)
+        if (next < end && __popc(live) <= (int)REFILL) {
+            if (!on) {
+                const size_t i = next + __popc(~live & ((1u << lane) - 1u));
+                fresh = i < end;
+                steps = 0;
+                if (fresh) {
+                    const uint32_t v = vertex_of(i, n, S);
+                    place = Place(V, S, (uint32_t)(i - (size_t)v * S));
+                    at = place(v);
                 }
             }
+            next += 32u - __popc(live);
+        } else if (!live) {
+            break;
+        }
+        uint32_t p = NONE, e = NONE;
+        double a = 0.0;
+        if (on || fresh) {
+            p = __ldg(&pred[at]);
+            e = __ldg(&eidx[at]);
+            a = ld_relaxed(&acc[at]);
+            if (fresh) on = leaf[at];
+            if (on && p >= V) {  // reached the source
+                on = false;
+            } else if (on && e == NONE) {  // (pred(x), x) is not an edge
+                set_status(hdr, SSSP_EINVAL);
+                on = false;
+            }
+        }
+        const bool act = on;
+        uint32_t left = 0;
+        if (act) {
+            at = place(p);
+            atomicAdd(&acc[at], a);
+            // release: my contributions before my decrement; acquire (last child): every
+            // sibling's contributions before the read of acc[p] in the next step
+            left = dec_acq_rel(&nchild[at]);
+        }
+        // (the edges' gradients, while the decrement is on its way)
+        bool first = act;
+        double sum = a;
+        if constexpr (SHARED) {
             // one addition to the edge's gradient for the lanes that share it: pairs, pairs of pairs, ... of
             // all edges at once (a lane of odd rank hands its sum to the one before and drops out)
-            const uint32_t same = __match_any_sync(0xFFFFFFFFu, on ? e : NONE);
-            uint32_t rank = __popc(same & ((1u << lane) - 1u)), rest = on ? same & (0xFFFFFFFEu << lane) : 0u;
-            const bool first = rank == 0u;
-            double sum = a;
+            const uint32_t same = __match_any_sync(0xFFFFFFFFu, act ? e : NONE);
+            uint32_t rank = __popc(same & ((1u << lane) - 1u)), rest = act ? same & (0xFFFFFFFEu << lane) : 0u;
+            first = act && rank == 0u;
             for (; __any_sync(0xFFFFFFFFu, rest != 0u); rank >>= 1) {
-                const uint32_t next = rest ? __ffs(rest) - 1u : lane;
-                const double t = __shfl_sync(0xFFFFFFFFu, sum, next);
+                const uint32_t other = rest ? __ffs(rest) - 1u : lane;
+                const double t = __shfl_sync(0xFFFFFFFFu, sum, other);
                 if (rest) sum += t;
                 rest &= __ballot_sync(0xFFFFFFFFu, !(rank & 1u));
             }
-            if (on) {
-                if (first) atomicAdd(&grad[e], sum);
-                at = (size_t)p * S + s;
-                atomicAdd(&acc[at], a);
-                // release: my contributions before my decrement; acquire (last child): every
-                // sibling's contributions before the read of acc[p] in the next step
-                on = dec_acq_rel(&nchild[at]) == 1u;
-            }
         }
+        if (first) atomicAdd(&grad[e], sum);
+        on = act && left == 1u && ++steps < V;  // (a tree path has fewer than V edges)
     }
 }
 
@@ -217,10 +285,19 @@ cudaError_t backward_launch(const sssp_graph* g, uint32_t S, const uint32_t* pre
     const size_t n = (size_t)S * g->V;
     cudaError_t e;
     if ((e = cudaMemsetAsync(hdr, 0, WS_HEADER_BYTES, st)) != cudaSuccess) return e;
-    k_bw_init<<<grid_for(std::max<size_t>(n, g->E)), 256, 0, st>>>(g->V, S, g->E, grad_dist, pred, b.nchild, b.acc, b.pred, b.grad);
-    k_bw_count<<<grid_for(n), 256, 0, st>>>(g->V, S, n, b.pred, b.nchild, hdr);
-    k_bw_leaves<<<grid_for(n), 256, 0, st>>>(g->V, S, n, g->row_ptr, g->col, b.pred, b.nchild, b.leaf, b.eidx);
-    k_bw_walk<<<grid_for(n), 256, 0, st>>>(g->V, S, n, b.pred, b.eidx, b.leaf, b.nchild, b.acc, b.grad, hdr);
+    const unsigned init = grid_for(std::max<size_t>(n, g->E));
+    if (S == 1) b.pred = nullptr;  // (the caller's is in this order)
+    if (S <= FEW)
+        k_bw_init_few<<<init, 256, 0, st>>>(g->V, S, g->E, grad_dist, pred, b.nchild, b.acc, b.pred, b.grad);
+    else
+        k_bw_init<<<init, 256, 0, st>>>(g->V, S, g->E, grad_dist, pred, b.nchild, b.acc, b.pred, b.grad);
+    if (S > 1) pred = b.pred;
+    k_bw_count<<<grid_for(n), 256, 0, st>>>(g->V, S, n, pred, b.nchild, hdr);
+    k_bw_leaves<<<grid_for(n), 256, 0, st>>>(g->V, S, n, g->row_ptr, g->col, pred, b.nchild, b.leaf, b.eidx);
+    const unsigned walks = grid_for(n);
+    const size_t per = ((n + walks * 8ull - 1) / (walks * 8ull) + 31) & ~(size_t)31;
+    (S > 1 ? k_bw_walk<true> : k_bw_walk<false>)<<<walks, 256, 0, st>>>(g->V, S, n, per, pred, b.eidx, b.leaf, b.nchild, b.acc,
+                                                                        b.grad, hdr);
     k_bw_out<<<grid_for(g->E), 256, 0, st>>>(g->E, b.grad, grad_w);
     return cudaGetLastError();
 }

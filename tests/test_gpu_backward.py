@@ -57,3 +57,20 @@ def test_paths(sssp, S):
     V = 1500
     src = np.arange(V - 1, dtype=np.uint32)
     check(sssp, V, src, src + 1, np.random.default_rng(2).uniform(0.5, 2.0, V - 1).astype(np.float32), list(range(S)))
+
+
+@pytest.mark.parametrize("S", [1, 2, 8, 9, 16, 17, 33, 47])
+@pytest.mark.parametrize("kind", ["grid", "star"])
+def test_deep_trees_and_many_children(sssp, S, kind):
+    """Walks of many steps, whose warps take other leaves meanwhile; and one parent of most vertices.  Blocks of
+    sixteen sources and their remainders."""
+    rng = np.random.default_rng(S)
+    if kind == "grid":
+        at = np.arange(60 * 55).reshape(60, 55)
+        a = np.concatenate([at[1:].ravel(), at[:, 1:].ravel()])
+        b = np.concatenate([at[:-1].ravel(), at[:, :-1].ravel()])
+    else:
+        a, b = np.zeros(4000, np.int64), np.arange(1, 4001)
+    src, dst = np.concatenate([a, b]).astype(np.uint32), np.concatenate([b, a]).astype(np.uint32)
+    V = int(src.max()) + 1
+    check(sssp, V, src, dst, rng.uniform(0.5, 2.0, src.size).astype(np.float32), rng.integers(0, V, S).tolist())
