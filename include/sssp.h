@@ -436,7 +436,8 @@ size_t sssp_batch_workspace_size(const sssp_batch* b, const sssp_options* opt);
  * (one partition), unpack -- with no message traffic between blocks.
  * Graphs of at most 47,104 vertices are solved in shared memory, up to 16 problems of a
  * graph together, by a second launch (threads and tile are then not used, and buckets are
- * three times as wide as delta says), unless a few larger ones are among them.
+ * three times as wide as delta says), unless a few larger ones, very dense ones or, at a
+ * given delta, large ones of fewer than five edges per vertex are among them.
  * Uploads the problem tables (host arrays) into ws on `stream` and waits for
  * that copy, then launches: unlike the other solve calls this one blocks the
  * host until the upload is done, and it cannot be captured into a CUDA graph

@@ -654,13 +654,27 @@ struct BatchTables {
     uint64_t total_out = 0, total_words = 0;
 };
 
-bool build_tables(const sssp_batch* b, BatchTables* t) {
+// Whether a graph is for shared memory.  Its blocks are few, and bound by instructions and by the barriers of their
+// rounds, so that the general kernel is the faster one for (general / shared memory, ms)
+//   very dense graphs, whose edges it reads faster: 20 graphs of 1,500 vertices, 200 edges each, 1 source: 0.71 / 0.97;
+//     dense ones if there are problems for several rounds of blocks: 100 R-MAT graphs of 4,000, 24 each, 16 sources:
+//     1.55 / 2.28, random ones of 48 each 2.5 / 3.0, but 200 of 1,000, 48 each, 1 source 0.30 / 0.22
+//   grids, at a width made for them, if there are more problems than blocks: 64 of 200 x 200, 16 sources, width 300:
+//     6.9 / 12.4 (at 16: 26.8 / 26.2)
+bool in_smem(const sssp_batch_graph& G, uint64_t n_problems, uint64_t blocks, bool delta_given) {
+    if (G.V > BATCH_ITEMS || G.E > 64ull * G.V) return false;
+    if (G.E > 24ull * G.V && G.V >= 512 && G.V < 8192 && n_problems > blocks) return false;
+    return !(G.E < 5ull * G.V && G.V >= 8192 && delta_given && n_problems > blocks / 2u);
+}
+
+bool build_tables(const sssp_batch* b, bool delta_given, BatchTables* t) {
     if (!b || !b->graphs || !b->prob_graph || !b->prob_source || !b->row_ptr || !b->dist) return false;
     if (b->wtype != SSSP_W_U32 && b->wtype != SSSP_W_F32) return false;
     if (b->n_problems == 0 || b->n_graphs == 0) return false;
     t->probs.resize(b->n_problems);
     uint64_t out = 0;
-    uint64_t large = 0;  // problems that shared memory does not hold
+    uint64_t large = 0;  // problems that are not for shared memory
+    const uint64_t blocks = 2u * (uint64_t)std::max(sm_count(), 1);
     for (uint32_t i = 0; i < b->n_problems; ++i) {
         const uint32_t gi = b->prob_graph[i];
         if (gi >= b->n_graphs) return false;
@@ -676,7 +690,7 @@ bool build_tables(const sssp_batch* b, BatchTables* t) {
         p.src = b->prob_source[i];
         p.E = G.E;
         p.pad = gi;
-        large += G.V > BATCH_ITEMS;
+        large += !in_smem(G, b->n_problems, blocks, delta_given);
         out += G.V;
     }
     t->total_out = out;
@@ -684,8 +698,7 @@ bool build_tables(const sssp_batch* b, BatchTables* t) {
     // largest graphs first (longest-processing-time order), stable
     std::stable_sort(t->probs.begin(), t->probs.end(),
                      [](const BatchProblem& x, const BatchProblem& y) { return x.E > y.E; });
-    const uint64_t blocks = 2u * (uint64_t)std::max(sm_count(), 1);
-    // Shared memory takes all problems that it holds if it holds every graph, or if the others fill the chip
+    // Shared memory takes all problems that are for it if every graph is, or if the others fill the chip
     // several times by themselves (the two kernels run one after the other: 512 graphs of 1,024 to 131,072
     // vertices, 16 sources each, 1,648 large problems, 30.8 -> 29.1 ms, float32 27.9 -> 24.4; 2 each, 206 large ones,
     // would go from 5.4 to 6.3).
@@ -697,7 +710,7 @@ bool build_tables(const sssp_batch* b, BatchTables* t) {
         const uint32_t most = (uint32_t)std::min<uint64_t>(std::max<uint64_t>((b->n_problems - large) / blocks, 1), BATCH_COPIES);
         for (size_t i = 0; i < t->probs.size();) {
             const BatchProblem& p = t->probs[i];
-            if (p.V > BATCH_ITEMS) {
+            if (!in_smem(b->graphs[p.pad], b->n_problems, blocks, delta_given)) {
                 rest.push_back(p);
                 rest.back().pad = 0;
                 ++i;
@@ -768,7 +781,8 @@ sssp_status prepare_batch(const sssp_batch* b, const sssp_options* opt, void* ws
                           cudaStream_t st, BatchLaunch* l, BatchSmem* x) {
     Resolved r;
     BatchTables t;
-    if (!ws || !aligned16(ws) || !resolve(opt, b ? b->wtype : 0, &r) || !build_tables(b, &t)) return SSSP_EINVAL;
+    if (!ws || !aligned16(ws) || !resolve(opt, b ? b->wtype : 0, &r) || !build_tables(b, r.delta_given, &t))
+        return SSSP_EINVAL;
     if (r.threads > BATCH_MAX_THREADS) return SSSP_EINVAL;
     const BatchWs L = batch_layout(t);
     if (ws_bytes < L.total) return SSSP_ENOMEM;
@@ -829,9 +843,9 @@ sssp_status prepare_batch(const sssp_batch* b, const sssp_options* opt, void* ws
 
 size_t sssp_batch_workspace_size(const sssp_batch* b, const sssp_options* opt) {
     Resolved r;
-    BatchTables t;
-    if (!resolve(opt, b ? b->wtype : 0, &r) || !build_tables(b, &t)) return 0;
-    return batch_layout(t).total;
+    BatchTables t, u;  // (enough for any options)
+    if (!resolve(opt, b ? b->wtype : 0, &r) || !build_tables(b, true, &t) || !build_tables(b, false, &u)) return 0;
+    return std::max(batch_layout(t).total, batch_layout(u).total);
 }
 
 sssp_status sssp_solve_batched(const sssp_batch* b, const sssp_options* opt, void* ws, size_t ws_bytes,

@@ -28,7 +28,9 @@
 namespace sssp {
 namespace {
 
-constexpr uint32_t HUB = 512;                    // rows from here on are cut into segments of this size
+// rows from here on are cut into segments of this size (512: the warp with the longest rows held up the round: 100 R-MAT
+// graphs of 4,000 vertices, 16 sources each, 0.80 -> 0.72 ms, 256 0.75, 64 0.65; 30 of 40,000, 16 edges each, 2.62 -> 2.79)
+constexpr uint32_t HUB = 128;
 constexpr uint32_t HCAP = 512;                   // hub segments of a round
 constexpr uint32_t EB = 1;                       // steps of 32 edges in flight
 constexpr uint64_t LIMIT_FACTOR = 3;
@@ -43,6 +45,7 @@ struct Mem {
     uint2 hub[HCAP];         // item, segment
     uint32_t next, hnext[2], nhub[2], low[2], flags[2];  // by round parity
     unsigned long long stats[6];
+    uint32_t reach[BATCH_COPIES];  // vertices that a copy's source has reached
 };
 
 // The items of a unit: copy * V + vertex.
@@ -162,20 +165,24 @@ struct Round {
         __syncwarp();
     }
 
-    // A round: the items marked near, 512 of them at a time (16 marks a lane), in turn by the block's
-    // warps, and then the hubs' segments.  A round that advances (a new thr) takes the items marked far
-    // that are below thr.
+    // A round: the items marked near, up to 512 of them at a time (16 marks a lane; fewer of a small unit, so that
+    // every warp gets some, and two lots if there are copies: 20 graphs of 1,500 vertices and 300,000 edges, 1 source
+    // each, 3.1 -> 1.0 ms; 100 R-MAT graphs of 4,000 vertices, 16 sources each, 1.30 -> 0.80, four lots the same, but
+    // random graphs 0.99 and 1.15), in turn by the block's warps, and then the hubs' segments.  A round that advances (a new thr) takes the
+    // items marked far that are below thr.
     __device__ __forceinline__ void work(uint32_t n_items, bool advance) {
         const uint32_t words = (n_items + 31u) / 32u, sh = 16u * (lane & 1u);
+        const uint32_t turns = n_items > V ? BT / 16u : BT / 32u;
+        const uint32_t few = min((words + turns - 1u) / turns, 16u);  // words at a time
         uint32_t nq = 0;
         for (;;) {
             uint32_t c = 0;
-            if (lane == 0) c = atomicAdd(&M.next, 16u);
+            if (lane == 0) c = atomicAdd(&M.next, few);
             c = __shfl_sync(0xFFFFFFFFu, c, 0);
             if (c >= words) break;
             const uint32_t wi = c + lane / 2u, first = wi * 32u + sh;
             uint32_t take = 0;
-            if (wi < words) {
+            if (wi < words && lane < 2u * few) {
                 if (advance) {
                     for (uint32_t t = *reinterpret_cast<volatile uint32_t*>(&I.far[wi]) >> sh & 0xFFFFu; t; t &= t - 1u) {
                         const uint32_t j = __ffs(t) - 1;
@@ -310,13 +317,41 @@ __device__ __forceinline__ void solve_unit(const BatchSmem& B, Mem<BT / 32>& M, 
         atomicExch(&B.hdr->abort_flag, 1u);
     }
 
-    for (uint32_t s = 0; s < S; ++s)
+    for (uint32_t s = 0; s < S; ++s) {
+        uint32_t n = 0;
         for (uint32_t v = tid; v < V; v += BT) {
-            B.dist[U.out[s] + v] = I.dist[s * V + v];
+            const uint32_t d = I.dist[s * V + v];
+            n += d < W::inf_out();
+            B.dist[U.out[s] + v] = d;
             if (B.pred) B.pred[U.out[s] + v] = NONE;
         }
+        n = __reduce_add_sync(0xFFFFFFFFu, n);
+        if (lane == 0 && n) atomicAdd(&M.reach[s], n);
+    }
     const bool over = __syncthreads_or((int)(R.bad & 2u));
+    // The walk over all edges is for the copies that have reached many vertices (an isolated source of 40,000
+    // vertices and 1.4 M edges: 229 -> 19 us); the rows of the few that the others have reached are gone through.
+    uint32_t many = 0;
+    for (uint32_t s = 0; s < S; ++s) many |= M.reach[s] > V / 8u ? 1u << s : 0u;
     if (B.pred && !stopped) {
+        for (uint32_t m = ~many & ((1u << S) - 1u); m; m &= m - 1u) {
+            const uint32_t s = __ffs(m) - 1u;
+            if (M.reach[s] < 2u) continue;
+            for (uint32_t v0 = wid * 32u; v0 < V; v0 += BT) {
+                const uint32_t mine = v0 + lane < V ? I.get(s * V + v0 + lane) : W::inf_out();
+                for (uint32_t b = __ballot_sync(0xFFFFFFFFu, mine < W::inf_out()); b; b &= b - 1u) {
+                    const uint32_t l = __ffs(b) - 1u, d = __shfl_sync(0xFFFFFFFFu, mine, l), end = __ldg(&R.row_ptr[v0 + l + 1u]);
+                    for (uint32_t e = __ldg(&R.row_ptr[v0 + l]) + lane; e < end; e += 32u) {
+                        const uint32_t v = __ldg(&R.col[e]), x = __ldg(&R.w[e]);
+                        uint32_t c;
+                        if (v < V && W::weight_ok(x) && W::add(d, x, c) && c == I.get(s * V + v))
+                            atomicMin(&B.pred[U.out[s] + v], v0 + l);
+                    }
+                }
+            }
+        }
+    }
+    if (B.pred && many && !stopped) {
         uint32_t* const rows = reinterpret_cast<uint32_t*>(M.row[wid]);
         RowWalk walk{R.row_ptr, V, rows, rows + 32};
         const uint32_t first = R.row_ptr[0], E = R.row_ptr[V] - first;
@@ -333,7 +368,8 @@ __device__ __forceinline__ void solve_unit(const BatchSmem& B, Mem<BT / 32>& M, 
             auto step = [&](uint32_t eb, int j) {
                 const uint32_t u = walk.step(eb, e1);
                 if (v[j] >= V || !W::weight_ok(x[j])) return;
-                for (uint32_t s = 0; s < S; ++s) {
+                for (uint32_t m = many; m; m &= m - 1u) {
+                    const uint32_t s = __ffs(m) - 1u;
                     uint32_t c;
                     if (W::add(I.get(s * V + u), x[j], c) && c == I.get(s * V + v[j]))
                         atomicMin(&B.pred[U.out[s] + v[j]], u);
@@ -389,6 +425,7 @@ __global__ void __launch_bounds__(BT, 1024 / BT) k_batch(BatchSmem B) {
             M.low[0] = M.low[1] = W::inf_out();
         }
         if (tid < 6u) M.stats[tid] = 0ull;
+        if (tid < BATCH_COPIES) M.reach[tid] = 0u;
         __syncthreads();
         if (M.unit_at >= B.n_units) break;
         if (tid < sizeof(BatchUnit) / 4)

@@ -194,3 +194,59 @@ def test_overflow_is_of_final_distances(sssp, V, preds, f32):
             d, p, _ = oracle.dijkstra(g, 10 * i)
             bd, bp = b.result(i)
             assert np.array_equal(u32(bd), d.view(np.uint32)) and (not preds or np.array_equal(u32(bp), p))
+
+
+@pytest.mark.parametrize("V", [40, 3000, 20000])
+def test_sources_that_reach_little(sssp, V):
+    """Isolated sources, sources with a few edges or a long row into vertices without edges, and sources that
+    reach an eighth of the graph and more, as copies of one graph."""
+    rng = np.random.default_rng(V)
+    k = V // 8
+    src, dst = rng.integers(k, V, 6 * V), rng.integers(k, V, 6 * V)  # vertices from k on; the first ones are apart
+    few = np.stack([[1, 1, 2, 3], [2, 3, 4, 4]])
+    row = np.stack([np.full(k - 5, 4), np.arange(5, k)]) if V > 40 else np.zeros((2, 0), int)
+    half = np.stack([np.arange(k, k + V // 16), np.arange(k + 1, k + 1 + V // 16)])
+    src, dst = np.concatenate([src, few[0], row[0], half[0]]), np.concatenate([dst, few[1], row[1], half[1]])
+    g = oracle.csr(V, src.astype(np.uint32), dst.astype(np.uint32), rng.integers(1, 9, src.size).astype(np.uint32))
+    sources = [0, 1, 2, 4, V - 1, k, 0, 3, V - 2, 1, 0, 4]
+    graphs = [g] + [graph(rng, 300, 1500) for _ in range(3)]
+    b = sssp.Batch(graphs, [sources, [1], [2] * 17, [5]], sssp.options(delta=3.0))
+    for _ in range(2):
+        b.solve()
+        check(b, graphs)
+
+
+@pytest.mark.parametrize("kind", ["dense", "very dense", "grids"])
+@pytest.mark.parametrize("delta", [0.0, 40.0])
+def test_graphs_that_shared_memory_leaves(sssp, kind, delta):
+    """Dense graphs and grids, with few and with many problems, at the default and a given width; a workspace of the
+    size for other options does."""
+    rng = np.random.default_rng(len(kind))
+    if kind == "grids":
+        at = np.arange(100 * 90).reshape(100, 90)
+        a, c = np.concatenate([at[1:].ravel(), at[:, 1:].ravel()]), np.concatenate([at[:-1].ravel(), at[:, :-1].ravel()])
+        g = oracle.csr(9000, np.concatenate([a, c]).astype(np.uint32), np.concatenate([c, a]).astype(np.uint32),
+                       rng.integers(1, 99, 2 * a.size).astype(np.uint32))
+    else:
+        g = graph(rng, 600, 600 * (40 if kind == "dense" else 90))
+    for n in (3, 1300):
+        b = sssp.Batch([g], [rng.integers(0, g.V, n).tolist()], sssp.options())
+        b.opts.delta = delta
+        b.solve()
+        check(b, [g], step=max(n // 9, 1))
+
+
+@pytest.mark.parametrize("V,S", [(900, 3), (16000, 5)])
+def test_rows_at_the_bound_of_segments(sssp, V, S):
+    """Rows of 127, 128, 129, 255, 256 and 257 edges, relaxed in the same rounds as short ones."""
+    rng = np.random.default_rng(V)
+    src, dst = [rng.integers(0, V, 4 * V)], [rng.integers(0, V, 4 * V)]
+    for k, d in enumerate((127, 128, 129, 255, 256, 257)):
+        for v in range(k, V, 100):
+            src.append(np.full(d, v))
+            dst.append(rng.choice(V, d, replace=False))
+    src, dst = np.concatenate(src).astype(np.uint32), np.concatenate(dst).astype(np.uint32)
+    g = oracle.csr(V, src, dst, rng.integers(1, 200, src.size).astype(np.uint32))
+    b = sssp.Batch([g] * 70, [rng.integers(0, V, S).tolist() for _ in range(70)], sssp.options(delta=16.0))
+    b.solve()
+    check(b, [g] * 70, step=7)
