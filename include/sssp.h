@@ -144,6 +144,8 @@ typedef enum {
  * termination count can never reach zero; the solve must then end with
  * SSSP_ETIMEOUT after `timeout_ns`, with the device still usable. */
 #define SSSP_FLAG_TEST_HOLD_PENDING 0x1u
+/* Test hook: sssp_solve and sssp_update run the persistent solve where they would sweep. */
+#define SSSP_FLAG_TEST_PERSISTENT 0x2u
 
 /* Device-side counters of the last solve (sssp_workspace_status). */
 typedef struct {

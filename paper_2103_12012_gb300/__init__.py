@@ -25,6 +25,7 @@ W_U32, W_F32 = 0, 1
 POLICY_RELATIVE, POLICY_FIXED, POLICY_NEAR_FAR, POLICY_ALL = range(4)
 POLICY_NAMES = ("relative", "fixed", "near_far", "all")
 FLAG_TEST_HOLD_PENDING = 0x1
+FLAG_TEST_PERSISTENT = 0x2
 NONE = 0xFFFFFFFF
 
 P = ctypes.c_void_p

@@ -304,7 +304,7 @@ static sssp_status solve_impl(const sssp_graph* g, const uint32_t* sources, uint
     const bool prune = prune_mode >= 0;
     // The sweep takes solves in the default policy (the others ask for a schedule of the persistent solve).
     const bool sweep =
-        L.sweep && !persistent && !prune && r.policy == SSSP_POLICY_RELATIVE && r.msg_buffer == 0 && !(r.flags & SSSP_FLAG_TEST_HOLD_PENDING) &&
+        L.sweep && !persistent && !prune && r.policy == SSSP_POLICY_RELATIVE && r.msg_buffer == 0 && !(r.flags & (SSSP_FLAG_TEST_HOLD_PENDING | SSSP_FLAG_TEST_PERSISTENT)) &&
         (warm ? warm_sweep_wins(S, n_tails, static_cast<char*>(ws) + L.off_packed) : sweep_wins(g, S, L, r.delta_given));
     int per_sm = 0;
     const uint32_t hubs = g->ids ? std::min(r.hub_count, L.B) : 0u;  // layout graphs only
