@@ -250,3 +250,16 @@ def test_rows_at_the_bound_of_segments(sssp, V, S):
     b = sssp.Batch([g] * 70, [rng.integers(0, V, S).tolist() for _ in range(70)], sssp.options(delta=16.0))
     b.solve()
     check(b, [g] * 70, step=7)
+
+
+@pytest.mark.parametrize("V", [3000, 40000])
+def test_limit_ends_a_batch(sssp, V):
+    """A limit of a nanosecond ends the batch with a status; the next call in the same workspace is right."""
+    rng = np.random.default_rng(V)
+    g = graph(rng, V, 8 * V)
+    b = sssp.Batch([g], [rng.integers(0, V, 400).tolist()], sssp.options(delta=16.0, timeout_ns=1))
+    b.solve()
+    assert b.status()[0] == sssp.SSSP_ETIMEOUT
+    b.opts.timeout_ns = 0
+    b.solve()
+    check(b, [g], step=40)

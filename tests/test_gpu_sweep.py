@@ -419,3 +419,54 @@ def test_graphs_of_many_hops(sssp, S, delta, kind):
                   sssp.options(delta=delta))
     kept = delta == 0.0 and kind != "units"
     assert (stats["remote_activations"] == 0) == kept
+
+
+@pytest.mark.parametrize("S", [1, 4, 9])
+def test_limit_of_a_sweep_ends_it(sssp, S):
+    """A limit of a nanosecond ends the waits of a cold and of a warm sweep with a status; the hand-over behind them
+    passes, and the next call in the same workspace is right."""
+    rng = np.random.default_rng(S)
+    V = 60000
+    src, dst, w = graph(rng, V, 8 * V)
+    w2 = np.maximum(1, w // 2).astype(np.uint32)
+    g, g2 = sssp.build_csr(V, src, dst, w, partitions=9), sssp.build_csr(V, src, dst, w2, partitions=9)
+    sources = torch.from_numpy(rng.integers(0, V, S).astype(np.int32)).cuda()
+    tails = torch.arange(17000, dtype=torch.int32, device="cuda")
+    cold, warm = sssp.Solver(g, S, sssp.options(timeout_ns=1)), sssp.Solver(g2, S, sssp.options(timeout_ns=1))
+    cold(sources, check=False)
+    assert cold.last_status == sssp.SSSP_ETIMEOUT
+    cold.opts.timeout_ns = 0
+    dist, pred = cold(sources)
+    assert cold.last_stats["remote_activations"] == 0  # (swept)
+    for i, s in enumerate(sources.tolist()):
+        d, p, _ = oracle.dijkstra(oracle.csr(V, src, dst, w), s)
+        assert np.array_equal(u32(dist[i]), d) and np.array_equal(u32(pred[i]), p)
+    warm.update(dist.clone(), pred.clone(), tails)
+    assert warm.status()[0] == sssp.SSSP_ETIMEOUT
+    warm.opts.timeout_ns = 0
+    dist, pred = warm.update(dist.clone(), pred.clone(), torch.arange(V, dtype=torch.int32, device="cuda"))
+    assert warm.status()[0] == 0
+    for i, s in enumerate(sources.tolist()):
+        d, p, _ = oracle.dijkstra(oracle.csr(V, src, dst, w2), s)
+        assert np.array_equal(u32(dist[i]), d) and np.array_equal(u32(pred[i]), p)
+
+
+def test_two_streams_and_few_blocks(sssp):
+    """Sweeps on two streams at a time, one of them with one block per SM."""
+    rng = np.random.default_rng(2)
+    V, S = 50000, 6
+    src, dst, w = graph(rng, V, 8 * V)
+    ref = oracle.csr(V, src, dst, w)
+    g = sssp.build_csr(V, src, dst, w)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    solvers = [sssp.Solver(g, S), sssp.Solver(g, S, sssp.options(blocks_per_sm=1))]
+    sources = [torch.from_numpy(rng.integers(0, V, S).astype(np.int32)).cuda() for _ in range(2)]
+    torch.cuda.synchronize()
+    for _ in range(10):
+        for k in range(2):
+            solvers[k].launch(sources[k], stream=streams[k])
+    for k in range(2):
+        assert solvers[k].status(streams[k])[0] == 0
+        for i, s in enumerate(sources[k].tolist()):
+            d, p, _ = oracle.dijkstra(ref, s)
+            assert np.array_equal(u32(solvers[k].dist[i]), d) and np.array_equal(u32(solvers[k].pred[i]), p)
