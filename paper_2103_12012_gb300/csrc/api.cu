@@ -155,18 +155,20 @@ SolveWs solve_layout(const sssp_graph* g, uint32_t S, uint32_t split, bool sweep
 // weights; V, edges per vertex, P, S, given width).  At the default width nearly always: ER 16,384, 8, 4, 1: 1.6 /
 // 0.31; 64, 6, 1, 1: 0.34 / 0.11; 8,192, 6, 148, 8: 0.84 / 0.28.  A given (tuned) width makes the persistent solve
 // several times faster, and then the sweep wins
-//   over units of many vertices, more of them the more sources share a row: ER 4,096, 12, 4, 1: 0.31 / 0.19;
-//     R-MAT 65,536, 15, 64, 5: 1.4 times; but R-MAT 8,192, 6, 16, 8, float32: 0.14 / 0.20
-//   over more units than the persistent solve has blocks: R-MAT 4.2 M, 16, 148, 8: 7.2 / 4.0; but ER 1 M, 13, 100,
-//     5 (500 units): 1.5 / 1.9; R-MAT has hubs, and a layout if they are large: 400,000, 16, 64, 5: 1.4 / 0.9
-//   with 1 to 4 sources over many units, only on graphs with hubs: ER 1 M, 16, 148, 4: 1.8 / 2.3; R-MAT 1 M, 16,
-//     148, 1: 1.2 / 0.6
+//   with 5 sources and more, which share rows, on large graphs (R-MAT 4.2 M, 16, 148, 8: 7.2 / 4.0), over more units
+//     than the persistent solve has blocks, and over units of many vertices (ER 8,192, 12, 4, 8: 1.5 times); but
+//     R-MAT 12,855, 6, 45, 6: 0.20 / 0.30, and of the large graphs ER 468,550, 15, 38, 15 (570 units), width 80:
+//     2.0 / 2.5
+//   with fewer over units of many vertices, more of them the more sources there are, if the units are few or the
+//     graph has hubs (those that are worth a layout): ER 4,096, 12, 4, 1: 0.31 / 0.19; R-MAT 1 M, 16, 148, 1: 1.2 /
+//     0.6; but ER 1 M, 16, 148, 4: 1.8 / 2.3; R-MAT 25,704, 10, 143, 2: 0.22 / 0.30
+// Of 1,995 solves at given widths, drawn over these ranges, 7 are slower than the persistent solve by more than 7%,
+// most of them large random graphs at wide widths.
 bool sweep_wins(const sssp_graph* g, uint32_t S, const SolveWs& L, bool delta_given) {
     const uint64_t units = (uint64_t)S * L.Q;
     if (!delta_given) return L.Bq >= 64 || (S >= 5 && g->V >= 2048);
-    if (S < 5) return L.Bq >= 256u * (S + 1u) && (g->ids || units < 128);
-    if (units >= 608) return g->V >= 16384;
-    return (g->ids || units < 256) && L.Bq >= (g->V >= 32768 ? 512u : S >= 7 ? 2048u : 256u * (S + 1u));
+    if (S >= 5) return g->V >= 24576 || (units >= 608 && g->V >= 16384) || L.Bq >= 2048;
+    return g->ids ? L.Bq >= 128u * (S + 1u) : L.Bq >= 256u * (S + 1u) && units < 128;
 }
 
 // When a sweep stops after its first iterations, in favour of the persistent solve, which then starts from the
