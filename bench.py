@@ -94,8 +94,8 @@ def code_sha256(path):
 
 
 def dram_traffic(edges_scanned):
-    """DRAM bytes per launch of the relaxation kernel from the committed ncu capture, scaled to this
-    launch by edges scanned; None if the kernel code changed since that capture."""
+    """DRAM bytes of a solve's relaxation kernels (k_sweep and k_sweep_out) from the committed ncu capture, scaled
+    to this launch by edges scanned; None if the kernel code changed since that capture."""
     try:
         rec = json.loads(open(os.path.join(ROOT, "profiles", "k_solve_dram_traffic.txt")).read())
         sha = code_sha256(os.path.join(ROOT, rec["source"]))
@@ -107,8 +107,9 @@ def dram_traffic(edges_scanned):
 
 
 def batched_traffic(edges_scanned):
-    """DRAM bytes of one k_batched launch from the committed one-pass capture of the full batch,
-    scaled by edges scanned; None if there is no capture or the kernel code changed since."""
+    """DRAM bytes of one solve of the full batch (k_batched, and k_batch on the graphs that fit in shared memory) from
+    its committed one-pass capture, scaled by edges scanned; None if there is no capture or the kernel code
+    changed since."""
     try:
         rec = json.loads(open(os.path.join(ROOT, "profiles", "k_batched_dram_traffic.txt")).read())
         if code_sha256(os.path.join(ROOT, rec["source"])) != rec["code_sha256"]:
@@ -716,7 +717,7 @@ def extras_batched(sssp, dev, rank=0, world=1):
             "graph_replay_ms": round(ms_plan, 3), "solves_per_s": round(n_prob / ms_plan * 1e3, 1),
             "reached_edges": E_r, "reached_vertices": V_r, "edges_scanned": stats["edges_scanned"],
             "work_inflation": round(stats["edges_scanned"] / max(E_r, 1), 3),
-            "roofline": {"bound": "hbm", "kernel": "k_batched", "achieved": round(achieved, 1), "peak": peak,
+            "roofline": {"bound": "hbm", "kernel": "k_batched + k_batch", "achieved": round(achieved, 1), "peak": peak,
                          "peak_kind": peak_kind, "unit": "GB/s", "frac": round(achieved / peak, 4),
                          "alg_bytes_per_launch": alg, "traffic": batched_traffic(stats["edges_scanned"])},
             "per_graph_launches_ms": round(ms_graph, 3), "per_problem_launches_ms": round(ms_prob, 3),

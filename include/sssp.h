@@ -117,8 +117,11 @@ typedef struct {
                               within delta / 2 (0 = no hubs; ignored on other graphs).  Processing a
                               high-degree vertex twice costs its whole row, so these wait for a
                               narrower bucket while the other vertices may take a wider one. */
-    void* ev_relax_begin;  /* cudaEvent_t or NULL: recorded on `stream` right before the relaxation kernel */
-    void* ev_relax_end;    /* cudaEvent_t or NULL: recorded right after it (for timing that kernel alone) */
+    void* ev_relax_begin;  /* cudaEvent_t or NULL: recorded on `stream` right before the relaxation kernel,
+                              on a swept solve before the sweep */
+    void* ev_relax_end;    /* cudaEvent_t or NULL: recorded right after it (for timing that kernel alone), on a
+                              swept solve after the sweep and the launches that follow it (its predecessors and
+                              a persistent kernel, which ends at once unless the sweep has left it work) */
 } sssp_options;
 
 /* Frontier policies of sssp_solve: how a round picks, among its unit's queued
@@ -268,8 +271,10 @@ size_t sssp_solve_workspace_size(const sssp_graph* g, uint32_t S, const sssp_opt
  * policy and without held messages, where that is the faster way: all sources
  * relax it together, in Bellman-Ford order (sweep.cu; tile, split, delta,
  * threads and hub_count do not apply to it, and its rounds are iterations
- * without messages between units).  What a sweep leaves (a graph of high
- * diameter), and every other call, goes to the persistent solve.
+ * without messages between units).  What a sweep leaves goes to the persistent
+ * solve, in the same call: a graph that after a few iterations looks to be of
+ * many hops starts from its sources again there, a long tail goes on.
+ * Every other call runs the persistent solve alone.
  * Launches an init kernel, one persistent cooperative relaxation kernel in
  * which each block owns (source, partition sub-block) units, and an unpack
  * kernel.  dist is also scratch until the end.  Needs every block co-resident; returns SSSP_EUNSUPPORTED if the
@@ -481,6 +486,8 @@ size_t sssp_backward_workspace_size(uint32_t V, uint32_t E, uint32_t S);
  * (an unreachable vertex, pred == 0xFFFFFFFF and not a source, starts no walk).
  *   grad_w    : device [E] float32 out, CSR edge order, summed over the S sources;
  *               non-tree edges get 0
+ *   ws        : device workspace >= sssp_backward_workspace_size(V, E, S): about 21 bytes per
+ *               vertex and source (a transposed copy of pred among them) and 8 per edge
  */
 sssp_status sssp_backward(const sssp_graph* g, uint32_t S, const uint32_t* pred, const float* grad_dist,
                           float* grad_w, void* ws, size_t ws_bytes, sssp_stream_t stream);

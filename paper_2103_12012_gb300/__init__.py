@@ -505,7 +505,8 @@ class Batch:
                  stream=None):
         """Choose the batched kernel's bucket width, tile and block size by timing sssp_solve_batched on
         this batch (coordinate search: delta; then tile and block size together; then delta again at
-        3/4, 5/4 and 3/2 of the best).  Sets self.opts and returns (options, ms)."""
+        3/4, 5/4 and 3/2 of the best).  Problems that are solved in shared memory use neither tile nor
+        block size, and three times delta.  Sets self.opts and returns (options, ms)."""
         torch = _torch()
 
         def run(o):

@@ -6,7 +6,8 @@
 //
 // Buckets of distances in turn: items below the bound are marked near, the others far.  A round takes
 // the near marks, 512 items at a time, and its warps relax their rows; a warp holds 32 rows and
-// walks their edges together, rows of HUB edges and more are cut into segments that all warps share.
+// walks their edges together, rows of HUB edges and more are cut into segments that all warps share (api.cu's
+// in_smem says which graphs are not for it: very dense ones, and wide grids at a given width).
 // When no near mark is left, the bound moves to the end of the bucket of the least far distance, and the
 // round takes the far marks below it.  A mark is cleared before its distance is read, and set after
 // the distance is lowered, so no fall is lost.  Predecessors come from one walk over the edges at the end:
@@ -14,9 +15,9 @@
 // converge too.
 //
 // Bound by instructions (half of the issue slots at 32 warps an SM) and by the rounds' barriers.  Against the
-// general kernel, ms (vertices, graphs x sources; uint32 / float32): 1,024-2,048, 512 x 16: 6.17 -> 1.96 / 6.25 -> 1.06;
-// 1,024-4,096, 32 x 16: 0.59 -> 0.32 / 0.58 -> 0.25; 1,024-16,384, 200 x 5: 1.30 -> 0.99 / 1.23 -> 0.61; 1,024-46,000,
-// 512 x 16: 14.5 -> 9.4 / 13.6 -> 6.6.  Two or four steps of a warp in flight: 1 to 8% slower.  Distances of
+// general kernel, ms (vertices, graphs x sources; uint32 / float32): 1,024-2,048, 512 x 16: 6.17 -> 1.87 / 6.26 -> 1.08;
+// 1,024-4,096, 32 x 16: 0.59 -> 0.24 / 0.58 -> 0.17; 1,024-16,384, 200 x 5: 1.28 -> 0.80 / 1.22 -> 0.52; 1,024-46,000,
+// 512 x 16: 14.6 -> 9.0 / 13.6 -> 6.3.  Two or four steps of a warp in flight: 1 to 8% slower.  Distances of
 // larger graphs in the shared memory of a cluster (2 or 4 blocks, 47,104 to 131,072 vertices) took 27 against 23
 // ms, in L2 with the marks in shared memory 40: there the general kernel's 64 warps an SM hide more.
 // 512 threads a block while units are small (several blocks an SM: 1,024-2,048, 512 x 2: 0.53 against 0.84 ms with

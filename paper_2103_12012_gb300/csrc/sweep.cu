@@ -13,8 +13,8 @@
 // and marks the items whose distances fall, which are the next iteration's; about 20 iterations in
 // all.  There is no bucket order: thresholds above the least queued distance of each source cut the
 // relaxations of random graphs to a third, but took more iterations and a second look at every item,
-// and on power-law graphs cut nothing (R-MAT scale 22, 8 sources: 4.7 against 4.2 ms; random graph of
-// 16,384 vertices: 0.36 against 0.24 ms).
+// and on power-law graphs cut nothing (in an earlier form of this kernel, R-MAT scale 22, 8 sources: 4.7 against 4.2
+// ms; random graph of 16,384 vertices: 0.36 against 0.24 ms).
 //   list A : rows of up to 31 edges; a warp takes 32 of them (fewer when the list is short) and
 //            walks their edges together
 //   list M : rows of 32 to 511 edges, up to 8 a warp in the same way
@@ -24,12 +24,14 @@
 // Predecessors come from one pass over the edges at the end (k_sweep_out): pred(v) is the least
 // label of a tail u with dist(u) + w = dist(v), to which the packed words of the persistent solve
 // converge too.  The loop then needs 4 bytes per vertex and source instead of 8.
-// Measured against the persistent solve, tuned (whole calls): R-MAT scale 22, edge factor 16, 8
-// sources 4.1 against 7.4 ms, DRAM traffic 7.7 against 13.1 GB; R-MAT scale 18, 32 float32 sources
-// 0.66 against 1.0 ms; random graph, 16,384 vertices, 4 partitions, 1 source 0.24 against 1.6 ms.
-// k_sweep (3.0 ms of the 4.1) is bound by the latency of its L2 accesses and by issue slots (44% busy
-// at the 32 warps per SM that 64 registers allow; with 48 warps at 40 registers it spills and is not
-// faster), k_sweep_out (0.81 ms) by random 32-byte sectors, 80 G a second.
+// Measured against the persistent solve (launches; a call has about 0.1 ms besides): R-MAT scale 22, edge factor
+// 16, 8 sources, locality layout 3.3 against 7.1 ms (tuned; whole calls on another graph and sources of this
+// recipe 4.1 against 7.4); DRAM traffic 6.2 against 13.1 GB; R-MAT scale 18, 32 float32 sources 0.58 against 1.0 ms
+// (tuned); random graph, 16,384 vertices, 4 partitions, 1 source 0.23 against 1.6 ms (default width).
+// k_sweep (2.4 ms of the 3.3) is bound by the latency of its L2 accesses, issue slots and barriers (scale 20, ncu: 47%
+// of the slots busy at the 32 warps per SM that 64 registers allow, stalls 5.8 cycles an instruction on loads and 4.4
+// at barriers; with 48 warps at 40 registers it spills and is not faster), k_sweep_out (0.81 ms) by random 32-byte
+// sectors, 80 G a second.
 // A warm start (sssp_update) with many tails goes the same way, from the tails' rows: there the rows are of
 // packed words (up to four), so that predecessors come along and no pass over all edges is needed, and
 // the lists and marks take the caller's dist.  R-MAT, 1 M vertices, 15 M edges, 4 sources, 15,000 tails: 0.39 ->
